@@ -2,21 +2,27 @@
 // data surface in a uniformly moving medium (Appendix B, Eqs. B.2-B.14),
 // advanced-time (source-time-dominant) form, in double precision.
 //
+//   k_fwh_delays : the smallest and largest delay R/c0 of each observer, from
+//                  which the host takes its unified window (Eq. B.13).
 //   k_fwh_series : per panel and source time, the thickness and loading
 //                  sources Q (Eq. A.5) and L_i (Eqs. A.7-A.8, sigma_ij
 //                  omitted), with u_i the disturbance velocity V - U_inf,
 //                  and their 4th-order finite-difference tau-derivatives.
+//   k_fwh_fix    : the series in 60-bit fixed point, one exponent per series.
 //   k_fwh_accum  : per (panel, spanwise copy) the radii R*, R and their
 //                  gradients (Eqs. B.8-B.12) give the integrand coefficients
 //                  of Eqs. B.2-B.3; each observer time t* (unified window,
 //                  step dtau) interpolates the panel integrand at
 //                  tau = t* - R/c0 (Eq. B.13) with a 4-point cubic Lagrange
-//                  stencil and sums (Eq. B.14); one partial row per panel group.
+//                  stencil and sums (Eq. B.14), on the integer pipe; one
+//                  partial row per panel group.
 //   k_fwh_reduce : sums the partial rows in a fixed order, divides by 4 pi.
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
+#include <cstring>
 #include <string>
 #include <vector>
 
@@ -25,6 +31,7 @@
 namespace {
 
 constexpr int NSER = 8;  // Q, L1, L2, L3, dQ, dL1, dL2, dL3
+constexpr int kFwhGroup = 32;   // panel copies per row of partial sums that the fixed scratch is counted by
 
 struct FwhConst {
     double M[3];
@@ -32,58 +39,144 @@ struct FwhConst {
     double b2;  // Prandtl-Glauert factor squared, 1 / (1 - |M|^2)
 };
 
-__device__ __forceinline__ void sources(const double* h, const double* n, const FwhConst& k, double* out) {
-    // h = (rho, V1, V2, V3, p) total; disturbance u = V - c0 M
-    double u[3];
-    double un = 0.0, Un = 0.0;
-    for (int i = 0; i < 3; ++i) {
-        u[i] = h[1 + i] - k.c0 * k.M[i];
-        un += u[i] * n[i];
-        Un += k.c0 * k.M[i] * n[i];
-    }
-    const double rho = h[0];
-    out[0] = rho * (un + Un) - k.rho0 * Un;
-    for (int i = 0; i < 3; ++i) out[1 + i] = (h[4] - k.p0) * n[i] + rho * u[i] * (un + Un);
+// The sources of one panel sample h = (rho, V1, V2, V3, p): n its normal, U = c0 M
+// the mean flow and Un = U.n; the disturbance u = V - U has u.n + U.n = V.n
+__device__ __forceinline__ void sources(const double* h, const double* n, const double* U, double Un,
+                                        const FwhConst& k, double* out) {
+    const double rv = h[0] * (h[1] * n[0] + h[2] * n[1] + h[3] * n[2]);
+    out[0] = rv - k.rho0 * Un;
+    const double dp = h[4] - k.p0;
+    for (int i = 0; i < 3; ++i) out[1 + i] = dp * n[i] + rv * (h[1 + i] - U[i]);
 }
 
-__global__ void k_fwh_series(const double* __restrict__ hist, int nt, int npts, const double* __restrict__ nrm,
-                             FwhConst k, double* __restrict__ X) {
-    const int64_t w = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (w >= int64_t(nt) * npts) return;
-    const int p = int(w % npts);
-    const int t = int(w / npts);
-    const double n[3] = {nrm[p * 3 + 0], nrm[p * 3 + 1], nrm[p * 3 + 2]};
-    // the 5-point stencil: central inside, one-sided 4th order at both ends
-    int j0;
-    double c[5];
+// The source series of a batch of panels: layout of one panel [nt places][4 pairs]
+// [2 series], pair 0 = (Q, L1), 1 = (L2, L3), 2 = (dQ, dL1), 3 = (dL2, dL3); pair v
+// of place a sits at v ^ ((a >> 1) & 3), so that 8 lanes reading the same pair of
+// neighbouring places touch every bank group once.  Places along time are ordered by t mod KO, then t / KO, so that
+// lanes of k_fwh_accum, which are KO samples apart, read neighbouring 16-byte
+// places whatever the delay.
+constexpr int KO = 4;   // consecutive samples of a lane of k_fwh_accum
+__host__ __device__ __forceinline__ int fwh_place(int t, int nt) {
+    const int r = t & (KO - 1);
+    return r * (nt / KO) + min(r, nt & (KO - 1)) + (t - r) / KO;   // t - r is a multiple of KO, also for t < 0
+}
+// 16-byte slot of pair v of place a within a panel
+__host__ __device__ __forceinline__ unsigned fwh_slot(unsigned a, unsigned v) { return 4 * a + (v ^ ((a >> 1) & 3)); }
+
+// k_fwh_series: a block takes 8 panels x 256 source times.  It evaluates the
+// four sources once per panel and time (4 more on each side for the stencil)
+// into shared memory, then warp w writes panel w's eight series, 32 neighbouring
+// places per store, and keeps each series' largest magnitude (high word of the
+// double, a total order on magnitudes) for the fixed-point form.  Bound by the FP64
+// pipe (31 operations a panel and time).  At 18,840 panels x 1000 times 1.45 ms;
+// one thread per (panel, time) with six source evaluations each and stores 64 kB
+// apart took 4.93 ms.
+constexpr int SER_P = 8, SER_T = 256, SER_H = 4, SER_W = SER_T + 2 * SER_H;
+constexpr size_t SER_SMEM = sizeof(double) * 4 * SER_P * SER_W;
+
+__global__ void __launch_bounds__(256) k_fwh_series(const double* __restrict__ hist, int nt, int npts, int p0, int np,
+                                                    const double* __restrict__ nrm, FwhConst k,
+                                                    double* __restrict__ X, int* __restrict__ hw) {
+    extern __shared__ double sq[];   // [4][SER_P][SER_W]
+    const int pb = blockIdx.x * SER_P, tb = blockIdx.y * SER_T;
+    {
+        const int lp = threadIdx.x % SER_P;
+        const int p = p0 + min(pb + lp, np - 1);
+        const double n[3] = {nrm[p * 3 + 0], nrm[p * 3 + 1], nrm[p * 3 + 2]};
+        const double U[3] = {k.c0 * k.M[0], k.c0 * k.M[1], k.c0 * k.M[2]};
+        const double Un = U[0] * n[0] + U[1] * n[1] + U[2] * n[2];
+        for (int i = threadIdx.x / SER_P; i < SER_W; i += 256 / SER_P) {
+            const int t = min(max(tb - SER_H + i, 0), nt - 1);
+            double q[4];
+            sources(hist + (int64_t(t) * npts + p) * 5, n, U, Un, k, q);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) sq[(v * SER_P + lp) * SER_W + i] = q[v];
+        }
+    }
+    __syncthreads();
+    const int lp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (pb + lp >= np) return;
+    double2* xp = reinterpret_cast<double2*>(X) + int64_t(pb + lp) * 4 * nt;
     const double s = 1.0 / (12.0 * k.dtau);
-    if (t >= 2 && t <= nt - 3) {
-        j0 = t - 2;
-        c[0] = 1; c[1] = -8; c[2] = 0; c[3] = 8; c[4] = -1;
-    } else if (t == 0) {
-        j0 = 0;
-        c[0] = -25; c[1] = 48; c[2] = -36; c[3] = 16; c[4] = -3;
-    } else if (t == 1) {
-        j0 = 0;
-        c[0] = -3; c[1] = -10; c[2] = 18; c[3] = -6; c[4] = 1;
-    } else if (t == nt - 1) {
-        j0 = nt - 5;
-        c[0] = 3; c[1] = -16; c[2] = 36; c[3] = -48; c[4] = 25;
-    } else {
-        j0 = nt - 5;
-        c[0] = -1; c[1] = 6; c[2] = -18; c[3] = 10; c[4] = 3;
+    int top[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    for (int r = 0; r < SER_T / 32; ++r) {
+        const int t = tb + 32 * KO * (r / KO) + KO * lane + r % KO;
+        if (t >= nt) continue;
+        double x[8];
+        if (t >= 2 && t <= nt - 3) {
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const double* q = sq + (v * SER_P + lp) * SER_W + (t - tb + SER_H);
+                x[v] = q[0];
+                x[4 + v] = ((q[-2] - q[2]) + 8.0 * (q[1] - q[-1])) * s;
+            }
+        } else {
+            // one-sided 4th-order stencils at both ends
+            const double c[4][5] = {{-25, 48, -36, 16, -3}, {-3, -10, 18, -6, 1}, {-1, 6, -18, 10, 3},
+                                    {3, -16, 36, -48, 25}};
+            const int j0 = t < 2 ? 0 : nt - 5, w = t < 2 ? t : t - nt + 4;
+            for (int v = 0; v < 4; ++v) {
+                const double* q = sq + (v * SER_P + lp) * SER_W + (SER_H - tb);
+                double der = 0.0;
+                for (int m = 0; m < 5; ++m) der += c[w][m] * q[j0 + m];
+                x[v] = q[t];
+                x[4 + v] = der * s;
+            }
+        }
+        const int at = fwh_place(t, nt);
+#pragma unroll
+        for (int w = 0; w < 4; ++w) xp[fwh_slot(at, w)] = make_double2(x[2 * w], x[2 * w + 1]);
+#pragma unroll
+        for (int v = 0; v < 8; ++v) top[v] = max(top[v], __double2hiint(x[v]) & 0x7fffffff);
     }
-    double here[4], der[4] = {0, 0, 0, 0};
-    sources(hist + (int64_t(t) * npts + p) * 5, n, k, here);
-    for (int m = 0; m < 5; ++m) {
-        double q[4];
-        sources(hist + (int64_t(j0 + m) * npts + p) * 5, n, k, q);
-        for (int v = 0; v < 4; ++v) der[v] += c[m] * q[v];
+#pragma unroll
+    for (int v = 0; v < 8; ++v) {
+        const int m = __reduce_max_sync(0xffffffffu, top[v]);
+        if (lane == 0) atomicMax(hw + (pb + lp) * 8 + v, m);
     }
-    double* xp = X + int64_t(p) * NSER * nt;
-    for (int v = 0; v < 4; ++v) {
-        xp[v * nt + t] = here[v];
-        xp[(4 + v) * nt + t] = der[v] * s;
+}
+
+// Fixed-point form of a number: N = x 2^(60 - e) for |x| < 2^e, as two limbs
+// N = h 2^30 + l with -2^29 <= l < 2^29.  e follows from the largest high word H
+// of the series.  A series of zeros has H = 0; a panel with an infinity, a NaN or
+// values below 2^-959 keeps its doubles and is summed in double (fwh_wide).
+__device__ __forceinline__ bool fwh_wide(int H) { return H >= 0x7ff00000 || (H > 0 && H < (64 << 20)); }
+__device__ __forceinline__ bool fwh_wide_panel(const int* hw) {
+    bool w = false;
+    for (int v = 0; v < 8; ++v) w = w || fwh_wide(hw[v]);
+    return w;
+}
+// mantissa of |x| as an integer < 2^53 (x normal or 0), shifted left by s and
+// right by d with rounding
+__device__ __forceinline__ long long fwh_fix(double x, int s, int d) {
+    const unsigned long long u = static_cast<unsigned long long>(__double_as_longlong(x));
+    const int ex = int(u >> 52) & 0x7ff;
+    if (ex == 0 || d > 62) return 0;
+    long long m = static_cast<long long>((u & 0xfffffffffffffull) | 0x10000000000000ull) << s;
+    if (d > 0) m = (m + (1ll << (d - 1))) >> d;
+    return (u >> 63) ? -m : m;
+}
+__device__ __forceinline__ int2 fwh_limbs(long long N) {
+    const int h = int((N + (1ll << 29)) >> 30);
+    return make_int2(h, int(N - (static_cast<long long>(h) << 30)));
+}
+
+// the series of a batch to fixed point, in place (16 bytes, two series, a thread)
+__global__ void k_fwh_fix(double* __restrict__ X, const int* __restrict__ hw, int nt, int np) {
+    const int64_t n = int64_t(np) * 4 * nt;
+    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
+        const int64_t p = i / (4 * int64_t(nt));
+        const unsigned at = unsigned(i - p * 4 * nt);
+        const int* H = hw + p * 8;
+        if (fwh_wide_panel(H)) continue;
+        const int v = 2 * ((at ^ (at >> 3)) & 3);   // the series of this slot (fwh_slot)
+        const double2 x = reinterpret_cast<const double2*>(X)[i];
+        auto conv = [](double x, int H) {
+            const int ex = (__double2hiint(x) >> 20) & 0x7ff;
+            return fwh_limbs(fwh_fix(x, 7, (H >> 20) - ex));
+        };
+        const int2 a = conv(x.x, H[v]), b = conv(x.y, H[v + 1]);
+        reinterpret_cast<int4*>(X)[i] = make_int4(a.x, a.y, b.x, b.y);
     }
 }
 
@@ -120,116 +213,356 @@ __device__ void panel_coefs(const double* y, double dS, const double* obs, const
     *delay = R / k.c0;
 }
 
-// Each thread accumulates FWH_KO consecutive observer-time samples over the
-// panel-copies of its block's group.  A panel-copy's stencil offset and cubic
-// weights are the same for every sample (t = tstart + i dtau advances the
-// source index by exactly 1 per sample), so they are computed once per block;
-// each source time j in the thread's window combines the 8 series once
-// (I_j = sum_v cf_v X_v(j)) and serves up to four samples.  Samples whose
-// stencil is clamped at the ends of the record take the general per-sample
-// path.  Small groups give many blocks per observer (the FP64 pipe needs the
-// parallelism).
-constexpr int FWH_KO = 4;
-constexpr int kFwhGroup = 32;      // panel-copies per block (groups of whole panels)
-constexpr int FWH_SH = NSER + 5;   // per panel-copy: cf[8], weights[4], source index of sample 0
-// dynamic shared memory per panel-copy: the doubles above, the offset of the
-// panel's series and the stencil start of sample 0 (integers, so that the
-// sample loop does no FP64 conversions)
-constexpr size_t FWH_SH_BYTES = sizeof(double) * FWH_SH + sizeof(int64_t) + sizeof(int);
+// One observer of a launch: position, first time and length of its window.
+struct FwhObs {
+    double x[3], tstart;
+    int T, pad;
+};
 
-__global__ void k_fwh_accum(const double* __restrict__ X, int nt, int npts, const double* __restrict__ y,
-                            const double* __restrict__ dS, FwhConst k, double ox, double oy, double oz,
-                            double tstart, int T, int ncopies, double Lspan, int group,
-                            double* __restrict__ partial) {
-    extern __shared__ double sh[];  // [cap][FWH_SH] doubles, then int64 [cap], then int [cap]
-    const int p0 = blockIdx.x * group;     // grid x: panel groups, grid y: sample blocks
-    const int np = min(group, npts - p0);
-    const int npc = np * ncopies;
-    const int cap = group * ncopies;
-    int64_t* xoff = reinterpret_cast<int64_t*>(sh + size_t(cap) * FWH_SH);
-    int* jbs = reinterpret_cast<int*>(xoff + cap);
-    const int K = (ncopies - 1) / 2;
-    const double obs[3] = {ox, oy, oz};
-    for (int w = threadIdx.x; w < npc; w += blockDim.x) {
-        const int p = p0 + w / ncopies;
-        const int cc = w % ncopies - K;
-        const double yy[3] = {y[p * 3 + 0], y[p * 3 + 1], y[p * 3 + 2] + cc * Lspan};
-        double delay;
-        double* cf = sh + w * FWH_SH;
-        panel_coefs(yy, dS[p], obs, k, cf, &delay);
-        const double off = (tstart - k.tau0 - delay) / k.dtau;   // source index of sample 0
-        const double fl = floor(off);
-        const double x = off - fl + 1.0;                        // position in the stencil, [1, 2)
-        cf[NSER + 0] = -(x - 1.0) * (x - 2.0) * (x - 3.0) / 6.0;
-        cf[NSER + 1] = x * (x - 2.0) * (x - 3.0) / 2.0;
-        cf[NSER + 2] = -x * (x - 1.0) * (x - 3.0) / 2.0;
-        cf[NSER + 3] = x * (x - 1.0) * (x - 2.0) / 6.0;
-        cf[NSER + 4] = off;
-        jbs[w] = int(fl) - 1;
-        xoff[w] = int64_t(p) * NSER * nt;
+// the delay R / c0 of a panel copy at y (Eqs. B.8, B.9)
+__device__ __forceinline__ double panel_delay(const double* y, const double* obs, const FwhConst& k) {
+    double Mr = 0, rr = 0;
+    for (int i = 0; i < 3; ++i) {
+        const double r = obs[i] - y[i];
+        Mr += k.M[i] * r;
+        rr += r * r;
     }
-    __syncthreads();
-    const int i0 = (blockIdx.y * blockDim.x + threadIdx.x) * FWH_KO;
-    if (i0 >= T) return;
-    double acc[FWH_KO];
+    const double Rs = sqrt(rr + k.b2 * Mr * Mr) / sqrt(k.b2);
+    return k.b2 * (Rs - Mr) / k.c0;
+}
+
+// ext[2 o], ext[2 o + 1]: largest delay of observer o and the complement of the
+// smallest, as bits of non-negative doubles (0 at the start).  One thread a panel
+// copy; the host loop this takes the place of took 8 ms for 2.0 million of them.
+__global__ void k_fwh_delays(const double* __restrict__ y, int npts, FwhConst k, const FwhObs* __restrict__ obs,
+                             int ncopies, double Lspan, unsigned long long* __restrict__ ext) {
+    const int o = blockIdx.y, K = (ncopies - 1) / 2;
+    const double ob[3] = {obs[o].x[0], obs[o].x[1], obs[o].x[2]};
+    unsigned long long hi = 0, lo = 0;
+    for (int64_t w = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; w < int64_t(npts) * ncopies;
+         w += int64_t(gridDim.x) * blockDim.x) {
+        const int64_t p = w / ncopies;
+        const double yy[3] = {y[p * 3 + 0], y[p * 3 + 1], y[p * 3 + 2] + (int(w - p * ncopies) - K) * Lspan};
+        const double d = panel_delay(yy, ob, k);
+        if (!(d >= 0.0)) continue;   // NaN: left out, as by a comparison
+        const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(d + 0.0));
+        hi = max(hi, b);
+        lo = max(lo, ~b);
+    }
+    for (int s = 16; s > 0; s >>= 1) {
+        hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, s));
+        lo = max(lo, __shfl_xor_sync(0xffffffffu, lo, s));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(ext + 2 * o, hi);
+        atomicMax(ext + 2 * o + 1, lo);
+    }
+}
+
+__device__ __forceinline__ void cubic_weights(double x, double (&wt)[4]) {
+    wt[0] = -(x - 1.0) * (x - 2.0) * (x - 3.0) / 6.0;
+    wt[1] = x * (x - 2.0) * (x - 3.0) / 2.0;
+    wt[2] = -x * (x - 1.0) * (x - 3.0) / 2.0;
+    wt[3] = x * (x - 1.0) * (x - 2.0) / 6.0;
+}
+// FP64 form of one sample at source index s (stencil clamped to the record), for
+// panel copies that are not in fixed point
+__device__ double fwh_sample_fp64(const int4* xp, const int* hw, bool wide, int nt, const double* cf, double s) {
+    const int j = max(0, min(nt - 4, int(floor(s)) - 1));
+    double wt[4];
+    cubic_weights(s - double(j), wt);
+    double sum = 0.0;
+    for (int m = 0; m < 4; ++m) {
+        double Ik = 0.0;
+        for (int v = 0; v < NSER; ++v) {
+            const int2 q = reinterpret_cast<const int2*>(xp + fwh_slot(fwh_place(j + m, nt), v >> 1))[v & 1];
+            double val;
+            if (wide) val = __hiloint2double(q.y, q.x);
+            else val = hw[v] ? scalbn(double((static_cast<long long>(q.x) << 30) + q.y), (hw[v] >> 20) - 1082) : 0.0;
+            Ik += cf[v] * val;
+        }
+        sum += wt[m] * Ik;
+    }
+    return sum;
+}
+
+// Coefficients and source index of sample 0 of panel copy (p, cc)
+__device__ void fwh_panel(const double* y, const double* dS, int p, int cc, double Lspan, const FwhObs& ob,
+                          const FwhConst& k, double* cf, double* off) {
+    const double yy[3] = {y[p * 3 + 0], y[p * 3 + 1], y[p * 3 + 2] + cc * Lspan};
+    double delay;
+    panel_coefs(yy, dS[p], ob.x, k, cf, &delay);
+    *off = (ob.tstart - k.tau0 - delay) / k.dtau;
+}
+__device__ __noinline__ double fwh_wide_sample(const int4* xp, const int* hw, bool wide, int nt, const double* y,
+                                        const double* dS, int p, int cc, double Lspan, const FwhObs* ob,
+                                        const FwhConst& k, int i) {
+    double cf[NSER], off;
+    fwh_panel(y, dS, p, cc, Lspan, *ob, k, cf, &off);
+    return fwh_sample_fp64(xp, hw, wide, nt, cf, double(i) + off);
+}
+
+// Sum over panel copies of the interpolated integrand (Eqs. B.2, B.13, B.14), in
+// fixed point on the integer pipe: this GPU multiplies 32-bit integers 32 times
+// as fast as it does FP64, and 18 FP64 operations a panel copy and sample bound
+// the sum in double (18,840 panels, 36 observers, 3 copies, 690 samples: 72 ms in
+// double at 0.6 of the FP64 rate, 13 ms here).
+//   I = sum_v cf_v X_v(j) with X_v = x_v 2^e_v and cf_v 2^e_v = c_v 2^E, E the
+//   panel copy's own exponent, |I| < 2^E: x, c and I have 60 bits below their
+//   exponents, products of limbs h h' + ((h l' + l h') >> 30) drop only l l',
+//   2^-58 of the bound; then p += sum_m w_m I(j + m) with the cubic weights
+//   scaled by 2^(E - Emax - b) (Emax over the block's copies, 2^b twice their
+//   number), kept as the two sums hh and mid of 64 bits, with which a sum over a
+//   block is exact; it becomes a double once, at the block's end.
+// Each quantity thus carries at least as many bits as a double of the size of its
+// bound (weights of copies that count for less than the block's largest lose bits
+// in proportion).  Error against a reference in another order of summation, 2-norm:
+// 1.3e-13 to 1.5e-12 here, 1.5e-13 to 1.8e-12 in double (it comes from the sources).
+// A block: one group of panels and one observer; a warp takes 124 samples of it, a
+// lane 4 consecutive ones (31 lanes; lane 31 only supplies the integrands that
+// lane 30's stencils need).  Each integrand is formed once and passed to the lane
+// before it by shuffles: 24 + 12 products of limb pairs, 4 loads of 16 bytes and
+// 1.5 shuffles a sample.  Bound by the multiplier (IMAD.WIDE, about 70% busy).  With
+// 8 samples a lane and 128 registers 1.80 ms against 1.51 ms at 2,198 panels.
+constexpr int ACC_PC = 96;        // panel copies set up at a time
+constexpr int ACC_LANES = 31;     // lanes with samples of their own
+constexpr int ACC_WARPS = 8;      // warps (sample chunks) of a block at most
+constexpr int ACC_S = KO * ACC_LANES;
+
+struct FwhPc {
+    int c[2 * NSER];   // coefficient limbs (h, l)
+    int w[8];          // weight limbs
+    int at[KO];        // place of t = jb + m, m < KO
+    double off;        // source index of sample 0
+    int E, sc;         // exponent E; weights are scaled by 2^sc
+    int jb, p, cc, kind;   // kind 1: fixed point, 0: double, 2: no contribution
+};
+
+// one integrand, N = I 2^60 / 2^E, of a panel's series at place `at`
+__device__ __forceinline__ long long fwh_integrand(const int (&c)[2 * NSER], const int4* xp, unsigned at) {
+    long long a = 0, b = 0;
 #pragma unroll
-    for (int q = 0; q < FWH_KO; ++q) acc[q] = 0.0;
-    const bool whole = i0 + FWH_KO <= T;
-    for (int w = 0; w < npc; ++w) {
-        const double* cf = sh + w * FWH_SH;
-        const int j0 = i0 + jbs[w];
-        const double* xp = X + xoff[w];
-        if (whole && j0 >= 0 && j0 + FWH_KO + 3 <= nt) {
-            double c[FWH_KO + 3];
+    for (int v = 0; v < 4; ++v) {
+        const int4 q = xp[fwh_slot(at, v)];
+        a += static_cast<long long>(c[4 * v]) * q.x;
+        b += static_cast<long long>(c[4 * v]) * q.y;
+        b += static_cast<long long>(c[4 * v + 1]) * q.x;
+        a += static_cast<long long>(c[4 * v + 2]) * q.z;
+        b += static_cast<long long>(c[4 * v + 2]) * q.w;
+        b += static_cast<long long>(c[4 * v + 3]) * q.z;
+    }
+    return a + (b >> 30);
+}
+// sample i of a panel copy whose stencil runs over an end of the record: the
+// stencil is clamped to the record and its weights are the sample's own
+__device__ __noinline__ void fwh_end(const FwhPc* rc, const int4* xp, int nt, int i, long long* hh, long long* mid) {
+    int c[2 * NSER];
 #pragma unroll
-            for (int m = 0; m < FWH_KO + 3; ++m) {
-                double Ik = 0.0;
+    for (int v = 0; v < 2 * NSER; v += 4) *reinterpret_cast<int4*>(c + v) = *reinterpret_cast<const int4*>(rc->c + v);
+    const double s = double(i) + rc->off;
+    const int j = max(0, min(nt - 4, int(floor(s)) - 1));
+    double wt[4];
+    cubic_weights(s - double(j), wt);
+    long long a = 0, b = 0;
+    for (int m = 0; m < 4; ++m) {
+        const int2 q = fwh_limbs(fwh_integrand(c, xp, fwh_place(j + m, nt)));
+        const int2 w = fwh_limbs(__double2ll_rn(scalbn(wt[m], rc->sc)));
+        a += static_cast<long long>(w.x) * q.x;
+        b += static_cast<long long>(w.x) * q.y;
+        b += static_cast<long long>(w.y) * q.x;
+    }
+    *hh = a + (b >> 30);
+    *mid = b & ((1ll << 30) - 1);
+}
+
+__global__ void __launch_bounds__(32 * ACC_WARPS, 3)
+    k_fwh_accum(const int4* __restrict__ X, const int* __restrict__ hwb, int nt, int p0, int np, int nrows,
+                const double* __restrict__ y, const double* __restrict__ dS, const __grid_constant__ FwhConst k,
+                const FwhObs* __restrict__ obs, int Tmax, int ncopies, double Lspan, int group,
+                double* __restrict__ partial) {
+    __shared__ __align__(16) FwhPc rec[ACC_PC];
+    __shared__ int s_top, s_wide;
+    const int o = blockIdx.x, row = blockIdx.y;
+    const int lane = threadIdx.x & 31;
+    const int T = obs[o].T;
+    const int unit = lane + ACC_LANES * (int(blockIdx.z) * int(blockDim.x >> 5) + int(threadIdx.x >> 5));
+    const int i0 = KO * unit;
+    const bool mine = lane < ACC_LANES && i0 < T;              // this lane stores samples i0.. of its own
+    const bool idle = __shfl_sync(0xffffffffu, i0, 0) >= T;    // no lane of this warp does
+    const int gp0 = row * group, gnp = min(group, np - gp0);   // panels of this block, within the batch
+    const int npc = gnp * ncopies, K = (ncopies - 1) / 2;
+    double* out = partial + (int64_t(o) * nrows + row) * Tmax;   // adds up over the batches of panels
+    const int headroom = 33 - __clz(min(npc, ACC_PC));         // b: 2^b >= 2 npc
+    for (int c0 = 0; c0 < npc; c0 += ACC_PC) {
+        const int n = min(ACC_PC, npc - c0);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            s_top = INT_MIN;
+            s_wide = 0;
+        }
+        __syncthreads();
+        // coefficients and weights of this chunk's panel copies
+        for (int base = 0; base < n; base += blockDim.x) {
+            const int w = base + threadIdx.x;
+            int E = INT_MIN;
+            if (w < n) {
+                FwhPc& rc = rec[w];
+                const int pl = gp0 + (c0 + w) / ncopies, cc = (c0 + w) % ncopies - K;
+                const int* hw = hwb + pl * 8;
+                double cf[NSER], off;
+                fwh_panel(y, dS, p0 + pl, cc, Lspan, obs[o], k, cf, &off);
+                bool fixed = fabs(off) < 1e9 && !fwh_wide_panel(hw);
 #pragma unroll
-                for (int v = 0; v < NSER; ++v) Ik += cf[v] * xp[v * nt + j0 + m];
-                c[m] = Ik;
-            }
-#pragma unroll
-            for (int q = 0; q < FWH_KO; ++q) {
-                double sum = 0.0;
-#pragma unroll
-                for (int m = 0; m < 4; ++m) sum += cf[NSER + m] * c[q + m];
-                acc[q] += sum;
-            }
-        } else {
-            const double off = cf[NSER + 4];
-            for (int q = 0; q < FWH_KO && i0 + q < T; ++q) {
-                const double s = double(i0 + q) + off;
-                int j = int(floor(s)) - 1;
-                j = max(0, min(nt - 4, j));
-                const double x = s - double(j);
-                const double wt[4] = {-(x - 1.0) * (x - 2.0) * (x - 3.0) / 6.0, x * (x - 2.0) * (x - 3.0) / 2.0,
-                                      -x * (x - 1.0) * (x - 3.0) / 2.0, x * (x - 1.0) * (x - 2.0) / 6.0};
-                double sum = 0.0;
-#pragma unroll
-                for (int m = 0; m < 4; ++m) {
-                    double Ik = 0.0;
-#pragma unroll
-                    for (int v = 0; v < NSER; ++v) Ik += cf[v] * xp[v * nt + j + m];
-                    sum += wt[m] * Ik;
+                for (int v = 0; v < NSER; ++v) {
+                    const int ex = (__double2hiint(cf[v]) >> 20) & 0x7ff;
+                    fixed = fixed && ex != 0x7ff && (ex != 0 || cf[v] == 0.0);
+                    if (ex != 0 && hw[v] != 0) E = max(E, ex + (hw[v] >> 20) - 2044);
                 }
-                acc[q] += sum;
+                rc.kind = !fixed ? 0 : E == INT_MIN ? 2 : 1;
+                if (rc.kind == 1) {
+                    E += 3;   // eight terms
+#pragma unroll
+                    for (int v = 0; v < NSER; ++v) {
+                        const int ex = (__double2hiint(cf[v]) >> 20) & 0x7ff;
+                        const int2 q = hw[v] == 0 ? make_int2(0, 0)
+                                                  : fwh_limbs(fwh_fix(cf[v], 4, E - 3 - (ex + (hw[v] >> 20) - 2044)));
+                        rc.c[2 * v] = q.x;
+                        rc.c[2 * v + 1] = q.y;
+                    }
+                    const int jb = int(floor(off)) - 1;
+#pragma unroll
+                    for (int m = 0; m < KO; ++m) rc.at[m] = fwh_place(jb + m, nt);
+                    rc.jb = jb;
+                    atomicMax(&s_top, E);
+                } else {
+                    E = INT_MIN;
+                    if (rc.kind == 0) s_wide = 1;
+                }
+                rc.p = pl;
+                rc.cc = cc;
+                rc.E = E;
+                rc.off = off;
             }
         }
-    }
+        __syncthreads();
+        const int top = s_top;
+        for (int w = threadIdx.x; w < n; w += blockDim.x) {
+            FwhPc& rc = rec[w];
+            if (rc.kind != 1) continue;
+            const int sc = max(-200, 60 - headroom + rc.E - top);
+            rc.sc = sc;
+            double wt[4];
+            cubic_weights(rc.off - floor(rc.off) + 1.0, wt);   // position in the stencil, [1, 2)
 #pragma unroll
-    for (int q = 0; q < FWH_KO; ++q)
-        if (i0 + q < T) partial[int64_t(blockIdx.x) * T + i0 + q] = acc[q];
+            for (int m = 0; m < 4; ++m) {
+                const int2 q = fwh_limbs(__double2ll_rn(scalbn(wt[m], sc)));
+                rc.w[2 * m] = q.x;
+                rc.w[2 * m + 1] = q.y;
+            }
+        }
+        __syncthreads();
+        if (idle) continue;
+        long long hh[KO], mid[KO];
+#pragma unroll
+        for (int q = 0; q < KO; ++q) hh[q] = mid[q] = 0;
+        bool carry = false;
+        int pl = gp0 + c0 / ncopies, copy = c0 % ncopies;   // panel copy w (kept uniform: one base address for all lanes)
+        for (int w = 0; w < n; ++w) {
+            const FwhPc& rc = rec[w];
+            const int4* xp = X + int64_t(pl) * 4 * nt;
+            if (++copy == ncopies) {
+                copy = 0;
+                ++pl;
+            }
+            if (rc.kind != 1) continue;
+            int ih[KO + 3], il[KO + 3];
+            {
+                int c[2 * NSER];
+#pragma unroll
+                for (int v = 0; v < 2 * NSER; v += 4)
+                    *reinterpret_cast<int4*>(c + v) = *reinterpret_cast<const int4*>(rc.c + v);
+#pragma unroll
+                for (int m = 0; m < KO; ++m) {
+                    // a place outside the record (a lane without samples there) reads the last one
+                    const unsigned at = min(unsigned(rc.at[m] + unit), unsigned(nt - 1));
+                    const int2 q = fwh_limbs(fwh_integrand(c, xp, at));
+                    ih[m] = q.x;
+                    il[m] = q.y;
+                }
+            }
+#pragma unroll
+            for (int m = 0; m < 3; ++m) {
+                ih[KO + m] = __shfl_down_sync(0xffffffffu, ih[m], 1);
+                il[KO + m] = __shfl_down_sync(0xffffffffu, il[m], 1);
+            }
+            const int t0 = i0 + rc.jb;
+            int wt[8];
+            *reinterpret_cast<int4*>(wt) = *reinterpret_cast<const int4*>(rc.w);
+            *reinterpret_cast<int4*>(wt + 4) = *reinterpret_cast<const int4*>(rc.w + 4);
+            auto add = [&](int q) {
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    hh[q] += static_cast<long long>(wt[2 * m]) * ih[q + m];
+                    mid[q] += static_cast<long long>(wt[2 * m]) * il[q + m];
+                    mid[q] += static_cast<long long>(wt[2 * m + 1]) * ih[q + m];
+                }
+            };
+            if (__all_sync(0xffffffffu, !mine || (t0 >= 0 && t0 + min(KO, T - i0) + 2 < nt))) {
+                // lanes without samples, and samples past T, add what is never stored
+#pragma unroll
+                for (int q = 0; q < KO; ++q) add(q);
+            } else if (mine) {
+#pragma unroll
+                for (int q = 0; q < KO; ++q)
+                    if (t0 + q >= 0 && t0 + q + 3 < nt) {
+                        add(q);
+                    } else if (i0 + q < T) {
+                        long long a, b;
+                        fwh_end(&rc, xp, nt, i0 + q, &a, &b);
+                        hh[q] += a;
+                        mid[q] += b;
+                    }
+            }
+            // a copy adds at most 2^61 to mid: carry it over every second time
+            carry = !carry;
+            if (!carry)
+#pragma unroll
+                for (int q = 0; q < KO; ++q) {
+                    hh[q] += mid[q] >> 30;
+                    mid[q] &= (1ll << 30) - 1;
+                }
+        }
+        if (mine)
+#pragma unroll
+            for (int q = 0; q < KO; ++q)
+                if (i0 + q < T) {
+                    double v = top == INT_MIN ? 0.0
+                                              : scalbn(double(hh[q]) + double(mid[q]) * (1.0 / 1073741824.0),
+                                                       top + headroom - 60);
+                    if (s_wide)   // panels that are not in fixed point
+                        for (int w = 0; w < n; ++w)
+                            if (rec[w].kind == 0) {
+                                const int* hw = hwb + rec[w].p * 8;
+                                v += fwh_wide_sample(X + int64_t(rec[w].p) * 4 * nt, hw, fwh_wide_panel(hw), nt, y, dS,
+                                              p0 + rec[w].p, rec[w].cc, Lspan, obs + o, k, i0 + q);
+                            }
+                    out[i0 + q] = p0 + c0 == 0 ? v : out[i0 + q] + v;
+                }
+    }
 }
 
 // p'(t_i) = (1/4 pi) sum over panel groups of the partial sums: 32 samples x
 // 32 group slices per block, each slice summing groups g = slice (mod 32) in
 // order, then a fixed-order tree over the slices (the same order every call)
-__global__ void k_fwh_reduce(const double* __restrict__ partial, int ngroups, int T, double* __restrict__ out) {
+__global__ void k_fwh_reduce(const double* __restrict__ partial, int ngroups, int Tmax,
+                             const FwhObs* __restrict__ obs, double* __restrict__ p_out, int cap) {
     __shared__ double red[32][33];
-    const int i = blockIdx.x * 32 + threadIdx.x;
+    const int i = blockIdx.x * 32 + threadIdx.x, o = blockIdx.y, T = obs[o].T;
+    const double* row = partial + int64_t(o) * ngroups * Tmax;
+    double* out = p_out + int64_t(o) * cap;
     double s = 0.0;
     if (i < T)
-        for (int g = threadIdx.y; g < ngroups; g += 32) s += partial[int64_t(g) * T + i];
+        for (int g = threadIdx.y; g < ngroups; g += 32) s += row[int64_t(g) * Tmax + i];
     red[threadIdx.y][threadIdx.x] = s;
     __syncthreads();
     for (int st = 16; st > 0; st >>= 1) {
@@ -252,22 +585,31 @@ namespace {
 // and the panel grouping of the accumulation kernel.
 struct FwhPlan {
     FwhConst k;
-    std::vector<double> tstart;   // first unified time per observer
-    std::vector<int> Tn;          // unified samples per observer
+    std::vector<FwhObs> obs;   // position, first unified time and samples per observer
     int group = 1, ngroups = 1, Tmax = 0;
 };
+
+// Device scratch of one integration: the source series of a batch of panels X
+// [nbatch][4][nt][2] doubles, their largest high words hw [nbatch][8], partial
+// sums [observers of a launch][groups][Tmax] (npartial doubles), and the
+// observer table of a launch (up to OBS_MAX observers) with its delay bounds.
+constexpr int OBS_MAX = 2048;
+struct FwhScratch {
+    double* X = nullptr;
+    int* hw = nullptr;
+    int nbatch = 0;
+    double* partial = nullptr;
+    size_t npartial = 0;
+    FwhObs* obs = nullptr;
+    unsigned long long* ext = nullptr;
+};
+constexpr size_t OBS_BYTES = OBS_MAX * (sizeof(FwhObs) + 2 * sizeof(unsigned long long));
 
 int fwh_plan(int nt, int npts, const double* y, const double* n, const double* dS, const double* hist, double dtau,
              double tau0, const double* obs, int nobs, const double Minf[3], double c0, double rho0, double p0,
              double Lspan, int ncopies, const double* p_out, int cap, const int* nt_out, const double* t0_out,
-             cudaStream_t s, FwhPlan& pl) {
-    if (!hist || !y || !n || !dS || !obs || !Minf || !p_out || !nt_out || !t0_out)
-        return fr_set_error_from_fwh(FR_EINVAL, "null argument");
-    if (nt < 5 || npts < 1 || nobs < 1 || cap < 1 || ncopies < 1 || ncopies % 2 == 0 || !(dtau > 0.0) ||
-        !(c0 > 0.0))
-        return fr_set_error_from_fwh(FR_EINVAL, "bad sizes (nt >= 5, odd ncopies, dtau > 0, c0 > 0 required)");
+             cudaStream_t s, const FwhScratch& sc, FwhPlan& pl) {
     const double MM = Minf[0] * Minf[0] + Minf[1] * Minf[1] + Minf[2] * Minf[2];
-    if (!(MM < 1.0)) return fr_set_error_from_fwh(FR_EINVAL, "|Minf| must be below 1");
     FwhConst& k = pl.k;
     for (int i = 0; i < 3; ++i) k.M[i] = Minf[i];
     k.c0 = c0;
@@ -276,72 +618,113 @@ int fwh_plan(int nt, int npts, const double* y, const double* n, const double* d
     k.dtau = dtau;
     k.tau0 = tau0;
     k.b2 = 1.0 / (1.0 - MM);
-    // unified observer windows (host, double): needs panel positions
-    std::vector<double> yh(size_t(npts) * 3);
-    if (cudaMemcpyAsync(yh.data(), y, yh.size() * 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-        return fr_set_error_from_fwh(FR_ECUDA, "cannot read panel positions");
-    const int K = (ncopies - 1) / 2;
-    pl.tstart.assign(nobs, 0.0);
-    pl.Tn.assign(nobs, 0);
-    for (int o = 0; o < nobs; ++o) {
-        double dmax = -1e300, dmin = 1e300;
-        for (int p = 0; p < npts; ++p)
-            for (int cc = -K; cc <= K; ++cc) {
-                double r[3] = {obs[o * 3 + 0] - yh[p * 3 + 0], obs[o * 3 + 1] - yh[p * 3 + 1],
-                               obs[o * 3 + 2] - (yh[p * 3 + 2] + cc * Lspan)};
-                double Mr = 0, rr = 0;
-                for (int i = 0; i < 3; ++i) {
-                    Mr += Minf[i] * r[i];
-                    rr += r[i] * r[i];
-                }
-                const double Rs = std::sqrt(rr + k.b2 * Mr * Mr) / std::sqrt(k.b2);
-                const double d = k.b2 * (Rs - Mr) / c0;
-                dmax = std::max(dmax, d);
-                dmin = std::min(dmin, d);
-            }
-        const double ts = tau0 + dmax;
-        const double te = tau0 + (nt - 1) * dtau + dmin;
-        if (te < ts) return fr_set_error_from_fwh(FR_EWINDOW, "empty observer window");
-        const int T = int(std::floor((te - ts) / dtau + 1e-9)) + 1;
-        if (T > cap) return fr_set_error_from_fwh(FR_EWINDOW, "observer window longer than the output capacity");
-        pl.tstart[o] = ts;
-        pl.Tn[o] = T;
+    pl.obs.assign(nobs, FwhObs{});
+    for (int o = 0; o < nobs; ++o)
+        for (int i = 0; i < 3; ++i) pl.obs[o].x[i] = obs[o * 3 + i];
+    // unified observer windows from the delay bounds
+    std::vector<unsigned long long> ext(2 * size_t(std::min(nobs, OBS_MAX)));
+    for (int o0 = 0; o0 < nobs; o0 += OBS_MAX) {
+        const int no = std::min(OBS_MAX, nobs - o0);
+        cudaError_t e = cudaMemcpyAsync(sc.obs, pl.obs.data() + o0, sizeof(FwhObs) * no, cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(sc.ext, 0, 16 * size_t(no), s);
+        if (e == cudaSuccess) {
+            const int64_t pcs = int64_t(npts) * ncopies;
+            k_fwh_delays<<<dim3(unsigned(std::min<int64_t>((pcs + 255) / 256, 1024)), no), 256, 0, s>>>(
+                y, npts, k, sc.obs, ncopies, Lspan, sc.ext);
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = cudaMemcpyAsync(ext.data(), sc.ext, 16 * size_t(no), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) return fr_set_error_from_fwh(FR_ECUDA, "cannot read panel positions");
+        for (int o = 0; o < no; ++o) {
+            if (ext[2 * o + 1] == 0) return fr_set_error_from_fwh(FR_EWINDOW, "empty observer window");   // NaN panels
+            double dmax, dmin;
+            const unsigned long long lo = ~ext[2 * o + 1];
+            std::memcpy(&dmax, &ext[2 * o], 8);
+            std::memcpy(&dmin, &lo, 8);
+            const double ts = tau0 + dmax;
+            const double te = tau0 + (nt - 1) * dtau + dmin;
+            if (!(te >= ts)) return fr_set_error_from_fwh(FR_EWINDOW, "empty observer window");
+            const double len = std::floor((te - ts) / dtau + 1e-9) + 1.0;
+            if (!(len <= double(cap)))
+                return fr_set_error_from_fwh(FR_EWINDOW, "observer window longer than the output capacity");
+            pl.obs[o0 + o].tstart = ts;
+            pl.obs[o0 + o].T = int(len);
+            pl.Tmax = std::max(pl.Tmax, int(len));
+        }
     }
     pl.group = std::max(1, kFwhGroup / ncopies);
     pl.ngroups = (npts + pl.group - 1) / pl.group;
-    if ((cap + 128 * FWH_KO - 1) / (128 * FWH_KO) > 65535)
-        return fr_set_error_from_fwh(FR_EINVAL, "observer window too long for one launch");
-    pl.Tmax = *std::max_element(pl.Tn.begin(), pl.Tn.end());
     return FR_OK;
 }
 
-// Scratch of a plan: the source series X [npts][NSER][nt] and one partial-sum
-// row per panel group [ngroups][Tmax], in doubles.
+// the argument checks of an integration (before any device work)
+int fwh_check(const double* hist, int nt, int npts, const double* y, const double* n, const double* dS, double dtau,
+              const double* obs, int nobs, const double* Minf, double c0, int ncopies, const double* p_out, int cap,
+              const int* nt_out, const double* t0_out) {
+    if (!hist || !y || !n || !dS || !obs || !Minf || !p_out || !nt_out || !t0_out)
+        return fr_set_error_from_fwh(FR_EINVAL, "null argument");
+    if (nt < 5 || npts < 1 || nobs < 1 || cap < 1 || ncopies < 1 || ncopies % 2 == 0 || !(dtau > 0.0) ||
+        !(c0 > 0.0))
+        return fr_set_error_from_fwh(FR_EINVAL, "bad sizes (nt >= 5, odd ncopies, dtau > 0, c0 > 0 required)");
+    const double MM = Minf[0] * Minf[0] + Minf[1] * Minf[1] + Minf[2] * Minf[2];
+    if (!(MM < 1.0)) return fr_set_error_from_fwh(FR_EINVAL, "|Minf| must be below 1");
+    if (ncopies > 2003) return fr_set_error_from_fwh(FR_ECUDA, "too many span copies (at most 2003)");
+    if ((cap + 512 - 1) / 512 > 65535)
+        return fr_set_error_from_fwh(FR_EINVAL, "observer window too long for one launch");
+    return FR_OK;
+}
+
+// Scratch that fwh_integrate_noalloc counts against its fixed array, in
+// doubles: the source series of all panels and one row of partial sums per
+// group of kFwhGroup panel copies.
 size_t fwh_series_doubles(int npts, int nt) { return size_t(npts) * NSER * nt; }
 size_t fwh_partial_doubles(const FwhPlan& pl) { return size_t(pl.ngroups) * pl.Tmax; }
 
-// The kernels of one integration on scratch X / partial (both fully written
-// before they are read), then a synchronisation of the stream.
+// The kernels of one integration (all scratch is fully written before it is
+// read), then a synchronisation of the stream.  Panels go in batches of
+// sc.nbatch, whose series are formed once for all observers of a launch.
+// Panels per block: enough for one resident wave of blocks over the GPU, at
+// most what one set-up pass of k_fwh_accum takes, and no fewer than the room for
+// partial sums asks for.
 int fwh_run(const FwhPlan& pl, const double* hist, int nt, int npts, const double* y, const double* n,
             const double* dS, const double* obs, int nobs, double Lspan, int ncopies, double* p_out, int cap,
-            int* nt_out, double* t0_out, double* X, double* partial, cudaStream_t s) {
-    const int64_t nw = int64_t(nt) * npts;
-    k_fwh_series<<<unsigned((nw + 255) / 256), 256, 0, s>>>(hist, nt, npts, n, pl.k, X);
-    const size_t sm = FWH_SH_BYTES * size_t(pl.group) * ncopies;
-    cudaError_t err = cudaGetLastError();
-    if (err == cudaSuccess && sm > 48 * 1024)
-        err = cudaFuncSetAttribute(k_fwh_accum, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
-    for (int o = 0; o < nobs && err == cudaSuccess; ++o) {
-        dim3 grid(unsigned(pl.ngroups), unsigned((pl.Tn[o] + 128 * FWH_KO - 1) / (128 * FWH_KO)));
-        k_fwh_accum<<<grid, 128, sm, s>>>(X, nt, npts, y, dS, pl.k, obs[o * 3 + 0], obs[o * 3 + 1],
-                                          obs[o * 3 + 2], pl.tstart[o], pl.Tn[o], ncopies, Lspan, pl.group,
-                                          partial);
-        k_fwh_reduce<<<unsigned((pl.Tn[o] + 31) / 32), dim3(32, 32), 0, s>>>(partial, pl.ngroups, pl.Tn[o],
-                                                                             p_out + size_t(o) * cap);
+            int* nt_out, double* t0_out, const FwhScratch& sc, cudaStream_t s) {
+    const int warps = (pl.Tmax + ACC_S - 1) / ACC_S, bw = std::min(warps, ACC_WARPS), chunks = (warps + bw - 1) / bw;
+    const int64_t wave = std::max(1, 152 * 24 / bw);
+    const int64_t nb = std::min(npts, sc.nbatch);
+    int group = int(std::min<int64_t>(std::max(1, ACC_PC / ncopies), (nb * nobs * chunks + wave - 1) / wave));
+    while (size_t((nb + group - 1) / group) * pl.Tmax > sc.npartial) ++group;
+    const int batch = nb == npts && npts <= 65535 * group ? npts : int(std::min<int64_t>(nb / group, 65535)) * group;
+    const int ngroups = (batch + group - 1) / group;
+    const int obs_fit = int(std::min<size_t>(OBS_MAX, sc.npartial / (size_t(ngroups) * pl.Tmax)));
+    cudaError_t err = cudaFuncSetAttribute(k_fwh_series, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SER_SMEM));
+    for (int o0 = 0; o0 < nobs && err == cudaSuccess; o0 += obs_fit) {
+        const int no = std::min(obs_fit, nobs - o0);
+        err = cudaMemcpyAsync(sc.obs, pl.obs.data() + o0, sizeof(FwhObs) * no, cudaMemcpyHostToDevice, s);
+        for (int p0 = 0; p0 < npts && err == cudaSuccess; p0 += batch) {
+            const int np = std::min(batch, npts - p0);
+            if (o0 == 0 || batch < npts) {
+                err = cudaMemsetAsync(sc.hw, 0, sizeof(int) * 8 * size_t(np), s);
+                if (err != cudaSuccess) break;
+                k_fwh_series<<<dim3((np + SER_P - 1) / SER_P, (nt + SER_T - 1) / SER_T), 256, SER_SMEM, s>>>(
+                    hist, nt, npts, p0, np, n, pl.k, sc.X, sc.hw);
+                const int64_t places = int64_t(np) * 4 * nt;
+                k_fwh_fix<<<unsigned(std::min<int64_t>((places + 255) / 256, 152 * 32)), 256, 0, s>>>(sc.X, sc.hw, nt, np);
+            }
+            k_fwh_accum<<<dim3(no, (np + group - 1) / group, chunks), 32 * bw, 0, s>>>(
+                reinterpret_cast<const int4*>(sc.X), sc.hw, nt, p0, np, ngroups, y, dS, pl.k, sc.obs,
+                pl.Tmax, ncopies, Lspan, group, sc.partial);
+            err = cudaGetLastError();
+        }
+        if (err != cudaSuccess) break;
+        k_fwh_reduce<<<dim3((pl.Tmax + 31) / 32, no), dim3(32, 32), 0, s>>>(sc.partial, ngroups, pl.Tmax, sc.obs,
+                                                                           p_out + size_t(o0) * cap, cap);
         err = cudaGetLastError();
-        nt_out[o] = pl.Tn[o];
-        t0_out[o] = pl.tstart[o];
+    }
+    for (int o = 0; o < nobs; ++o) {
+        nt_out[o] = pl.obs[o].T;
+        t0_out[o] = pl.obs[o].tstart;
     }
     if (err == cudaSuccess) err = cudaStreamSynchronize(s);
     if (err != cudaSuccess) return fr_set_error_from_fwh(FR_ECUDA, cudaGetErrorString(err));
@@ -355,43 +738,70 @@ extern "C" int fwh_integrate(const double* hist, int nt, int npts, const double*
                              const double Minf[3], double c0, double rho0, double p0, double Lspan,
                              int ncopies, double* p_out, int cap, int* nt_out, double* t0_out, void* stream) {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    FwhPlan pl;
-    int rc = fwh_plan(nt, npts, y, n, dS, hist, dtau, tau0, obs, nobs, Minf, c0, rho0, p0, Lspan, ncopies, p_out,
-                      cap, nt_out, t0_out, s, pl);
+    int rc = fwh_check(hist, nt, npts, y, n, dS, dtau, obs, nobs, Minf, c0, ncopies, p_out, cap, nt_out, t0_out);
     if (rc != FR_OK) return rc;
-    double *X = nullptr, *partial = nullptr;
-    if (cudaMalloc(&X, sizeof(double) * fwh_series_doubles(npts, nt)) != cudaSuccess ||
-        cudaMalloc(&partial, sizeof(double) * fwh_partial_doubles(pl)) != cudaSuccess) {
-        if (X) cudaFree(X);
+    FwhScratch sc;
+    void *tab = nullptr, *buf = nullptr;
+    if (cudaMalloc(&tab, OBS_BYTES) != cudaSuccess)
         return fr_set_error_from_fwh(FR_ENOMEM, "cannot allocate FW-H scratch");
+    sc.obs = static_cast<FwhObs*>(tab);
+    sc.ext = reinterpret_cast<unsigned long long*>(sc.obs + OBS_MAX);
+    FwhPlan pl;
+    rc = fwh_plan(nt, npts, y, n, dS, hist, dtau, tau0, obs, nobs, Minf, c0, rho0, p0, Lspan, ncopies, p_out,
+                  cap, nt_out, t0_out, s, sc, pl);
+    if (rc == FR_OK) {
+        // up to 160 MiB of series at a time and 64 MiB of partial sums (never
+        // less than the panels of one block and the rows of one observer)
+        const size_t per = sizeof(double) * NSER * size_t(nt);
+        sc.nbatch = int(std::min<size_t>(size_t(npts), std::max<size_t>(ACC_PC, (size_t(160) << 20) / per)));
+        const size_t rows = size_t(sc.nbatch) * pl.Tmax * nobs;
+        sc.npartial = std::min(rows, std::max(fwh_partial_doubles(pl), size_t(8) << 20));
+        const size_t nx = fwh_series_doubles(sc.nbatch, nt);
+        if (cudaMalloc(&buf, sizeof(double) * (nx + sc.npartial) + 32 * size_t(sc.nbatch)) != cudaSuccess) {
+            cudaFree(tab);
+            return fr_set_error_from_fwh(FR_ENOMEM, "cannot allocate FW-H scratch");
+        }
+        sc.X = static_cast<double*>(buf);
+        sc.hw = reinterpret_cast<int*>(sc.X + nx);
+        sc.partial = sc.X + nx + 4 * size_t(sc.nbatch);
+        rc = fwh_run(pl, hist, nt, npts, y, n, dS, obs, nobs, Lspan, ncopies, p_out, cap, nt_out, t0_out, sc, s);
+        cudaFree(buf);
     }
-    rc = fwh_run(pl, hist, nt, npts, y, n, dS, obs, nobs, Lspan, ncopies, p_out, cap, nt_out, t0_out, X, partial, s);
-    cudaFree(X);
-    cudaFree(partial);
+    cudaFree(tab);
     return rc;
 }
 
 // ---------------------------------------------------------------------------
 // fwh_integrate_noalloc: the same computation with its scratch (the source
 // series and the partial sums) in a fixed file-scope device array, for callers
-// that cannot call cudaMalloc/cudaFree.  On the host the array's name is only
-// a stand-in, never a device address: every call looks the address up on the
-// current device with cudaGetSymbolAddress (which allocates nothing), so the
-// address always belongs to the context the kernels run in.
+// that cannot call cudaMalloc/cudaFree.  On the host the arrays' names are only
+// stand-ins, never device addresses: every call looks the addresses up on the
+// current device with cudaGetSymbolAddress (which allocates nothing), so they
+// always belong to the context the kernels run in.
 
 namespace {
 
 constexpr size_t kNoallocScratchDoubles = size_t(1) << 22;  // 32 MiB per device
 __device__ __align__(256) double g_fwh_scratch[kNoallocScratchDoubles];
+// the high words of the series' panels (at most 2^22 / (8 * 5) panels fit the
+// scratch) and the observer table
+constexpr size_t kNoallocPanels = kNoallocScratchDoubles / (NSER * 5) + 1;
+__device__ __align__(256) int g_fwh_hw[kNoallocPanels * 8];
+__device__ __align__(256) unsigned char g_fwh_tab[OBS_BYTES];
 
-// Device address of g_fwh_scratch in the current device's context.
-int noalloc_scratch(double** out) {
-    void* p = nullptr;
-    const cudaError_t e = cudaGetSymbolAddress(&p, g_fwh_scratch);
-    if (e != cudaSuccess || !p)
+// Device addresses of the fixed arrays in the current device's context.
+int noalloc_scratch(FwhScratch* sc) {
+    void *p = nullptr, *h = nullptr, *t = nullptr;
+    cudaError_t e = cudaGetSymbolAddress(&p, g_fwh_scratch);
+    if (e == cudaSuccess) e = cudaGetSymbolAddress(&h, g_fwh_hw);
+    if (e == cudaSuccess) e = cudaGetSymbolAddress(&t, g_fwh_tab);
+    if (e != cudaSuccess || !p || !h || !t)
         return fr_set_error_from_fwh(FR_ECUDA, (std::string("cudaGetSymbolAddress of the FW-H scratch: ") +
                                                 cudaGetErrorString(e)).c_str());
-    *out = static_cast<double*>(p);
+    sc->X = static_cast<double*>(p);
+    sc->hw = static_cast<int*>(h);
+    sc->obs = static_cast<FwhObs*>(t);
+    sc->ext = reinterpret_cast<unsigned long long*>(sc->obs + OBS_MAX);
     return FR_OK;
 }
 
@@ -403,9 +813,14 @@ extern "C" int fwh_integrate_noalloc(const double* hist, int nt, int npts, const
                                      int ncopies, double* p_out, int cap, int* nt_out, double* t0_out,
                                      void* stream) {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    int rc = fwh_check(hist, nt, npts, y, n, dS, dtau, obs, nobs, Minf, c0, ncopies, p_out, cap, nt_out, t0_out);
+    if (rc != FR_OK) return rc;
+    FwhScratch sc;
+    rc = noalloc_scratch(&sc);
+    if (rc != FR_OK) return rc;
     FwhPlan pl;
-    int rc = fwh_plan(nt, npts, y, n, dS, hist, dtau, tau0, obs, nobs, Minf, c0, rho0, p0, Lspan, ncopies, p_out,
-                      cap, nt_out, t0_out, s, pl);
+    rc = fwh_plan(nt, npts, y, n, dS, hist, dtau, tau0, obs, nobs, Minf, c0, rho0, p0, Lspan, ncopies, p_out,
+                  cap, nt_out, t0_out, s, sc, pl);
     if (rc != FR_OK) return rc;
     // the series and the partial rows must fit the fixed scratch
     const size_t need = fwh_series_doubles(npts, nt) + fwh_partial_doubles(pl);
@@ -414,9 +829,8 @@ extern "C" int fwh_integrate_noalloc(const double* hist, int nt, int npts, const
             FR_EINVAL, ("fwh_integrate_noalloc: needs " + std::to_string(need) + " doubles of scratch, the fixed "
                         "maximum is " + std::to_string(kNoallocScratchDoubles) +
                         " (8*npts*nt + ceil(npts/max(1,32/ncopies))*window); use fwh_integrate").c_str());
-    double* X = nullptr;
-    rc = noalloc_scratch(&X);
-    if (rc != FR_OK) return rc;
-    return fwh_run(pl, hist, nt, npts, y, n, dS, obs, nobs, Lspan, ncopies, p_out, cap, nt_out, t0_out, X,
-                   X + fwh_series_doubles(npts, nt), s);
+    sc.nbatch = npts;
+    sc.partial = sc.X + fwh_series_doubles(npts, nt);
+    sc.npartial = kNoallocScratchDoubles - fwh_series_doubles(npts, nt);
+    return fwh_run(pl, hist, nt, npts, y, n, dS, obs, nobs, Lspan, ncopies, p_out, cap, nt_out, t0_out, sc, s);
 }
