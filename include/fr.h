@@ -333,7 +333,8 @@ int fwh_integrate(const double* hist, int nt, int npts, const double* y, const d
  * convenience.  Same arguments, results and errors as fwh_integrate, but it
  * allocates no device memory: its scratch lives in one fixed device array
  * of 2^22 doubles (32 MiB; its tables take 3.5 MB more) that the library
- * reserves on every GPU it is loaded on, until the process exits.  It is for callers that cannot call
+ * reserves on every GPU it is loaded on, until the process exits.  It is for
+ * callers that cannot call
  * cudaMalloc/cudaFree, e.g. an application whose device memory is all owned
  * by its own pool allocator, or one that must not pay the device-wide
  * synchronisation of cudaFree in the middle of its work.

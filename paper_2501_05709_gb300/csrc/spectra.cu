@@ -4,11 +4,10 @@
 // length L = 2 floor(nt / (nseg + 1)), step L / 2, periodic Hann window, each
 // segment's mean removed, one-sided density averaged over the segments.
 //
-// Three kernels, all FP64: the table of cos/sin(2 pi m / L); the windowed,
-// mean-free segments (one block per observer and segment, fixed-order
-// reduction); and a direct DFT with one thread per (observer, frequency) that
-// streams each segment through shared memory and walks the twiddle index
-// k n mod L incrementally (no modulo, no per-term trigonometry).
+// Two kernels, all FP64: the table of cos/sin(2 pi m / L) and the windowed,
+// mean-free segments y_n folded about L / 2 (one block per observer and segment,
+// fixed-order reduction); and a direct DFT of the folded segments, one warp per
+// pair of frequencies.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -20,19 +19,22 @@ int fr_set_error_from_fwh(int code, const char* msg);
 
 namespace {
 
-__global__ void k_psd_twiddle(int L, double2* __restrict__ cs) {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= L) return;
-    double s, c;
-    sincospi(2.0 * double(m) / double(L), &s, &c);
-    cs[m] = make_double2(c, s);
-}
-
-// ws[o][s][n] = w_n (x[o][s*step + n] - mean of the segment), w_n = (1 - cos(2 pi n / L)) / 2
-__global__ void k_psd_segments(const double* __restrict__ p, int ld, int L, const double2* __restrict__ cs,
+// Blocks x < nseg: segment x of observer y, folded: with y_n = w_n (x_n - mean),
+// w_n = (1 - cos(2 pi n / L)) / 2 and H = L / 2, ws[o][s][0][n] = y_n + y_{L-n},
+// ws[o][s][1][n] = y_n - y_{L-n} for 0 < n < H; y_n and 0 at n = 0 and H.
+// Blocks x = nseg, together: the table cs[m] = (cos, sin)(2 pi m / L).
+__global__ void k_psd_segments(const double* __restrict__ p, int ld, int L, double2* __restrict__ cs,
                                double* __restrict__ ws) {
-    const int s = blockIdx.x, o = blockIdx.y, nseg = gridDim.x;
-    const double* x = p + size_t(o) * ld + size_t(s) * (L / 2);
+    const int s = blockIdx.x, o = blockIdx.y, nseg = int(gridDim.x) - 1, H = L / 2;
+    if (s == nseg) {
+        for (int64_t m = int64_t(o) * blockDim.x + threadIdx.x; m < L; m += int64_t(gridDim.y) * blockDim.x) {
+            double sn, c;
+            sincospi(2.0 * double(m) / double(L), &sn, &c);
+            cs[m] = make_double2(c, sn);
+        }
+        return;
+    }
+    const double* x = p + size_t(o) * ld + size_t(s) * H;
     __shared__ double red[256];
     double acc = 0.0;
     for (int n = threadIdx.x; n < L; n += blockDim.x) acc += x[n];
@@ -43,45 +45,75 @@ __global__ void k_psd_segments(const double* __restrict__ p, int ld, int L, cons
         __syncthreads();
     }
     const double mean = red[0] / double(L);
-    double* out = ws + (size_t(o) * nseg + s) * L;
-    for (int n = threadIdx.x; n < L; n += blockDim.x) out[n] = (0.5 - 0.5 * cs[n].x) * (x[n] - mean);
+    double* even = ws + (size_t(o) * nseg + s) * 2 * (H + 1);
+    double* odd = even + H + 1;
+    for (int n = threadIdx.x; n <= H; n += blockDim.x) {
+        double sn, c;
+        sincospi(2.0 * double(n) / double(L), &sn, &c);
+        const double w = 0.5 - 0.5 * c, a = w * (x[n] - mean);
+        const bool mid = n > 0 && n < H;
+        const double b = mid ? w * (x[L - n] - mean) : 0.0;   // w_{L-n} = w_n
+        even[n] = a + b;
+        odd[n] = mid ? a - b : 0.0;
+    }
 }
 
-constexpr int PSD_TILE = 2048;   // segment samples staged per pass (16 KB)
-
-// psd[o][k] = scale_k * mean over segments of |sum_n ws_n e^{-2 pi i k n / L}|^2
-__global__ void k_psd_dft(const double* __restrict__ ws, int nseg, int L, const double2* __restrict__ cs,
-                          double inv_norm, double* __restrict__ psd, int cap) {
-    __shared__ double tile[PSD_TILE];
-    const int o = blockIdx.y;
-    const int nf = L / 2 + 1;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    double acc = 0.0;
-    for (int s = 0; s < nseg; ++s) {
-        const double* y = ws + (size_t(o) * nseg + s) * L;
-        double re = 0.0, im = 0.0;
-        int idx = 0;
-        for (int n0 = 0; n0 < L; n0 += PSD_TILE) {
-            const int cnt = min(PSD_TILE, L - n0);
-            __syncthreads();
-            for (int n = threadIdx.x; n < cnt; n += blockDim.x) tile[n] = y[n0 + n];
-            __syncthreads();
-            if (k < nf) {
-                for (int n = 0; n < cnt; ++n) {
-                    const double2 t = cs[idx];
-                    re += tile[n] * t.x;
-                    im -= tile[n] * t.y;
-                    idx += k;
-                    if (idx >= L) idx -= L;
+// psd[o][k] = scale_k * mean over segments of |sum_n y_n e^{-2 pi i k n / L}|^2.
+// A warp forms frequencies k and H - k (H = L / 2) from the same products: with
+// theta = 2 pi k n / L the angle of H - k is pi n - theta, so its cosine and sine
+// are (-1)^n cos and -(-1)^n sin theta, and the sums over even and odd n give both
+// frequencies.  With the fold about H that is a quarter of the direct sum's FP64
+// operations.  Lane l takes n = l (mod 32), so its n keep their parity, and walks
+// the twiddle index k n mod L without a division.  Bound by latency at one
+// observer (a chain of H / 32 steps; L = 974: 264 us with one thread per frequency, 30 us
+// here) and by the FP64 pipe at many (36 observers, L = 324: 28 us).
+constexpr int PSD_WARPS = 8, PSD_SEG = 4;
+__global__ void __launch_bounds__(32 * PSD_WARPS) k_psd_dft(const double* __restrict__ ws, int nseg, int L,
+                                                            const double2* __restrict__ cs, double inv_norm,
+                                                            double* __restrict__ psd, int cap) {
+    const int o = blockIdx.y, lane = threadIdx.x & 31, H = L / 2;
+    const int k = blockIdx.x * PSD_WARPS + (threadIdx.x >> 5);
+    if (2 * k > H) return;
+    const int step = int((32ll * k) % L), idx0 = int((static_cast<long long>(k) * lane) % L);
+    double pa = 0.0, pb = 0.0;   // powers at k and H - k, summed over the segments
+    for (int s0 = 0; s0 < nseg; s0 += PSD_SEG) {
+        const int ns = min(PSD_SEG, nseg - s0);
+        const double* y = ws + (size_t(o) * nseg + s0) * 2 * (H + 1);
+        double re[PSD_SEG], im[PSD_SEG];
+#pragma unroll
+        for (int s = 0; s < PSD_SEG; ++s) re[s] = im[s] = 0.0;
+        int idx = idx0;
+        for (int n = lane; n <= H; n += 32) {
+            const double2 t = cs[idx];
+#pragma unroll
+            for (int s = 0; s < PSD_SEG; ++s)
+                if (s < ns) {
+                    re[s] += y[s * 2 * (H + 1) + n] * t.x;
+                    im[s] -= y[(s * 2 + 1) * (H + 1) + n] * t.y;
                 }
+            idx += step;
+            if (idx >= L) idx -= L;
+        }
+#pragma unroll
+        for (int s = 0; s < PSD_SEG; ++s) {
+#pragma unroll
+            for (int d = 16; d > 1; d >>= 1) {
+                re[s] += __shfl_xor_sync(0xffffffffu, re[s], d);
+                im[s] += __shfl_xor_sync(0xffffffffu, im[s], d);
+            }
+            const double ro = __shfl_xor_sync(0xffffffffu, re[s], 1), io = __shfl_xor_sync(0xffffffffu, im[s], 1);
+            // lane 0: (re, im) over even n, (ro, io) over odd n
+            const double ra = re[s] + ro, ia = im[s] + io, rb = re[s] - ro, ib = io - im[s];
+            if (s < ns) {
+                pa += ra * ra + ia * ia;
+                pb += rb * rb + ib * ib;
             }
         }
-        acc += re * re + im * im;
     }
-    if (k < nf) {
-        const double c = (k == 0 || 2 * k == L) ? 1.0 : 2.0;
-        psd[size_t(o) * cap + k] = c * acc * inv_norm / double(nseg);
-    }
+    if (lane != 0) return;
+    const double c = (k == 0 ? 1.0 : 2.0) * inv_norm / double(nseg);
+    psd[size_t(o) * cap + k] = c * pa;
+    if (2 * k != H) psd[size_t(o) * cap + H - k] = c * pb;
 }
 
 }  // namespace
@@ -104,20 +136,16 @@ extern "C" int fwh_psd(const double* p, int nobs, int nt, int ld, double dt, int
         w2 += w * w;
     }
     const double inv_norm = dt / w2;   // 1 / (f_s sum w^2)
+    // one allocation: the table, then the folded segments
     double2* cs = nullptr;
-    double* ws = nullptr;
-    if (cudaMalloc(&cs, sizeof(double2) * size_t(L)) != cudaSuccess ||
-        cudaMalloc(&ws, sizeof(double) * size_t(nobs) * nseg * L) != cudaSuccess) {
-        cudaFree(cs);
+    if (cudaMalloc(&cs, sizeof(double2) * size_t(L) + sizeof(double) * size_t(nobs) * nseg * (L + 2)) != cudaSuccess)
         return fr_set_error_from_fwh(FR_ENOMEM, "cannot allocate PSD scratch");
-    }
-    k_psd_twiddle<<<(L + 255) / 256, 256, 0, s>>>(L, cs);
-    k_psd_segments<<<dim3(nseg, nobs), 256, 0, s>>>(p, ld, L, cs, ws);
-    k_psd_dft<<<dim3((nf + 127) / 128, nobs), 128, 0, s>>>(ws, nseg, L, cs, inv_norm, psd, cap);
+    double* ws = reinterpret_cast<double*>(cs + L);
+    k_psd_segments<<<dim3(nseg + 1, nobs), 256, 0, s>>>(p, ld, L, cs, ws);
+    k_psd_dft<<<dim3((L / 4 + PSD_WARPS) / PSD_WARPS, nobs), 32 * PSD_WARPS, 0, s>>>(ws, nseg, L, cs, inv_norm, psd, cap);
     cudaError_t err = cudaGetLastError();
     if (err == cudaSuccess) err = cudaStreamSynchronize(s);
     cudaFree(cs);
-    cudaFree(ws);
     if (err != cudaSuccess) return fr_set_error_from_fwh(FR_ECUDA, cudaGetErrorString(err));
     *nfreq_out = nf;
     return FR_OK;
