@@ -702,15 +702,24 @@ int tpe_of(const fr_ctx* c) {
 }
 int max_epb(const fr_ctx* c) { return tpe_of(c) == 64 ? 15 : 32; }
 
-// default: 8 warps (elements) per block, fewer when a block would need more
+// the default tiles: asked of the launchers (frl::best_tile); the tensor-core
+// residual kernels take 8 elements per block, fewer when a block would need more
 // than 96 KB of shared memory
+template <typename Real>
+void default_launch_of(fr_ctx* c) {
+    for (auto& l : c->lc) l.epb = -1;
+    const frk::Stage<Real> st{0, Real(0), nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+    const int64_t launches = c->launches;
+    int epb[3] = {L_traces<Real>(c, nullptr, nullptr, nullptr), L_visc<Real>(c, nullptr, nullptr, nullptr), 8};
+    if (c->prec < FR_TF32_TC) epb[2] = L_resid<Real>(c, nullptr, nullptr, st, nullptr);
+    else
+        while (epb[2] > 1 && smem_of(c, 2, epb[2]) > 96 * 1024) epb[2] /= 2;
+    c->launches = launches;
+    for (int k = 0; k < 3; ++k) c->lc[k] = frk::Launch{epb[k], tpe_of(c) * epb[k]};
+}
 void default_launch(fr_ctx* c) {
-    for (int k = 0; k < 3; ++k) {
-        int epb = 8;
-        while (epb > 1 && smem_of(c, k, epb) > 96 * 1024) epb /= 2;
-        c->lc[k].epb = epb;
-        c->lc[k].threads = tpe_of(c) * epb;
-    }
+    if (c->prec == FR_FP64) default_launch_of<double>(c);
+    else default_launch_of<float>(c);
 }
 
 size_t smem_of(const fr_ctx* c, int kernel, int epb) {

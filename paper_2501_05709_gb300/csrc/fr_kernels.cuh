@@ -449,11 +449,12 @@ __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(
 //   visc : A su[U] | B sj[F] | C sl[F] | D sg[max(DIM*U, F)]  (D holds the
 //          staged neighbour traces during the face phase; affine meshes need
 //          no gradient volume, so there D is [F] only)
-//   resid: A su[U] | B sj[max(U,F)] (sd after the gradient) | C sc[F]
-//          (staged own viscous fluxes until each entry is replaced by the
-//          common flux of the same face point) | D sF[max(DIM*U, 2F)] (own +
-//          staged neighbour traces during the face phase) | E staged
-//          neighbour viscous fluxes [F] (face phase)
+//   resid: A su[U] | B sj[max(U,F)] (staged own traces until each entry is
+//          replaced by the jump of the same face point; sd after the gradient)
+//          | C sc[F] (staged own viscous fluxes until each entry is replaced by
+//          the common flux of the same face point) | D sF[max(DIM*U, 2F)]
+//          (staged neighbour traces and viscous fluxes during the face phase)
+//          | E S, 1/|J| [G] (curved meshes only)
 template <int DIM, int P>
 struct Smem {
     using Z = Sz<DIM, P>;
@@ -465,13 +466,12 @@ struct Smem {
     static constexpr int visc = vD + imax(DIM * U, F);
     static constexpr int visc_a = vD + F;   // affine: no gradient volume, region D holds the neighbour traces
     static constexpr int rB = U, rC = rB + imax(U, F), rD = rC + F, rE = rD + imax(DIM * U, 2 * F);
-    static constexpr int resid = rE + F;
+    static constexpr int resid = rE;
     // curved meshes also stage the element's S [DIM*DIM][NSP] and 1/|J| [NSP]:
-    // in an extra region after visc's, and in resid's region E once the face
-    // phase is over
+    // in an extra region after visc's and in resid's region E
     static constexpr int G = DIM * DIM * Z::NSP + Z::NSP;
     static constexpr int visc_c = visc + G;
-    static constexpr int resid_c = rE + imax(F, G);
+    static constexpr int resid_c = rE + G;
     // pipelined face kernel on affine meshes: two buffers per element group,
     // each [state U | own traces F | neighbour traces F | S, 1/|J|, normals]
     static constexpr int GEO = (DIM * DIM + 1 + 2 * DIM * DIM + 3) / 4 * 4;
@@ -1368,9 +1368,12 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? 80 : 168) k_visc_face(const Real
 // BND as for k_visc_face; VISC: Navier-Stokes (BR2 viscous terms) or Euler;
 // OPM: the gradient and divergence line operators as FP32 FMAs (0) or on the
 // tensor cores with TF32 (1) or BF16x3 (2) operands (float only).  Register
-// caps: 96 in FP32 (88 for p = 4 in 3D, 3.6% faster there), 168 in FP64.
+// caps in FP32: 88 for p = 4 in 3D and for curved meshes (p = 4 box 227 us, with
+// 72: 229, with 96: 238; 100,000 curved elements at p = 3: 314 us, with 72: 323,
+// with 96: 319), else 72 (Euler box of 50^3 at p = 2: 190 us, with 96: 196; of
+// 40^3 at p = 3: 131 against 137; Navier-Stokes the same); 168 in FP64.
 template <int DIM, int P, typename Real, int MP, bool VISC, bool BND, int OPM = 0>
-__global__ void __maxnreg__(sizeof(Real) == 4 ? (DIM == 3 && P == 4 ? 88 : 96) : 168) k_residual(const Real* __restrict__ u, const Real* __restrict__ uf,
+__global__ void __maxnreg__(sizeof(Real) == 4 ? (DIM == 3 && P == 4 || MP == 0 ? 88 : 72) : 168) k_residual(const Real* __restrict__ u, const Real* __restrict__ uf,
                            const Real* __restrict__ fvn, int64_t E, const __grid_constant__ Ops<Real> op,
                            const __grid_constant__ Phys<Real> ph, const __grid_constant__ Geo<Real> g,
                            const __grid_constant__ Stage<Real> st) {
@@ -1391,15 +1394,15 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? (DIM == 3 && P == 4 ? 88 : 96) :
     constexpr bool curved = MP == 0;                // per-point metrics, staged in region E
     constexpr bool diag = MP == 2;                  // affine, diagonal S
     Real* su = reinterpret_cast<Real*>(smem) + warp * (curved ? SM::resid_c : SM::resid);
-    Real* sj = su + SM::rB;              // jumps u_c - u_f      [f][v][fp]
+    Real* sl = su + SM::rB;              // own traces            [f][v][fp]  (face phase)
+    Real* sj = sl;                       // jumps u_c - u_f      [f][v][fp]
     Real* sd = sj;                       // divergence [v][sp], after the gradient
     Real* sc = su + SM::rC;              // Fc.N - own viscous flux [f][v][fp]
-    Real* sF = su + SM::rD;              // own/neighbour traces, q_d, then F~_d  [d][v][sp]
-    Real* sl = sF;                       // own traces            [f][v][fp]  (face phase)
-    Real* sn = sF + NF * NV * NFP;       // neighbour traces      [f][v][fp]  (face phase)
+    Real* sF = su + SM::rD;              // neighbour face data, q_d, then F~_d  [d][v][sp]
+    Real* sn = sF;                       // neighbour traces      [f][v][fp]  (face phase)
+    Real* sm = sF + NF * NV * NFP;       // neighbour viscous fluxes [f][v][fp] (face phase)
     Real* so = sc;                       // own viscous fluxes    [f][v][fp]  (face phase)
-    Real* sm = su + SM::rE;              // neighbour viscous fluxes [f][v][fp] (face phase)
-    Real* sg = sm;                       // curved: S [k][sp], 1/|J| [sp] (after the face phase)
+    Real* sg = su + SM::rE;              // curved: S [k][sp], 1/|J| [sp]
     const int64_t base = e * NV * NSP;
     int codes[NF];
     {
@@ -1408,8 +1411,8 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? (DIM == 3 && P == 4 ? 88 : 96) :
         for (int f = 0; f < NF; ++f) codes[f] = __shfl_sync(0xffffffffu, mine, f);
     }
     constexpr bool VW = (SM::resid * sizeof(Real)) % 16 == 0 && (SM::resid_c * sizeof(Real)) % 16 == 0;
-    constexpr bool VS = VW && (NV * NFP * sizeof(Real)) % 16 == 0 && (SM::rC * sizeof(Real)) % 16 == 0 &&
-                        (SM::rD * sizeof(Real)) % 16 == 0 && (SM::rE * sizeof(Real)) % 16 == 0;
+    constexpr bool VS = VW && (NV * NFP * sizeof(Real)) % 16 == 0 && (SM::rB * sizeof(Real)) % 16 == 0 &&
+                        (SM::rC * sizeof(Real)) % 16 == 0 && (SM::rD * sizeof(Real)) % 16 == 0;
     warp_stage_vol<DIM, P>(su, u + base, lane, T);
     cp_async_commit();
     warp_stage<NF * NV * NFP, VS>(sl, uf + e * NF * NV * NFP, lane, T);
@@ -1422,6 +1425,13 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? (DIM == 3 && P == 4 ? 88 : 96) :
         }
     if constexpr (VISC) warp_stage<NF * NV * NFP, VS>(so, fvn + e * NF * NV * NFP, lane, T);
     cp_async_commit();
+    // curved meshes: S and 1/|J|, needed after the gradient pass
+    if constexpr (curved) {
+        warp_stage_auto<DIM * DIM * NSP, VW && (SM::rE * sizeof(Real)) % 16 == 0>(sg, g.S + e * g.sS_e, lane, T);
+        warp_stage_auto<NSP, VW && ((SM::rE + DIM * DIM * NSP) * sizeof(Real)) % 16 == 0>(
+            sg + DIM * DIM * NSP, g.iJ + e * g.sJ_e, lane, T);
+        cp_async_commit();
+    }
     // face normals of this lane's face points, and the RK stage arrays (needed
     // only at the end): issue their loads now
     Real Nr[DIM][NFI][DIM];
@@ -1447,7 +1457,7 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? (DIM == 3 && P == 4 ? 88 : 96) :
             }
         }
     }
-    cp_async_wait<0>();
+    cp_async_wait<curved ? 1 : 0>();
     grp_sync<T>(warp);
     // B: common normal flux (Rusanov minus common viscous) and jumps
 #pragma unroll
@@ -1496,14 +1506,6 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? (DIM == 3 && P == 4 ? 88 : 96) :
         }
     }
     grp_sync<T>(warp);
-    // curved meshes: stage S and 1/|J| into region E (free after the face
-    // phase); the copy overlaps the gradient pass
-    if (curved) {
-        warp_stage_auto<DIM * DIM * NSP, VW && (SM::rE * sizeof(Real)) % 16 == 0>(sg, g.S + e * g.sS_e, lane, T);
-        warp_stage_auto<NSP, VW && ((SM::rE + DIM * DIM * NSP) * sizeof(Real)) % 16 == 0>(
-            sg + DIM * DIM * NSP, g.iJ + e * g.sJ_e, lane, T);
-        cp_async_commit();
-    }
     // tensor-core mode: this thread's B fragment of the line operators, and
     // its place in the MMA tiles (warp wg of the element group, g, t)
     static_assert(OPM == 0 || sizeof(Real) == 4, "tensor-core line operators take float data");

@@ -3,6 +3,7 @@
 #include "fr_kernels.cuh"
 
 #include <algorithm>
+#include <atomic>
 
 namespace frl {
 
@@ -36,13 +37,53 @@ cudaError_t prep(K kernel, size_t smem, unsigned long long& done) {
 
 inline unsigned grid_of(int64_t E, int epb) { return unsigned((E + epb - 1) / epb); }
 
+inline int sm_count() {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 1;
+    return n;
+}
+template <typename K>
+int blocks_per_sm(K kernel, int threads, size_t smem) {
+    int n = 0;
+    if (threads > 1024 || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem) != cudaSuccess) n = 0;
+    return n;
+}
+
+// Default elements per block of a kernel (T threads an element, smem(epb) bytes a
+// block) on E elements: the tile that keeps most warps resident, found by the
+// occupancy calculator, since these kernels wait on latency (FP32) and an SM holds
+// 16 to 24 of their warps: at p = 3 k_residual runs 92 us on the 32^3 box with 20
+// warps (2 or 4 elements a block) and 108 us with 16 (8 a block), on 100,000 curved
+// elements 319 against 342 us.  With fewer than 20 elements per SM the last wave
+// counts more than the number of warps, and blocks of one element level it (2,400
+// curved elements in FP64: 420 us against 440 to 510 us with 2 to 8).  `tie`: the
+// tile taken among equal ones if it is one of them, else the smallest above 1.
+template <typename K, typename S>
+int best_tile(K kernel, int T, S smem, int64_t E, int tie = 2) {
+    int best = 1, most = blocks_per_sm(kernel, T, smem(1));
+    if (E < 20 * int64_t(sm_count())) return 1;
+    for (int epb : {8, 6, 1, 4, 3, 2, tie}) {   // of equal ones the last
+        const int n = smem(epb) <= 227 * 1024 ? epb * blocks_per_sm(kernel, T * epb, smem(epb)) : 0;
+        if (n >= most) {
+            most = n;
+            best = epb;
+        }
+    }
+    return best;
+}
+
+// every launcher below: lc.epb < 0 asks for the default tile for E elements (a
+// positive result; nothing is launched), E = 0 only sets the kernel up
 template <int P>
 int traces_p(const FR_REAL* u, FR_REAL* uf, int64_t E, const frk::Ops<FR_REAL>& op, frk::Launch lc,
              cudaStream_t s) {
     auto k = frk::k_traces<FR_DIM, P, FR_REAL>;
-    const size_t sm = frk::smem_traces<FR_DIM, P, FR_REAL>(lc.epb);
+    const auto smem = [](int n) { return frk::smem_traces<FR_DIM, P, FR_REAL>(n); };
+    const size_t sm = smem(std::max(lc.epb, 1));
     static unsigned long long done = 0;
     cudaError_t e = prep(k, sm, done);
+    if (lc.epb < 0) return e == cudaSuccess ? best_tile(k, frk::Grp<FR_DIM, P>::T, smem, E) : 1;
     if (e != cudaSuccess) return int(e);
     if (E == 0) return 0;
     k<<<grid_of(E, lc.epb), frk::Grp<FR_DIM, P>::T * lc.epb, sm, s>>>(u, uf, E, op);
@@ -52,51 +93,40 @@ int traces_p(const FR_REAL* u, FR_REAL* uf, int64_t E, const frk::Ops<FR_REAL>& 
 // metric path of the kernels: 0 per-point metrics, 1 affine, 2 affine with diagonal S
 inline int metric_path(const frk::Geo<FR_REAL>& g) { return g.sS_sp != 0 ? 0 : g.diag ? 2 : 1; }
 
-// Blocks of a persistent launch: as many as fit on every SM at once (threads,
-// registers in units of 8 per thread, shared memory with 1 KB reserved per
-// block), at most one per tile of elements.
-inline unsigned persistent_grid(int64_t E, int epb, int threads, size_t smem, int regs, int nsm) {
-    const int r8 = (std::max(regs, 1) + 7) / 8 * 8;
-    int per = std::min(2048 / threads, 32);
-    per = std::min(per, 65536 / (threads * r8));
-    per = std::min(per, int(233472 / (smem + 1024)));
-    const int64_t cap = int64_t(std::max(per, 1)) * std::max(nsm, 1);
-    return unsigned(std::min<int64_t>(int64_t(grid_of(E, epb)), cap));
-}
-
 template <int P, int MP, bool BND>
 int visc_p(const FR_REAL* u, const FR_REAL* uf, FR_REAL* fvn, int64_t E, const frk::Ops<FR_REAL>& op,
            const frk::Phys<FR_REAL>& ph, const frk::Geo<FR_REAL>& g, frk::Launch lc, cudaStream_t s) {
     if constexpr (MP == 0) {
         auto k = frk::k_visc_face<FR_DIM, P, FR_REAL, MP, BND>;
-        const size_t sm = frk::smem_visc<FR_DIM, P, FR_REAL>(lc.epb, true);
+        const auto smem = [](int n) { return frk::smem_visc<FR_DIM, P, FR_REAL>(n, true); };
+        const size_t sm = smem(std::max(lc.epb, 1));
         static unsigned long long done = 0;
         cudaError_t e = prep(k, sm, done);
+        if (lc.epb < 0) return e == cudaSuccess ? best_tile(k, frk::Grp<FR_DIM, P>::T, smem, E) : 1;
         if (e != cudaSuccess) return int(e);
         if (E == 0) return 0;
         k<<<grid_of(E, lc.epb), frk::Grp<FR_DIM, P>::T * lc.epb, sm, s>>>(u, uf, fvn, E, op, ph, g);
         return int(cudaGetLastError());
     } else {
-        // affine meshes: the pipelined kernel on a persistent grid, sized from
-        // the kernel's registers and the SM count read at set-up (the first,
-        // empty launch at mesh load, outside any stream capture)
+        // affine meshes: the pipelined kernel on a persistent grid of as many
+        // blocks as fit on every SM at once, at most one per tile of elements
+        // (kept per tile: all devices are alike)
         auto k = frk::k_visc_face_aff<FR_DIM, P, FR_REAL, MP, BND>;
-        const size_t sm = frk::smem_visc<FR_DIM, P, FR_REAL>(lc.epb, false);
+        const auto smem = [](int n) { return frk::smem_visc<FR_DIM, P, FR_REAL>(n, false); };
+        const size_t sm = smem(std::max(lc.epb, 1));
         static unsigned long long done = 0;
-        static int regs = 0, nsm = 0;
         cudaError_t e = prep(k, sm, done);
+        if (lc.epb < 0) return e == cudaSuccess ? best_tile(k, frk::Grp<FR_DIM, P>::T, smem, E, 4) : 1;
         if (e != cudaSuccess) return int(e);
-        if (!regs) {
-            cudaFuncAttributes fa;
-            int dev = 0;
-            if ((e = cudaFuncGetAttributes(&fa, k)) != cudaSuccess) return int(e);
-            if ((e = cudaGetDevice(&dev)) != cudaSuccess) return int(e);
-            if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return int(e);
-            regs = fa.numRegs;
-        }
         if (E == 0) return 0;
         const int threads = frk::Grp<FR_DIM, P>::T * lc.epb;
-        k<<<persistent_grid(E, lc.epb, threads, sm, regs, nsm), threads, sm, s>>>(u, uf, fvn, E, op, ph, g);
+        static std::atomic<int> resident[33];
+        int cap = resident[lc.epb & 31].load();
+        if (cap == 0) {
+            cap = std::max(1, blocks_per_sm(k, threads, sm)) * sm_count();
+            resident[lc.epb & 31].store(cap);
+        }
+        k<<<std::min(grid_of(E, lc.epb), unsigned(cap)), threads, sm, s>>>(u, uf, fvn, E, op, ph, g);
         return int(cudaGetLastError());
     }
 }
@@ -106,9 +136,12 @@ int resid_p(const FR_REAL* u, const FR_REAL* uf, const FR_REAL* fvn, int64_t E,
             const frk::Ops<FR_REAL>& op, const frk::Phys<FR_REAL>& ph, const frk::Geo<FR_REAL>& g,
             const frk::Stage<FR_REAL>& st, frk::Launch lc, cudaStream_t s) {
     auto k = frk::k_residual<FR_DIM, P, FR_REAL, MP, VISC, BND>;
-    const size_t sm = frk::smem_resid<FR_DIM, P, FR_REAL>(lc.epb, g.sS_sp != 0);
+    const bool curved = g.sS_sp != 0;
+    const auto smem = [curved](int n) { return frk::smem_resid<FR_DIM, P, FR_REAL>(n, curved); };
+    const size_t sm = smem(std::max(lc.epb, 1));
     static unsigned long long done = 0;
     cudaError_t e = prep(k, sm, done);
+    if (lc.epb < 0) return e == cudaSuccess ? best_tile(k, frk::Grp<FR_DIM, P>::T, smem, E) : 1;
     if (e != cudaSuccess) return int(e);
     if (E == 0) return 0;
     k<<<grid_of(E, lc.epb), frk::Grp<FR_DIM, P>::T * lc.epb, sm, s>>>(u, uf, fvn, E, op, ph, g, st);
