@@ -100,6 +100,7 @@ struct fr_ctx {
     void* hlen = nullptr;                // device Real [E]: element length
     int64_t* cand_off_d = nullptr;       // device [ncand + 1]
     unsigned long long* lam = nullptr;   // device [ncand]: max spectral rate (double bits)
+    float* cfl_up = nullptr;             // device [E + ncand]: FP32 bounds of the rates (not in FP64)
     // variable polynomial order (sponge zones), see frk::Sponge
     std::vector<std::vector<int32_t>> order;  // per candidate: [count] degree caps (empty: all p)
     int sp_n = 0;                             // capped elements (0: none)
@@ -453,12 +454,14 @@ int enqueue_adaptive_dt(fr_ctx* c, cudaStream_t s) {
     const auto ph = phys_of<Real>(c);
     const Real* u = static_cast<const Real*>(c->u0);
     const Real* h = static_cast<const Real*>(c->hlen);
-    int rc = c->dim == 2 ? frl::cfl<Real, 2>(c->p, u, h, c->E, c->cand_off_d, c->ncand, ph, c->lam, s)
-                         : frl::cfl<Real, 3>(c->p, u, h, c->E, c->cand_off_d, c->ncand, ph, c->lam, s);
+    unsigned* low = reinterpret_cast<unsigned*>(c->cfl_up ? c->cfl_up + c->E : nullptr);
+    if (low) CK(cudaMemsetAsync(low, 0, sizeof(unsigned) * c->ncand, s));
+    int rc = c->dim == 2 ? frl::cfl<Real, 2>(c->p, u, h, c->E, c->cand_off_d, c->ncand, ph, c->lam, c->cfl_up, low, s)
+                         : frl::cfl<Real, 3>(c->p, u, h, c->E, c->cand_off_d, c->ncand, ph, c->lam, c->cfl_up, low, s);
     CKL(rc, "time step kernel");
     k_dt_fill<Real><<<256, 256, 0, s>>>(c->lam, c->adaptive_cfl, c->cand_off_d, c->ncand, c->E,
                                         static_cast<Real*>(c->dte), c->dtc);
-    c->launches += 2;
+    c->launches += low ? 3 : 2;
     CK(cudaGetLastError());
     return FR_OK;
 }
@@ -735,7 +738,8 @@ void release(fr_ctx* c) {
     void* bufs[] = {c->u0, c->us, c->acc, c->ufb[0], c->ufb[1], c->fvn, c->S, c->J, c->iJ, c->N, c->nbr,
                     c->wall_ef, c->wall_off_d, c->fnow, c->fsum, c->fcnt, c->partial, c->stage64, c->dte,
                     c->fpart, c->src_elem, c->src_cand, c->src_w, c->src_A, c->src_f, c->tnow, c->dtc,
-                    c->hlen, c->cand_off_d, c->lam, c->sp_elem, c->sp_cap, c->nonfinite, c->ufb3};
+                    c->hlen, c->cand_off_d, c->lam, c->sp_elem, c->sp_cap, c->nonfinite, c->ufb3,
+                    c->cfl_up};
     for (void* b : bufs)
         if (b) cudaFree(b);
     for (int q = 0; q < frk::MAXNP; ++q) {
@@ -1726,6 +1730,10 @@ int ensure_dt_buffers(fr_ctx* c) {
     }
     if (!c->lam && cudaMalloc(&c->lam, nc * sizeof(unsigned long long)) != cudaSuccess)
         return fail(FR_ENOMEM, "cannot allocate step buffers");
+    if (!c->cfl_up && c->prec != FR_FP64 && cudaMalloc(&c->cfl_up, (size_t(c->E) + nc) * sizeof(float)) != cudaSuccess) {
+        c->cfl_up = nullptr;
+        return fail(FR_ENOMEM, "cannot allocate step buffers");
+    }
     return FR_OK;
 }
 

@@ -213,10 +213,11 @@ int source_stage(int P, const frk::Src<Real>& src, const frk::Stage<Real>& st, c
                  void* stream);
 
 // per-candidate maximum spectral rate of the adaptive time step (lam holds
-// the bits of non-negative doubles, zeroed by the caller)
+// the bits of non-negative doubles, zeroed by the caller).  up [E] and low [ncand]
+// (zeroed; null: none, for FP64): scratch of the FP32 bounds that leave most elements out
 template <typename Real, int DIM>
 int cfl(int P, const Real* u, const Real* hlen, int64_t E, const int64_t* cand_off, int ncand,
-        const frk::Phys<Real>& ph, unsigned long long* lam, void* stream);
+        const frk::Phys<Real>& ph, unsigned long long* lam, float* up, unsigned* low, void* stream);
 
 // residual of the tensor-core precision modes (3D, P = 3 or 4; opm 1: TF32,
 // 2: BF16x3), float data

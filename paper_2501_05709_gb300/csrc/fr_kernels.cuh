@@ -1971,43 +1971,123 @@ __global__ void k_sponge(const __grid_constant__ Sponge<Real> sp, Real* __restri
 // in double, h_e the element length (min over points and directions of
 // 2 |J| / |S[d,:]|, precomputed); the candidate's maximum is kept by an
 // atomic maximum on the bits of the non-negative double (order-independent).
+// Five FP64 divisions and roots a point bind this to the FP64 pipe (708 us on
+// 125,000 elements at p = 2).  For FP32 states k_cfl_bound first takes bounds
+// up_e >= lambda_e in FP32 and the largest lower bound of each candidate; k_cfl then
+// evaluates only the elements whose upper bound reaches it, so the maximum is the
+// same double (708 to about 90 us a
+// step).
+//
+// Bounds of one point: v = |V| + sqrt(gamma p / rho) in FP32 is off by at most 16
+// roundings (divisions and roots by approximations of 2 units in the last place)
+// of each term, the pressure's own cancellation included, which is relative to
+// gamma - 1 times the sum of its two terms: 1e-6 covers 16 roundings of 6e-8.  A
+// point without a positive finite pressure has no bound (up_e = infinity).
 template <int DIM, int P, typename Real>
-__global__ void k_cfl(const Real* __restrict__ u, const Real* __restrict__ hlen, int64_t E,
-                      const int64_t* __restrict__ cand_off, int ncand, const __grid_constant__ Phys<Real> ph,
-                      unsigned long long* __restrict__ lam) {
+__global__ void k_cfl_bound(const Real* __restrict__ u, const Real* __restrict__ hlen, int64_t E,
+                            const int64_t* __restrict__ cand_off, int ncand, const __grid_constant__ Phys<Real> ph,
+                            float* __restrict__ up, unsigned* __restrict__ low) {
     using Z = Sz<DIM, P>;
     constexpr int NSP = Z::NSP, NV = Z::NV;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t e = int64_t(blockIdx.x) * (blockDim.x >> 5) + warp;
     if (e >= E) return;
     const Real* ue = u + e * NV * NSP;
-    double vmax = 0.0, numax = 0.0;
+    const float gm1 = float(ph.gm1), mu = float(ph.mu);
+    float hi = 0.0f, lo = 0.0f, nhi = 0.0f, nlo = 0.0f;
     for (int sp = lane; sp < NSP; sp += 32) {
-        const double rho = double(ue[sp]);
-        double m2 = 0.0;
+        const float rho = float(ue[sp]);
+        float m2 = 0.0f;
 #pragma unroll
         for (int i = 0; i < DIM; ++i) {
-            const double m = double(ue[(1 + i) * NSP + sp]);
+            const float m = float(ue[(1 + i) * NSP + sp]);
             m2 += m * m;
         }
-        const double p = double(ph.gm1) * (double(ue[(NV - 1) * NSP + sp]) - 0.5 * m2 / rho);
-        const double v = sqrt(m2) / rho + sqrt(double(ph.gamma) * p / rho);
-        vmax = fmax(vmax, v);
-        numax = fmax(numax, double(ph.mu) / rho);
+        const float En = float(ue[(NV - 1) * NSP + sp]);
+        const float ir = 1.0f / rho, ke = 0.5f * m2 * ir, p = gm1 * (En - ke);
+        const float V = sqrtf(m2) * ir, c = sqrtf(float(ph.gamma) * p * ir);
+        const float off = 1e-6f * (V + c * (1.0f + gm1 * (fabsf(En) + fabsf(ke)) / p));
+        // (bit tests: fast-math code may drop comparisons with infinity)
+        if (!(p > 0.0f && rho > 0.0f) || not_finite(V) || not_finite(c) || not_finite(off)) {
+            hi = __int_as_float(0x7f800000);
+        } else {
+            hi = fmaxf(hi, V + c + off);
+            lo = fmaxf(lo, V + c - off);
+            const float nu = mu * ir;
+            nhi = fmaxf(nhi, nu * (1.0f + 1e-6f));
+            nlo = fmaxf(nlo, nu * (1.0f - 1e-6f));
+        }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        vmax = fmax(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
-        numax = fmax(numax, __shfl_xor_sync(0xffffffffu, numax, o));
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        lo = fmaxf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        nhi = fmaxf(nhi, __shfl_xor_sync(0xffffffffu, nhi, o));
+        nlo = fmaxf(nlo, __shfl_xor_sync(0xffffffffu, nlo, o));
     }
     if (lane == 0) {
         int c = 0;
         while (c + 1 < ncand && e >= cand_off[c + 1]) ++c;
-        const double h = double(hlen[e]);
-        const double k = double((P + 1) * (P + 1));
-        double l = vmax * k / h;
-        if (ph.viscous) l += numax * k * k / (h * h);
-        atomicMax(lam + c, static_cast<unsigned long long>(__double_as_longlong(l)));
+        const float ih = 1.0f / float(hlen[e]), k = float((P + 1) * (P + 1));
+        const float vis = ph.viscous ? k * k * ih * ih : 0.0f;
+        float l = hi * k * ih + nhi * vis;
+        if (not_finite(hi) || not_finite(l)) l = __int_as_float(0x7f800000);
+        else l *= 1.0f + 1e-6f;
+        up[e] = l;
+        const float b = (lo * k * ih + nlo * vis) * (1.0f - 1e-6f);
+        if (b > 0.0f && !not_finite(b)) atomicMax(low + c, __float_as_uint(b));
+    }
+}
+
+// a warp looks at 32 elements (all of them without bounds) and evaluates, one
+// after the other, those that can hold the candidate's maximum
+template <int DIM, int P, typename Real>
+__global__ void k_cfl(const Real* __restrict__ u, const Real* __restrict__ hlen, int64_t E,
+                      const int64_t* __restrict__ cand_off, int ncand, const __grid_constant__ Phys<Real> ph,
+                      const float* __restrict__ up, const unsigned* __restrict__ low,
+                      unsigned long long* __restrict__ lam) {
+    using Z = Sz<DIM, P>;
+    constexpr int NSP = Z::NSP, NV = Z::NV;
+    const int lane = threadIdx.x & 31;
+    const int64_t e0 = (int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32;
+    if (e0 >= E) return;
+    const int64_t mine = e0 + lane;
+    int c = 0;
+    while (c + 1 < ncand && mine >= cand_off[c + 1]) ++c;
+    // non-negative floats (and infinity) order as their bits do
+    unsigned todo = __ballot_sync(0xffffffffu, mine < E && (!up || __float_as_uint(up[mine < E ? mine : 0]) >= low[c]));
+    while (todo) {
+        const int w = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const int64_t e = e0 + w;
+        const int ce = __shfl_sync(0xffffffffu, c, w);
+        const Real* ue = u + e * NV * NSP;
+        double vmax = 0.0, numax = 0.0;
+        for (int sp = lane; sp < NSP; sp += 32) {
+            const double rho = double(ue[sp]);
+            double m2 = 0.0;
+#pragma unroll
+            for (int i = 0; i < DIM; ++i) {
+                const double m = double(ue[(1 + i) * NSP + sp]);
+                m2 += m * m;
+            }
+            const double p = double(ph.gm1) * (double(ue[(NV - 1) * NSP + sp]) - 0.5 * m2 / rho);
+            const double v = sqrt(m2) / rho + sqrt(double(ph.gamma) * p / rho);
+            vmax = fmax(vmax, v);
+            numax = fmax(numax, double(ph.mu) / rho);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            vmax = fmax(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
+            numax = fmax(numax, __shfl_xor_sync(0xffffffffu, numax, o));
+        }
+        if (lane == 0) {
+            const double h = double(hlen[e]);
+            const double k = double((P + 1) * (P + 1));
+            double l = vmax * k / h;
+            if (ph.viscous) l += numax * k * k / (h * h);
+            atomicMax(lam + ce, static_cast<unsigned long long>(__double_as_longlong(l)));
+        }
     }
 }
 

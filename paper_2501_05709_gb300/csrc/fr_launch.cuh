@@ -296,11 +296,13 @@ int sponge<FR_REAL, FR_DIM>(int P, const frk::Sponge<FR_REAL>& sp, FR_REAL* a, F
 
 template <>
 int cfl<FR_REAL, FR_DIM>(int P, const FR_REAL* u, const FR_REAL* hlen, int64_t E, const int64_t* cand_off,
-                         int ncand, const frk::Phys<FR_REAL>& ph, unsigned long long* lam, void* stream) {
+                         int ncand, const frk::Phys<FR_REAL>& ph, unsigned long long* lam, float* up, unsigned* low,
+                         void* stream) {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (E == 0) return 0;
     const unsigned blocks = unsigned((E + 7) / 8);
-#define C(PP) (frk::k_cfl<FR_DIM, PP, FR_REAL><<<blocks, 256, 0, s>>>(u, hlen, E, cand_off, ncand, ph, lam), \
+#define C(PP) ((up ? (frk::k_cfl_bound<FR_DIM, PP, FR_REAL><<<blocks, 256, 0, s>>>(u, hlen, E, cand_off, ncand, ph, up, low), 0) : 0), \
+               frk::k_cfl<FR_DIM, PP, FR_REAL><<<unsigned((E + 255) / 256), 256, 0, s>>>(u, hlen, E, cand_off, ncand, ph, up, low, lam), \
                int(cudaGetLastError()))
     FR_DISPATCH(C)
 #undef C
