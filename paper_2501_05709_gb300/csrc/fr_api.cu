@@ -72,6 +72,11 @@ struct fr_ctx {
     double *fnow = nullptr, *fsum = nullptr, *fcnt = nullptr, *partial = nullptr, *fpart = nullptr;
     int partial_blocks = 0;
     std::vector<Surface> surf;
+    void* surf_d = nullptr;                  // frk::Surf<Real> of every surface
+    // wall forces and surface records of a step run on aux_stream beside the first
+    // stage's residual kernel (both read the state at the start of the step)
+    cudaStream_t aux_stream = nullptr;
+    cudaEvent_t ev_aux[2] = {nullptr, nullptr};
     frk::Launch lc[3]{};
     cudaStream_t cap_stream = nullptr;
     // the reduced-degree kernels of a step run on red_stream[q] (one per
@@ -394,16 +399,17 @@ int L_forces(fr_ctx* c, cudaStream_t s) {
                                       c->fnow, c->fsum, c->fcnt, s);
 }
 
+// one record of n surfaces from surface `first` on
 template <typename Real>
-int L_sample(fr_ctx* c, Surface& sf, cudaStream_t s) {
+int L_sample(fr_ctx* c, int first, int n, cudaStream_t s) {
+    if (n <= 0) return 0;
     const auto ph = phys_of<Real>(c);
+    int most = 1;
+    for (int k = first; k < first + n; ++k) most = std::max(most, c->surf[size_t(k)].npts);
     c->launches += 2;
-    return c->dim == 2 ? frl::sample<Real, 2>(c->p, static_cast<const Real*>(c->u0), sf.pe,
-                                              static_cast<const Real*>(sf.pw), sf.npts, ph,
-                                              static_cast<Real*>(sf.hist), sf.count, sf.cap, sf.every, s)
-                       : frl::sample<Real, 3>(c->p, static_cast<const Real*>(c->u0), sf.pe,
-                                              static_cast<const Real*>(sf.pw), sf.npts, ph,
-                                              static_cast<Real*>(sf.hist), sf.count, sf.cap, sf.every, s);
+    const auto* sf = static_cast<const frk::Surf<Real>*>(c->surf_d) + first;
+    const Real* u = static_cast<const Real*>(c->u0);
+    return c->dim == 2 ? frl::sample<Real, 2>(c->p, u, sf, n, most, ph, s) : frl::sample<Real, 3>(c->p, u, sf, n, most, ph, s);
 }
 
 // Optional per-launch event pairs for fr_profile_step: kind 0..5.  With
@@ -531,15 +537,20 @@ int enqueue_step(fr_ctx* c, cudaStream_t s, Prof* pr = nullptr) {
             CKL(rc, "viscous face kernel");
             if (fork) CK(join_red(c, s));
         }
+        const bool aux = stage == 1 && ns > 1 && !pr && (!c->surf.empty() || (!c->wall_off.empty() && c->wall_off.back() > 0));
         if (stage == 1) {
-            if (pr) pr->mark_begin(3);
-            rc = L_forces<Real>(c, s);
-            CKL(rc, "forces kernel");
-            for (auto& sf : c->surf) {
-                rc = L_sample<Real>(c, sf, s);
-                CKL(rc, "sampling kernel");
+            cudaStream_t sa = aux ? c->aux_stream : s;
+            if (aux) {
+                CK(cudaEventRecord(c->ev_aux[0], s));
+                CK(cudaStreamWaitEvent(sa, c->ev_aux[0], 0));
             }
+            if (pr) pr->mark_begin(3);
+            rc = L_forces<Real>(c, sa);
+            CKL(rc, "forces kernel");
+            rc = L_sample<Real>(c, 0, int(c->surf.size()), sa);
+            CKL(rc, "sampling kernel");
             if (pr) pr->mark_end();
+            if (aux) CK(cudaEventRecord(c->ev_aux[1], sa));
         }
         frk::Stage<Real> st;
         st.stage = stage;
@@ -585,6 +596,7 @@ int enqueue_step(fr_ctx* c, cudaStream_t s, Prof* pr = nullptr) {
             if (pr) pr->mark_end();
             CKL(rc, "source kernel");
         }
+        if (aux) CK(cudaStreamWaitEvent(s, c->ev_aux[1], 0));
     }
     if (c->src_nentry > 0) {
         k_time_advance<<<1, 32, 0, s>>>(c->tnow, c->dtc, c->ncand);
@@ -739,7 +751,7 @@ void release(fr_ctx* c) {
                     c->wall_ef, c->wall_off_d, c->fnow, c->fsum, c->fcnt, c->partial, c->stage64, c->dte,
                     c->fpart, c->src_elem, c->src_cand, c->src_w, c->src_A, c->src_f, c->tnow, c->dtc,
                     c->hlen, c->cand_off_d, c->lam, c->sp_elem, c->sp_cap, c->nonfinite, c->ufb3,
-                    c->cfl_up};
+                    c->surf_d, c->cfl_up};
     for (void* b : bufs)
         if (b) cudaFree(b);
     for (int q = 0; q < frk::MAXNP; ++q) {
@@ -760,6 +772,9 @@ void release(fr_ctx* c) {
         if (c->ev_join[q]) cudaEventDestroy(c->ev_join[q]);
     }
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
+    if (c->aux_stream) cudaStreamDestroy(c->aux_stream);
+    for (cudaEvent_t ev : c->ev_aux)
+        if (ev) cudaEventDestroy(ev);
     delete c;
 }
 
@@ -1116,7 +1131,10 @@ extern "C" int fr_mesh_load(const fr_mesh_desc* m, int ncand, const fr_options* 
     }
     cudaMemset(c->nonfinite, 0, sizeof(int) * ncand);
     bool streams_ok = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) == cudaSuccess &&
-                      cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) == cudaSuccess;
+                      cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) == cudaSuccess &&
+                      cudaStreamCreateWithFlags(&c->aux_stream, cudaStreamNonBlocking) == cudaSuccess &&
+                      cudaEventCreateWithFlags(&c->ev_aux[0], cudaEventDisableTiming) == cudaSuccess &&
+                      cudaEventCreateWithFlags(&c->ev_aux[1], cudaEventDisableTiming) == cudaSuccess;
     for (int q = 0; q < c->p && streams_ok; ++q)
         streams_ok = cudaStreamCreateWithFlags(&c->red_stream[q], cudaStreamNonBlocking) == cudaSuccess &&
                      cudaEventCreateWithFlags(&c->ev_join[q], cudaEventDisableTiming) == cudaSuccess;
@@ -1852,6 +1870,29 @@ extern "C" int fr_integrals(fr_ctx* c, int cand, double* out) {
 }
 
 // ---------------------------------------------------------------- FW-H surfaces
+namespace {
+
+// the device table of the surfaces (after one was added; work that reads the old
+// table has finished before it is freed)
+template <typename Real>
+int upload_surfaces(fr_ctx* c) {
+    std::vector<frk::Surf<Real>> h;
+    for (const Surface& s : c->surf)
+        h.push_back({s.pe, static_cast<const Real*>(s.pw), static_cast<Real*>(s.hist), s.count, s.npts, s.cap, s.every, 0});
+    void* d = nullptr;
+    const int rc = upload(&d, h);
+    if (rc) {
+        if (d) cudaFree(d);
+        return rc;
+    }
+    CK(cudaDeviceSynchronize());
+    if (c->surf_d) cudaFree(c->surf_d);
+    c->surf_d = d;
+    return FR_OK;
+}
+
+}  // namespace
+
 extern "C" int fwh_register(fr_ctx* c, int cand, int npts, const double* xyz, int capacity, int every,
                             int* handle) {
     if (!c || !xyz || !handle || npts < 1 || capacity < 1 || every < 1 || cand < 0 || cand >= c->ncand)
@@ -1973,6 +2014,13 @@ extern "C" int fwh_register(fr_ctx* c, int cand, int npts, const double* xyz, in
     }
     CK(cudaMemset(sf.count, 0, 3 * sizeof(int)));
     c->surf.push_back(sf);
+    rc = c->prec == FR_FP64 ? upload_surfaces<double>(c) : upload_surfaces<float>(c);
+    if (rc) {
+        c->surf.pop_back();
+        void* sb[] = {sf.pe, sf.pw, sf.hist, sf.count};
+        for (void* b : sb) cudaFree(b);
+        return rc;
+    }
     invalidate_graph(c);
     *handle = int(c->surf.size()) - 1;
     return FR_OK;
@@ -1989,8 +2037,8 @@ extern "C" int fwh_sample(fr_ctx* c, int handle, void* stream) {
     const int phase = cnt[1];
     int aligned[3] = {cnt[0], 0, cnt[2]};
     CK(cudaMemcpy(sf.count, aligned, sizeof(aligned), cudaMemcpyHostToDevice));
-    const int rc = c->prec == FR_FP64 ? L_sample<double>(c, sf, static_cast<cudaStream_t>(stream))
-                                      : L_sample<float>(c, sf, static_cast<cudaStream_t>(stream));
+    const int rc = c->prec == FR_FP64 ? L_sample<double>(c, handle, 1, static_cast<cudaStream_t>(stream))
+                                      : L_sample<float>(c, handle, 1, static_cast<cudaStream_t>(stream));
     CKL(rc, "sampling kernel");
     CK(cudaStreamSynchronize(static_cast<cudaStream_t>(stream)));
     CK(cudaMemcpy(&aligned, sf.count, sizeof(aligned), cudaMemcpyDeviceToHost));

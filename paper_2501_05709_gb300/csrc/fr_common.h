@@ -129,6 +129,18 @@ struct Src {
     double cfac = 0.0;
 };
 
+// An FW-H data surface on the device: element and 1D Lagrange weights [DIM][NP] of
+// each point, history [cap][npts][5] of deviations from the free stream, and
+// count = {records, steps seen, overflow flag}.
+template <typename Real>
+struct Surf {
+    const int64_t* pe;
+    const Real* pw;
+    Real* hist;
+    int* count;
+    int npts, cap, every, pad;
+};
+
 // One warp per element; epb elements (warps) per block.
 struct Launch {
     int epb;          // elements (warps) per block
@@ -192,10 +204,10 @@ int forces(int P, const Real* uf, const Real* fvn, const int32_t* wall_ef, const
            int ncand, const frk::Ops<Real>& op, const frk::Geo<Real>& g, Real gm1, int viscous,
            double* part, double* fnow, double* fsum, double* fcnt, void* stream);
 
-// count: device int[3] = records, steps seen, overflow flag
+// nsurf surfaces (device array), `most` the largest number of points
 template <typename Real, int DIM>
-int sample(int P, const Real* u, const int64_t* pe, const Real* pw, int npts, const frk::Phys<Real>& ph,
-           Real* hist, int* count, int cap, int every, void* stream);
+int sample(int P, const Real* u, const frk::Surf<Real>* surf, int nsurf, int most, const frk::Phys<Real>& ph,
+           void* stream);
 
 template <typename Real, int DIM>
 int integrals(int P, const Real* u, int64_t e_first, int64_t ne, const frk::Ops<Real>& op,

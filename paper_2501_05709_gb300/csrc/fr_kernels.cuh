@@ -2184,23 +2184,22 @@ static __global__ void k_forces_fin(const double* __restrict__ part, int nblk, d
 // FW-H data-surface sampling (Section 3.1): one warp per surface point
 // evaluates the element's tensor Lagrange interpolant (1D weights pw
 // [npts][DIM][NP] precomputed at the located reference coordinates) and
-// stores (rho, V_1, V_2, V_3, p) minus the free stream into record *count.
-// counter[0] = records written, counter[1] = steps seen, counter[2] = overflow;
-// the kernel samples only on steps that are multiples of `every`.
+// stores (rho, V_1, V_2, V_3, p) minus the free stream into record count[0]
+// of its surface (grid y: all surfaces in one launch; 12 of them took 24 launches
+// of 2 to 5 us a step).  It samples only on steps that are multiples of `every`.
 template <int DIM, int P, typename Real>
-__global__ void k_sample(const Real* __restrict__ u, const int64_t* __restrict__ pe,
-                         const Real* __restrict__ pw, int npts, Phys<Real> ph, Real* __restrict__ hist,
-                         const int* __restrict__ count, int cap, int every) {
+__global__ void k_sample(const Real* __restrict__ u, const Surf<Real>* __restrict__ surf, Phys<Real> ph) {
+    const Surf<Real> sf = surf[blockIdx.y];
     using Z = Sz<DIM, P>;
     constexpr int NP = Z::NP, NSP = Z::NSP, NV = Z::NV;
     const int lane = threadIdx.x & 31;
     const int k = int((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5);
-    if (k >= npts) return;
-    if (count[1] % every != 0) return;
-    const int rec = count[0];
-    if (rec >= cap) return;
-    const Real* ue = u + pe[k] * NV * NSP;
-    const Real* wk = pw + int64_t(k) * DIM * NP;
+    if (k >= sf.npts) return;
+    if (sf.count[1] % sf.every != 0) return;
+    const int rec = sf.count[0];
+    if (rec >= sf.cap) return;
+    const Real* ue = u + sf.pe[k] * NV * NSP;
+    const Real* wk = sf.pw + int64_t(k) * DIM * NP;
     Real acc[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) acc[v] = Real(0);
@@ -2218,7 +2217,7 @@ __global__ void k_sample(const Real* __restrict__ u, const int64_t* __restrict__
     if (lane == 0) {
         const Real rho = acc[0];
         const Real p = pressure<DIM>(acc, ph.gm1);
-        Real* dst = hist + (int64_t(rec) * npts + k) * 5;
+        Real* dst = sf.hist + (int64_t(rec) * sf.npts + k) * 5;
         dst[0] = rho - ph.rho_inf;
 #pragma unroll
         for (int i = 0; i < 3; ++i) dst[1 + i] = (i < DIM) ? acc[1 + i] / rho - ph.vel_inf[i] : Real(0);
@@ -2227,14 +2226,16 @@ __global__ void k_sample(const Real* __restrict__ u, const int64_t* __restrict__
 }
 
 // advances the counters after the sampling kernel of the same step
-static __global__ void k_bump(int* count, int cap, int every) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        if (count[1] % every == 0) {
-            if (count[0] < cap) count[0] += 1;
-            else count[2] = 1;
-        }
-        count[1] += 1;
+template <typename Real>
+__global__ void k_bump(const Surf<Real>* __restrict__ surf, int n) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    int* count = surf[i].count;
+    if (count[1] % surf[i].every == 0) {
+        if (count[0] < surf[i].cap) count[0] += 1;
+        else count[2] = 1;
     }
+    count[1] += 1;
 }
 
 // Volume integrals (double) of the conserved variables and of the kinetic
