@@ -15,6 +15,7 @@
 #include "fr.h"
 #include "fr_common.h"
 #include "fr_geom.h"
+#include "fr_pool.h"
 
 static thread_local std::string g_err;
 
@@ -827,6 +828,7 @@ extern "C" int fr_mesh_load(const fr_mesh_desc* m, int ncand, const fr_options* 
     if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev < 1)
         return fail(FR_ECUDA, "no CUDA device available (libfr has no CPU path)");
 
+    fr_pool_trim();   // the context may need what per-call scratch holds
     fr_ctx* c = new fr_ctx();
     cudaGetDevice(&c->device);
     c->dim = dim;
@@ -1181,6 +1183,7 @@ extern "C" int fr_destroy(fr_ctx* c) {
     if (!c) return FR_OK;
     cudaDeviceSynchronize();
     release(c);
+    fr_pool_trim();
     return FR_OK;
 }
 

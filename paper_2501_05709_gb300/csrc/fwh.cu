@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "fr.h"
+#include "fr_pool.h"
 
 namespace {
 
@@ -741,8 +742,18 @@ extern "C" int fwh_integrate(const double* hist, int nt, int npts, const double*
     int rc = fwh_check(hist, nt, npts, y, n, dS, dtau, obs, nobs, Minf, c0, ncopies, p_out, cap, nt_out, t0_out);
     if (rc != FR_OK) return rc;
     FwhScratch sc;
+    // scratch from the pool, or (no pool) by cudaMalloc
+    auto get = [s](void** p, size_t bytes, bool* pooled) {
+        *pooled = fr_pool_alloc(p, bytes, s);
+        return *pooled || cudaMalloc(p, bytes) == cudaSuccess;
+    };
+    auto put = [s](void* p, bool pooled) {
+        if (pooled) fr_pool_free(p, s);
+        else cudaFree(p);
+    };
     void *tab = nullptr, *buf = nullptr;
-    if (cudaMalloc(&tab, OBS_BYTES) != cudaSuccess)
+    bool tab_pooled = false, buf_pooled = false;
+    if (!get(&tab, OBS_BYTES, &tab_pooled))
         return fr_set_error_from_fwh(FR_ENOMEM, "cannot allocate FW-H scratch");
     sc.obs = static_cast<FwhObs*>(tab);
     sc.ext = reinterpret_cast<unsigned long long*>(sc.obs + OBS_MAX);
@@ -757,17 +768,17 @@ extern "C" int fwh_integrate(const double* hist, int nt, int npts, const double*
         const size_t rows = size_t(sc.nbatch) * pl.Tmax * nobs;
         sc.npartial = std::min(rows, std::max(fwh_partial_doubles(pl), size_t(8) << 20));
         const size_t nx = fwh_series_doubles(sc.nbatch, nt);
-        if (cudaMalloc(&buf, sizeof(double) * (nx + sc.npartial) + 32 * size_t(sc.nbatch)) != cudaSuccess) {
-            cudaFree(tab);
+        if (!get(&buf, sizeof(double) * (nx + sc.npartial) + 32 * size_t(sc.nbatch), &buf_pooled)) {
+            put(tab, tab_pooled);
             return fr_set_error_from_fwh(FR_ENOMEM, "cannot allocate FW-H scratch");
         }
         sc.X = static_cast<double*>(buf);
         sc.hw = reinterpret_cast<int*>(sc.X + nx);
         sc.partial = sc.X + nx + 4 * size_t(sc.nbatch);
         rc = fwh_run(pl, hist, nt, npts, y, n, dS, obs, nobs, Lspan, ncopies, p_out, cap, nt_out, t0_out, sc, s);
-        cudaFree(buf);
+        put(buf, buf_pooled);
     }
-    cudaFree(tab);
+    put(tab, tab_pooled);
     return rc;
 }
 

@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "fr.h"
+#include "fr_pool.h"
 
 int fr_set_error_from_fwh(int code, const char* msg);
 
@@ -137,15 +138,19 @@ extern "C" int fwh_psd(const double* p, int nobs, int nt, int ld, double dt, int
     }
     const double inv_norm = dt / w2;   // 1 / (f_s sum w^2)
     // one allocation: the table, then the folded segments
-    double2* cs = nullptr;
-    if (cudaMalloc(&cs, sizeof(double2) * size_t(L) + sizeof(double) * size_t(nobs) * nseg * (L + 2)) != cudaSuccess)
+    const size_t bytes = sizeof(double2) * size_t(L) + sizeof(double) * size_t(nobs) * nseg * (L + 2);
+    void* buf = nullptr;
+    const bool pooled = fr_pool_alloc(&buf, bytes, s);
+    if (!pooled && cudaMalloc(&buf, bytes) != cudaSuccess)
         return fr_set_error_from_fwh(FR_ENOMEM, "cannot allocate PSD scratch");
+    double2* cs = static_cast<double2*>(buf);
     double* ws = reinterpret_cast<double*>(cs + L);
     k_psd_segments<<<dim3(nseg + 1, nobs), 256, 0, s>>>(p, ld, L, cs, ws);
     k_psd_dft<<<dim3((L / 4 + PSD_WARPS) / PSD_WARPS, nobs), 32 * PSD_WARPS, 0, s>>>(ws, nseg, L, cs, inv_norm, psd, cap);
     cudaError_t err = cudaGetLastError();
     if (err == cudaSuccess) err = cudaStreamSynchronize(s);
-    cudaFree(cs);
+    if (pooled) fr_pool_free(buf, s);
+    else cudaFree(buf);
     if (err != cudaSuccess) return fr_set_error_from_fwh(FR_ECUDA, cudaGetErrorString(err));
     *nfreq_out = nf;
     return FR_OK;
