@@ -446,9 +446,8 @@ __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(
 // Per-element (per-warp) shared-memory footprint of each kernel, in Reals.
 // Regions (Reals) of one warp's shared memory.  F = NF*NV*NFP is one
 // element's face data, U = NV*NSP its state.
-//   visc : A su[U] | B sj[F] | C sl[F] | D sg[max(DIM*U, F)]  (D holds the
-//          staged neighbour traces during the face phase; affine meshes need
-//          no gradient volume, so there D is [F] only)
+//   visc : A su[U] | D sg[DIM*U] | S, 1/|J| [G] (curved meshes; affine ones run
+//          the pipelined kernel on two buffers per element group)
 //   resid: A su[U] | B sj[max(U,F)] (staged own traces until each entry is
 //          replaced by the jump of the same face point; sd after the gradient)
 //          | C sc[F] (staged own viscous fluxes until each entry is replaced by
@@ -462,15 +461,11 @@ struct Smem {
     static constexpr int F = Z::NF * Z::NV * Z::NFP;
     static constexpr int imax(int a, int b) { return a > b ? a : b; }
     static constexpr int traces = U;
-    static constexpr int vB = U, vC = vB + F, vD = vC + F;
-    static constexpr int visc = vD + imax(DIM * U, F);
-    static constexpr int visc_a = vD + F;   // affine: no gradient volume, region D holds the neighbour traces
     static constexpr int rB = U, rC = rB + imax(U, F), rD = rC + F, rE = rD + imax(DIM * U, 2 * F);
     static constexpr int resid = rE;
-    // curved meshes also stage the element's S [DIM*DIM][NSP] and 1/|J| [NSP]:
-    // in an extra region after visc's and in resid's region E
+    // curved meshes also stage the element's S [DIM*DIM][NSP] and 1/|J| [NSP]
     static constexpr int G = DIM * DIM * Z::NSP + Z::NSP;
-    static constexpr int visc_c = visc + G;
+    static constexpr int vD = U, vS = vD + DIM * U, visc_c = vS + G;
     static constexpr int resid_c = rE + G;
     // pipelined face kernel on affine meshes: two buffers per element group,
     // each [state U | own traces F | neighbour traces F | S, 1/|J|, normals]
@@ -1146,13 +1141,15 @@ __global__ void k_visc_face_aff(
     }
 }
 
-// Sweep B: BR2 face gradients and the own-side viscous normal flux.  For a
-// boundary face the common viscous flux F_vis(u_b, G).N (energy entry zero at
-// an adiabatic wall) is written instead.  MP is the mesh's metric path, fixed
-// at compile time: 0 per-point metrics (curved), 1 one metric set per element
-// (affine), 2 affine with diagonal S (axis-aligned); BND false: the mesh has
-// no boundary faces (fully periodic), so the boundary-state code is left out.
-template <int DIM, int P, typename Real, int MP, bool BND>
+// Sweep B on curved meshes: BR2 face gradients and the own-side viscous normal
+// flux.  For a boundary face the common viscous flux F_vis(u_b, G).N (energy entry
+// zero at an adiabatic wall) is written instead.  The state and the metrics are
+// staged in shared memory; the traces of both sides of a lane's face points go
+// straight to registers, where the jump and the flux of that point need them.
+// Bound by the L1 / shared-memory pipe: with both sides' traces staged and the jumps
+// kept in shared memory 227 us on 100,000 elements at p = 3 in FP32 and 144 us on
+// 20,000 at p = 4; now 214 and 127 (with 96 registers 219, with 112: 257 at p = 3).
+template <int DIM, int P, typename Real>
 __global__ void __maxnreg__(sizeof(Real) == 4 ? 80 : 168) k_visc_face(const Real* __restrict__ u, const Real* __restrict__ uf, Real* __restrict__ fvn,
                             int64_t E, const __grid_constant__ Ops<Real> op, const __grid_constant__ Phys<Real> ph,
                             const __grid_constant__ Geo<Real> g) {
@@ -1169,14 +1166,9 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? 80 : 168) k_visc_face(const Real
     if (e >= E || (g.order && g.order[e] < P)) return;   // reduced: k_red_*
     using SM = Smem<DIM, P>;
     using VL = Vol<DIM, P, Real>;
-    constexpr bool curved = MP == 0;                // per-point metrics, staged after region D
-    constexpr bool diag = MP == 2;                  // affine, diagonal S
-    Real* su = reinterpret_cast<Real*>(smem) + warp * (curved ? SM::visc_c : SM::visc_a);
-    Real* sj = su + SM::vB;              // jumps u_c - u_f   [f][v][fp]
-    Real* sl = su + SM::vC;              // own traces u_f    [f][v][fp]
+    Real* su = reinterpret_cast<Real*>(smem) + warp * SM::visc_c;
     Real* sg = su + SM::vD;              // gradient          [d or i][v][sp]
-    Real* sn = sg;                       // staged neighbour traces [f][v][fp] (face phase only)
-    Real* sS = su + SM::visc;            // curved: S [k][sp], 1/|J| [sp]
+    Real* sS = su + SM::vS;              // S [k][sp], 1/|J| [sp]
     // face codes of this element, broadcast to every lane
     int codes[NF];
     {
@@ -1184,115 +1176,89 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? 80 : 168) k_visc_face(const Real
 #pragma unroll
         for (int f = 0; f < NF; ++f) codes[f] = __shfl_sync(0xffffffffu, mine, f);
     }
-    // stage the element state, its own and its neighbours' face traces (the
-    // traces array holds them for every element) and (curved) the metrics, in
-    // three groups
-    constexpr bool VW = (SM::visc * sizeof(Real)) % 16 == 0 && (SM::visc_c * sizeof(Real)) % 16 == 0 &&
-                        (SM::visc_a * sizeof(Real)) % 16 == 0;
-    constexpr bool VS = VW && (NV * NFP * sizeof(Real)) % 16 == 0 && (SM::vD * sizeof(Real)) % 16 == 0 &&
-                        (SM::vC * sizeof(Real)) % 16 == 0;
+    constexpr bool VW = (SM::visc_c * sizeof(Real)) % 16 == 0;
     warp_stage_vol<DIM, P>(su, u + e * NV * NSP, lane, T);
     cp_async_commit();
-    warp_stage<NF * NV * NFP, VS>(sl, uf + e * NF * NV * NFP, lane, T);
-#pragma unroll
-    for (int f = 0; f < NF; ++f)
-        if (!BND || codes[f] >= 0)
-            warp_stage<NV * NFP, VS>(sn + f * NV * NFP, uf + int64_t(codes[f] >> 3) * NV * NFP, lane, T);
+    warp_stage_auto<DIM * DIM * NSP, VW && (SM::vS * sizeof(Real)) % 16 == 0>(sS, g.S + e * g.sS_e, lane, T);
+    warp_stage_auto<NSP, VW && ((SM::vS + DIM * DIM * NSP) * sizeof(Real)) % 16 == 0>(sS + DIM * DIM * NSP,
+                                                                                     g.iJ + e * g.sJ_e, lane, T);
     cp_async_commit();
-    if (curved) {
-        warp_stage_auto<DIM * DIM * NSP, VW>(sS, g.S + e * g.sS_e, lane, T);
-        warp_stage_auto<NSP, VW && ((SM::visc + DIM * DIM * NSP) * sizeof(Real)) % 16 == 0>(
-            sS + DIM * DIM * NSP, g.iJ + e * g.sJ_e, lane, T);
-    }
-    cp_async_commit();
-    cp_async_wait<1>();
-    grp_sync<T>(warp);
-    {
-    // B: jumps per face point
+    // own and neighbour traces of this lane's face points
+    Real tL[DIM][NFI][NV], tR[DIM][NFI][NV];
 #pragma unroll
-    for (int d = 0; d < DIM; ++d) {
+    for (int d = 0; d < DIM; ++d)
 #pragma unroll
         for (int it = 0; it < NFI; ++it) {
             int side, fp;
             if (!face_pt<DIM, P>(lane, it, side, fp)) continue;
-            const int f = 2 * d + side;
-            Real uL[NV], uc[NV];
-#pragma unroll
-            for (int v = 0; v < NV; ++v) uL[v] = sl[(f * NV + v) * NFP + fp];
             const int code = side ? codes[2 * d + 1] : codes[2 * d];  // static register indices
-            if (!BND || code >= 0) {
-                const Real* un = sn + f * NV * NFP;
-                const int fpn = omap<DIM, NP>(code & 7, fp);
+            const Real* own = uf + (e * NF + 2 * d + side) * NL + fp;
 #pragma unroll
-                for (int v = 0; v < NV; ++v) uc[v] = Real(0.5) * (uL[v] + un[v * NFP + fpn]);
-            } else {
-                Real N[DIM], ug[NV];
-                load_normal<DIM>(g, e, f, fp, N);
-                bc_state<DIM>(-code, uL, N, ph, ug, uc);
+            for (int v = 0; v < NV; ++v) tL[d][it][v] = own[v * NFP];
+            if (code >= 0) {
+                const Real* un = uf + int64_t(code >> 3) * NL + omap<DIM, NP>(code & 7, fp);
+#pragma unroll
+                for (int v = 0; v < NV; ++v) tR[d][it][v] = un[v * NFP];
             }
+        }
+    cp_async_wait<1>();
+    grp_sync<T>(warp);
+    // C1: uncorrected reference gradient along lines: q_d = D_d u
 #pragma unroll
-            for (int v = 0; v < NV; ++v) sj[(f * NV + v) * NFP + fp] = uc[v] - uL[v];
+    for (int d = 0; d < DIM; ++d) {
+#pragma unroll
+        for (int it = 0; it < NLI; ++it) {
+            const LineTask<DIM, P> tk(lane, it);
+            if (NL % T != 0 && tk.t >= NL) break;
+            Real s[NP], q[NP];
+            vload_line<DIM, P>(su + tk.shift, tk.vref, d, tk.ln, s);
+#pragma unroll
+            for (int i = 0; i < NP; ++i) q[i] = Real(0);
+            apply_D<NP>(op, s, q);
+            vstore_line<DIM, P>(sg + tk.shift, d * NV + tk.vref, d, tk.ln, q);
         }
     }
-    grp_sync<T>(warp);  // the gradient below overwrites the staged neighbour traces
-    {
-        // C1: uncorrected reference gradient along lines: q_d = D_d u
+    cp_async_wait<0>();
+    grp_sync<T>(warp);
+    // C2: physical gradient (1/|J|) S^T q at each solution point, in place
 #pragma unroll
-        for (int d = 0; d < DIM; ++d) {
+    for (int s = 0; s < NSPW; ++s) {
+        const int sp = lane + T * s;
+        if (NSP % T != 0 && sp >= NSP) break;
+        Real q[DIM][NV];
 #pragma unroll
-            for (int it = 0; it < NLI; ++it) {
-                const LineTask<DIM, P> tk(lane, it);
-                if (NL % T != 0 && tk.t >= NL) break;
-                Real s[NP], q[NP];
-                vload_line<DIM, P>(su + tk.shift, tk.vref, d, tk.ln, s);
+        for (int d = 0; d < DIM; ++d)
 #pragma unroll
-                for (int i = 0; i < NP; ++i) q[i] = Real(0);
-                apply_D<NP>(op, s, q);
-                vstore_line<DIM, P>(sg + tk.shift, d * NV + tk.vref, d, tk.ln, q);
-            }
-        }
-        cp_async_wait<0>();
-        grp_sync<T>(warp);
-        // C2: physical gradient (1/|J|) S^T q at each solution point, in place
+            for (int v = 0; v < NV; ++v) q[d][v] = sg[VL::pt(d * NV + v, sp)];
+        Real S[DIM * DIM];
 #pragma unroll
-        for (int s = 0; s < NSPW; ++s) {
-            const int sp = lane + T * s;
-            if (NSP % T != 0 && sp >= NSP) break;
-            Real q[DIM][NV];
-#pragma unroll
-            for (int d = 0; d < DIM; ++d)
-#pragma unroll
-                for (int v = 0; v < NV; ++v) q[d][v] = sg[VL::pt(d * NV + v, sp)];
-            Real S[DIM * DIM];
-#pragma unroll
-            for (int k = 0; k < DIM * DIM; ++k) S[k] = sS[k * NSP + sp];
-            const Real iJ = sS[DIM * DIM * NSP + sp];
-            if constexpr (sizeof(Real) == 4) {
-                // pairs of variables as packed FP32x2 (the same order of operations)
-#pragma unroll
-                for (int i = 0; i < DIM; ++i)
-#pragma unroll
-                    for (int v = 0; v + 1 < NV; v += 2) {
-                        float2 a = make_float2(0.0f, 0.0f);
-#pragma unroll
-                        for (int d = 0; d < DIM; ++d)
-                            a = __ffma2_rn(make_float2(S[d * DIM + i], S[d * DIM + i]),
-                                           make_float2(q[d][v], q[d][v + 1]), a);
-                        a = __fmul2_rn(a, make_float2(iJ, iJ));
-                        sg[VL::pt(i * NV + v, sp)] = a.x;
-                        sg[VL::pt(i * NV + v + 1, sp)] = a.y;
-                    }
-            }
+        for (int k = 0; k < DIM * DIM; ++k) S[k] = sS[k * NSP + sp];
+        const Real iJ = sS[DIM * DIM * NSP + sp];
+        if constexpr (sizeof(Real) == 4) {
+            // pairs of variables as packed FP32x2 (the same order of operations)
 #pragma unroll
             for (int i = 0; i < DIM; ++i)
 #pragma unroll
-                for (int v = sizeof(Real) == 4 ? NV - NV % 2 : 0; v < NV; ++v) {
-                    Real acc = Real(0);
+                for (int v = 0; v + 1 < NV; v += 2) {
+                    float2 a = make_float2(0.0f, 0.0f);
 #pragma unroll
-                    for (int d = 0; d < DIM; ++d) acc += S[d * DIM + i] * q[d][v];
-                    sg[VL::pt(i * NV + v, sp)] = acc * iJ;
+                    for (int d = 0; d < DIM; ++d)
+                        a = __ffma2_rn(make_float2(S[d * DIM + i], S[d * DIM + i]),
+                                       make_float2(q[d][v], q[d][v + 1]), a);
+                    a = __fmul2_rn(a, make_float2(iJ, iJ));
+                    sg[VL::pt(i * NV + v, sp)] = a.x;
+                    sg[VL::pt(i * NV + v + 1, sp)] = a.y;
                 }
         }
+#pragma unroll
+        for (int i = 0; i < DIM; ++i)
+#pragma unroll
+            for (int v = sizeof(Real) == 4 ? NV - NV % 2 : 0; v < NV; ++v) {
+                Real acc = Real(0);
+#pragma unroll
+                for (int d = 0; d < DIM; ++d) acc += S[d * DIM + i] * q[d][v];
+                sg[VL::pt(i * NV + v, sp)] = acc * iJ;
+            }
     }
     // normals of this lane's face points, all directions at once
     Real Nr[DIM][NFI][DIM];
@@ -1335,30 +1301,34 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? 80 : 168) k_visc_face(const Real
             Real tr[DIM * NV];   // traces of the physical gradient [i][v]
             traces_at<DIM, P, DIM * NV>(sg, d, fp, cf, tr);
             Real G[NV][DIM];
-            Real uL[NV];
+            const Real* N = Nr[d][it];
+            const int code = side ? codes[2 * d + 1] : codes[2 * d];  // static register indices
+            const Real* uL = tL[d][it];
+            Real uc[NV];   // common solution
+            if (code >= 0) {
+#pragma unroll
+                for (int v = 0; v < NV; ++v) uc[v] = Real(0.5) * (uL[v] + tR[d][it][v]);
+            } else {
+                Real ug[NV];
+                bc_state<DIM>(-code, uL, N, ph, ug, uc);
+            }
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
-                const Real jv = sj[(f * NV + v) * NFP + fp];
-                uL[v] = sl[(f * NV + v) * NFP + fp];
+                const Real jv = uc[v] - uL[v];
 #pragma unroll
                 for (int i = 0; i < DIM; ++i) G[v][i] = tr[i * NV + v] + ph.eta * lc[i] * jv;
             }
-            const Real* N = Nr[d][it];
-            const int code = side ? codes[2 * d + 1] : codes[2 * d];  // static register indices
             Real Fn[NV];
-            if (!BND || code >= 0) {
+            if (code >= 0) {
                 visc_flux_n<DIM>(uL, G, ph.mu, ph.kappa, N, Fn);
             } else {
-                Real ug[NV], ub[NV];
-                bc_state<DIM>(-code, uL, N, ph, ug, ub);
-                visc_flux_n<DIM>(ub, G, ph.mu, ph.kappa, N, Fn);
+                visc_flux_n<DIM>(uc, G, ph.mu, ph.kappa, N, Fn);
                 if (code == -FR_BC_WALL) Fn[NV - 1] = Real(0);
             }
             Real* dst = fvn + (e * NF + f) * NV * NFP + fp;
 #pragma unroll
             for (int v = 0; v < NV; ++v) dst[v * NFP] = Fn[v];
         }
-    }
     }
 }
 

@@ -97,7 +97,7 @@ template <int P, int MP, bool BND>
 int visc_p(const FR_REAL* u, const FR_REAL* uf, FR_REAL* fvn, int64_t E, const frk::Ops<FR_REAL>& op,
            const frk::Phys<FR_REAL>& ph, const frk::Geo<FR_REAL>& g, frk::Launch lc, cudaStream_t s) {
     if constexpr (MP == 0) {
-        auto k = frk::k_visc_face<FR_DIM, P, FR_REAL, MP, BND>;
+        auto k = frk::k_visc_face<FR_DIM, P, FR_REAL>;
         const auto smem = [](int n) { return frk::smem_visc<FR_DIM, P, FR_REAL>(n, true); };
         const size_t sm = smem(std::max(lc.epb, 1));
         static unsigned long long done = 0;
