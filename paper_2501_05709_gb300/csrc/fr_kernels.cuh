@@ -460,17 +460,24 @@ struct Smem {
     static constexpr int U = Z::NV * Z::NSP;
     static constexpr int F = Z::NF * Z::NV * Z::NFP;
     static constexpr int imax(int a, int b) { return a > b ? a : b; }
-    static constexpr int traces = U;
-    static constexpr int rB = U, rC = rB + imax(U, F), rD = rC + F, rE = rD + imax(DIM * U, 2 * F);
+    static constexpr int al(int n) { return (n + 3) / 4 * 4; }   // regions start 16-byte aligned
+    static constexpr bool SHIFT = U % 4 != 0;                     // states start at any multiple of sizeof(Real)
+    static constexpr int UA = SHIFT ? al(U + 3) : U;              // a staged state, with its shift
+    static constexpr int traces = UA;
+    // a face's data are a multiple of 16 bytes in either precision (k_residual then
+    // stages them, see there)
+    static constexpr bool rows16 = (Z::NV * Z::NFP) % 2 == 0;
+    static constexpr int rB = UA, rC = rB + al(imax(U, F)), rD = rC + al(F);
+    static constexpr int rE = rD + al(rows16 ? imax(DIM * U, 2 * F) : DIM * U);
     static constexpr int resid = rE;
     // curved meshes also stage the element's S [DIM*DIM][NSP] and 1/|J| [NSP]
     static constexpr int G = DIM * DIM * Z::NSP + Z::NSP;
-    static constexpr int vD = U, vS = vD + DIM * U, visc_c = vS + G;
-    static constexpr int resid_c = rE + G;
+    static constexpr int vD = UA, vS = vD + al(DIM * U), visc_c = vS + al(G);
+    static constexpr int resid_c = rE + al(G);
     // pipelined face kernel on affine meshes: two buffers per element group,
     // each [state U | own traces F | neighbour traces F | S, 1/|J|, normals]
     static constexpr int GEO = (DIM * DIM + 1 + 2 * DIM * DIM + 3) / 4 * 4;
-    static constexpr int pl = U, pn = U + F, pg = U + 2 * F;
+    static constexpr int pl = UA, pn = pl + al(F + 3), pg = pn + al(F);
     static constexpr int visc_buf = (pg + GEO + 3) / 4 * 4;
     static constexpr int visc_p = 2 * visc_buf;
 };
@@ -806,10 +813,30 @@ __device__ __forceinline__ void warp_stage_auto(Real* s, const Real* g, int lane
         warp_stage<N, false>(s, g, lane, T);
 }
 
-// stage one element's state [NV][NSP] (canonical global layout) into the
-// volume placement; rows go as 16-byte copies when the global rows are aligned
+// N contiguous Reals g -> s in 16-byte copies whatever the alignment of g: the copy
+// starts as far from a 16-byte boundary of s as g does from its own (s is aligned
+// and has room for 16 / sizeof(Real) - 1 more), so only the ends go one by one.
+// At p = 2 and 4 an element's rows are not multiples of 16 bytes and went one by
+// one altogether (Smem::SHIFT).  Returns where the copy starts: s + stage_shift(g).
+template <typename Real>
+__device__ __forceinline__ int stage_shift(const Real* g) {
+    return int((reinterpret_cast<uintptr_t>(g) & 15u) / sizeof(Real));
+}
+template <int N, typename Real>
+__device__ __forceinline__ Real* warp_stage_shift(Real* s, const Real* g, int lane, int T) {
+    constexpr int RPC = int(16 / sizeof(Real));
+    const int mis = stage_shift(g), head = (RPC - mis) & (RPC - 1), nch = (N - head) / RPC, tail = head + nch * RPC;
+    Real* d = s + mis;
+    for (int c = lane; c < nch; c += T) cp_async16(d + head + c * RPC, g + head + c * RPC);
+    if (lane < head) cp_async_small<int(sizeof(Real))>(d + lane, g + lane);
+    if (lane < N - tail) cp_async_small<int(sizeof(Real))>(d + tail + lane, g + tail + lane);
+    return d;
+}
+
+// stage one element's state [NV][NSP] (canonical global layout) into the volume
+// placement at s (16-byte aligned); returns where it starts
 template <int DIM, int P, typename Real>
-__device__ __forceinline__ void warp_stage_vol(Real* s, const Real* g, int lane, int T = 32) {
+__device__ __forceinline__ Real* warp_stage_vol(Real* s, const Real* g, int lane, int T = 32) {
     using V = Vol<DIM, P, Real>;
     constexpr int NV = DIM + 2, NP = P + 1, NSP = V::NSP;
     if constexpr (V::ROW4) {
@@ -819,11 +846,24 @@ __device__ __forceinline__ void warp_stage_vol(Real* s, const Real* g, int lane,
                 const int v = k / (NSP / NP), r = k % (NSP / NP);
                 cp_async16(s + V::at(v, 0, r % NP, r / NP), g + k * NP);
             }
-            return;
+            return s;
         }
     }
-    for (int k = lane; k < NV * NSP; k += T)
-        cp_async_small<int(sizeof(Real))>(s + V::pt(k / NSP, k % NSP), g + k);
+    if constexpr (Smem<DIM, P>::SHIFT) {
+        return warp_stage_shift<NV * NSP>(s, g, lane, T);
+    } else if constexpr (!V::SWZ && !V::ROW4) {
+        warp_stage_auto<NV * NSP, true>(s, g, lane, T);
+        return s;
+    } else {
+        for (int k = lane; k < NV * NSP; k += T)
+            cp_async_small<int(sizeof(Real))>(s + V::pt(k / NSP, k % NSP), g + k);
+        return s;
+    }
+}
+// the same of an element that was staged before
+template <int DIM, int P, typename Real>
+__device__ __forceinline__ Real* staged_vol(Real* s, const Real* g) {
+    return Smem<DIM, P>::SHIFT ? s + stage_shift(g) : s;
 }
 
 // trace on face (d, side) at face point fp of variable v of volume array X:
@@ -907,7 +947,7 @@ __global__ void k_traces(const Real* __restrict__ u, Real* __restrict__ uf, int6
     const int64_t e = int64_t(blockIdx.x) * (blockDim.x / T) + warp;
     if (e >= E) return;
     Real* su = reinterpret_cast<Real*>(smem) + warp * Smem<DIM, P>::traces;
-    warp_stage_vol<DIM, P>(su, u + e * NV * NSP, lane, T);
+    su = warp_stage_vol<DIM, P>(su, u + e * NV * NSP, lane, T);
     cp_async_commit();
     cp_async_wait<0>();
     grp_sync<T>(warp);
@@ -1099,7 +1139,8 @@ __global__ void k_visc_face_aff(
         for (int f = 0; f < NF; ++f) codes[f] = __shfl_sync(0xffffffffu, mine, f);
         if (g.order && g.order[el] < P) return;   // a reduced-degree element (k_red_face)
         warp_stage_vol<DIM, P>(b, u + el * NV * NSP, lane, T);
-        warp_stage<NF * NV * NFP, VS>(b + SM::pl, uf + el * NF * NV * NFP, lane, T);
+        if constexpr (VS) warp_stage<NF * NV * NFP, VS>(b + SM::pl, uf + el * NF * NV * NFP, lane, T);
+        else warp_stage_shift<NF * NV * NFP>(b + SM::pl, uf + el * NF * NV * NFP, lane, T);
 #pragma unroll
         for (int f = 0; f < NF; ++f)
             if (!BND || codes[f] >= 0)
@@ -1129,8 +1170,10 @@ __global__ void k_visc_face_aff(
 #pragma unroll
         for (int f = 0; f < NF; ++f) codes[f] = __shfl_sync(0xffffffffu, mineA, f);
         if (!g.order || g.order[e] >= P)
-            visc_faces_affine<DIM, P, Real, MP == 2, BND, VS>(cur, cur + SM::pl, cur + SM::pn, cur + SM::pg, codes,
-                                                              e, fvn, op, ph, lane);
+            visc_faces_affine<DIM, P, Real, MP == 2, BND, VS>(
+                staged_vol<DIM, P>(cur, u + e * NV * NSP),
+                cur + SM::pl + (VS ? 0 : stage_shift(uf + e * NF * NV * NFP)), cur + SM::pn, cur + SM::pg, codes, e,
+                fvn, op, ph, lane);
         if (en >= E) break;
         grp_sync<T>(grp);   // every thread is done with cur before it is refilled
         e = en;
@@ -1168,7 +1211,7 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? 80 : 168) k_visc_face(const Real
     using VL = Vol<DIM, P, Real>;
     Real* su = reinterpret_cast<Real*>(smem) + warp * SM::visc_c;
     Real* sg = su + SM::vD;              // gradient          [d or i][v][sp]
-    Real* sS = su + SM::vS;              // S [k][sp], 1/|J| [sp]
+    Real* const sS = su + SM::vS;              // S [k][sp], 1/|J| [sp]
     // face codes of this element, broadcast to every lane
     int codes[NF];
     {
@@ -1177,7 +1220,7 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? 80 : 168) k_visc_face(const Real
         for (int f = 0; f < NF; ++f) codes[f] = __shfl_sync(0xffffffffu, mine, f);
     }
     constexpr bool VW = (SM::visc_c * sizeof(Real)) % 16 == 0;
-    warp_stage_vol<DIM, P>(su, u + e * NV * NSP, lane, T);
+    su = warp_stage_vol<DIM, P>(su, u + e * NV * NSP, lane, T);
     cp_async_commit();
     warp_stage_auto<DIM * DIM * NSP, VW && (SM::vS * sizeof(Real)) % 16 == 0>(sS, g.S + e * g.sS_e, lane, T);
     warp_stage_auto<NSP, VW && ((SM::vS + DIM * DIM * NSP) * sizeof(Real)) % 16 == 0>(sS + DIM * DIM * NSP,
@@ -1338,12 +1381,13 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? 80 : 168) k_visc_face(const Real
 // BND as for k_visc_face; VISC: Navier-Stokes (BR2 viscous terms) or Euler;
 // OPM: the gradient and divergence line operators as FP32 FMAs (0) or on the
 // tensor cores with TF32 (1) or BF16x3 (2) operands (float only).  Register
-// caps in FP32: 88 for p = 4 in 3D and for curved meshes (p = 4 box 227 us, with
-// 72: 229, with 96: 238; 100,000 curved elements at p = 3: 314 us, with 72: 323,
-// with 96: 319), else 72 (Euler box of 50^3 at p = 2: 190 us, with 96: 196; of
-// 40^3 at p = 3: 131 against 137; Navier-Stokes the same); 168 in FP64.
+// caps in FP32: 72 on affine meshes (box at p = 4 195 us, with 88: 212; Euler box
+// of 50^3 at p = 2 175, with 80: 187; of 40^3 at p = 3 131, with 96: 137); on
+// curved ones 88 (100,000 elements at p = 3: 314 us, with 72: 323, with 96: 319), at
+// p = 4 96 (20,000 elements: 156, with 88: 167, with 72: 199), at p = 2 80 (49, with
+// 88 or 96: 52, with 72: 58); 168 in FP64.
 template <int DIM, int P, typename Real, int MP, bool VISC, bool BND, int OPM = 0>
-__global__ void __maxnreg__(sizeof(Real) == 4 ? (DIM == 3 && P == 4 || MP == 0 ? 88 : 72) : 168) k_residual(const Real* __restrict__ u, const Real* __restrict__ uf,
+__global__ void __maxnreg__(sizeof(Real) == 4 ? (MP != 0 ? 72 : DIM == 3 && P == 4 ? 96 : DIM == 3 && P == 2 ? 80 : 88) : 168) k_residual(const Real* __restrict__ u, const Real* __restrict__ uf,
                            const Real* __restrict__ fvn, int64_t E, const __grid_constant__ Ops<Real> op,
                            const __grid_constant__ Phys<Real> ph, const __grid_constant__ Geo<Real> g,
                            const __grid_constant__ Stage<Real> st) {
@@ -1363,8 +1407,8 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? (DIM == 3 && P == 4 || MP == 0 ?
     using VL = Vol<DIM, P, Real>;
     constexpr bool curved = MP == 0;                // per-point metrics, staged in region E
     constexpr bool diag = MP == 2;                  // affine, diagonal S
-    Real* su = reinterpret_cast<Real*>(smem) + warp * (curved ? SM::resid_c : SM::resid);
-    Real* sl = su + SM::rB;              // own traces            [f][v][fp]  (face phase)
+    Real* su = reinterpret_cast<Real*>(smem) + warp * (curved ? SM::resid_c : SM::resid);   // state (with its shift)
+    Real* sl = su + SM::rB;              // own traces            [f][v][fp]  (face phase, staged)
     Real* sj = sl;                       // jumps u_c - u_f      [f][v][fp]
     Real* sd = sj;                       // divergence [v][sp], after the gradient
     Real* sc = su + SM::rC;              // Fc.N - own viscous flux [f][v][fp]
@@ -1383,18 +1427,50 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? (DIM == 3 && P == 4 || MP == 0 ?
     constexpr bool VW = (SM::resid * sizeof(Real)) % 16 == 0 && (SM::resid_c * sizeof(Real)) % 16 == 0;
     constexpr bool VS = VW && (NV * NFP * sizeof(Real)) % 16 == 0 && (SM::rB * sizeof(Real)) % 16 == 0 &&
                         (SM::rC * sizeof(Real)) % 16 == 0 && (SM::rD * sizeof(Real)) % 16 == 0;
-    warp_stage_vol<DIM, P>(su, u + base, lane, T);
-    cp_async_commit();
-    warp_stage<NF * NV * NFP, VS>(sl, uf + e * NF * NV * NFP, lane, T);
+    // The face data (both sides' traces and viscous fluxes) are staged in 16-byte
+    // copies where their rows allow it (VS); else each lane loads those of its own
+    // face points to registers, one direction ahead.  Staged one by one they cost
+    // more than the staging saves (32^3 box at p = 4 227 us, in registers 199; Euler
+    // box of 50^3 at p = 2 190 against 175), in 16-byte copies less (p = 3: staged
+    // 92 us, in registers 103; 100,000 curved elements 314 against 363).
+    static_assert(VS == SM::rows16, "region D is laid out for the way the face data go");
+    Real xL[2][NFI][NV], xR[2][NFI][NV], xo[2][NFI][NV], xn[2][NFI][NV];
+    auto face_load = [&](int d, int b) {
 #pragma unroll
-    for (int f = 0; f < NF; ++f)
-        if (!BND || codes[f] >= 0) {
-            warp_stage<NV * NFP, VS>(sn + f * NV * NFP, uf + int64_t(codes[f] >> 3) * NV * NFP, lane, T);
-            if constexpr (VISC)
-                warp_stage<NV * NFP, VS>(sm + f * NV * NFP, fvn + int64_t(codes[f] >> 3) * NV * NFP, lane, T);
+        for (int it = 0; it < NFI; ++it) {
+            int side, fp;
+            if (!face_pt<DIM, P>(lane, it, side, fp)) continue;
+            const int code = side ? codes[2 * d + 1] : codes[2 * d];  // static register indices
+            const int64_t own = (e * NF + 2 * d + side) * NL + fp;
+            const bool nbr = !BND || code >= 0;
+            const int64_t nb = nbr ? int64_t(code >> 3) * NL + omap<DIM, NP>(code & 7, fp) : own;
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                xL[b][it][v] = uf[own + v * NFP];
+                xR[b][it][v] = uf[nb + v * NFP];
+                if constexpr (VISC) {
+                    xo[b][it][v] = fvn[own + v * NFP];
+                    xn[b][it][v] = fvn[nb + v * NFP];
+                }
+            }
         }
-    if constexpr (VISC) warp_stage<NF * NV * NFP, VS>(so, fvn + e * NF * NV * NFP, lane, T);
+    };
+    su = warp_stage_vol<DIM, P>(su, u + base, lane, T);
     cp_async_commit();
+    if constexpr (VS) {
+        warp_stage<NF * NV * NFP, VS>(sl, uf + e * NF * NV * NFP, lane, T);
+#pragma unroll
+        for (int f = 0; f < NF; ++f)
+            if (!BND || codes[f] >= 0) {
+                warp_stage<NV * NFP, VS>(sn + f * NV * NFP, uf + int64_t(codes[f] >> 3) * NV * NFP, lane, T);
+                if constexpr (VISC)
+                    warp_stage<NV * NFP, VS>(sm + f * NV * NFP, fvn + int64_t(codes[f] >> 3) * NV * NFP, lane, T);
+            }
+        if constexpr (VISC) warp_stage<NF * NV * NFP, VS>(so, fvn + e * NF * NV * NFP, lane, T);
+        cp_async_commit();
+    } else {
+        face_load(0, 0);
+    }
     // curved meshes: S and 1/|J|, needed after the gradient pass
     if constexpr (curved) {
         warp_stage_auto<DIM * DIM * NSP, VW && (SM::rE * sizeof(Real)) % 16 == 0>(sg, g.S + e * g.sS_e, lane, T);
@@ -1427,11 +1503,14 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? (DIM == 3 && P == 4 || MP == 0 ?
             }
         }
     }
-    cp_async_wait<curved ? 1 : 0>();
-    grp_sync<T>(warp);
+    if constexpr (VS) {
+        cp_async_wait<curved ? 1 : 0>();
+        grp_sync<T>(warp);
+    }
     // B: common normal flux (Rusanov minus common viscous) and jumps
 #pragma unroll
     for (int d = 0; d < DIM; ++d) {
+        if (!VS && d + 1 < DIM) face_load(d + 1, (d + 1) & 1);
 #pragma unroll
         for (int it = 0; it < NFI; ++it) {
             int side, fp;
@@ -1439,7 +1518,7 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? (DIM == 3 && P == 4 || MP == 0 ?
             const int f = 2 * d + side;
             Real uL[NV], uR[NV], uc[NV];
 #pragma unroll
-            for (int v = 0; v < NV; ++v) uL[v] = sl[(f * NV + v) * NFP + fp];
+            for (int v = 0; v < NV; ++v) uL[v] = VS ? sl[(f * NV + v) * NFP + fp] : xL[d & 1][it][v];
             const Real* N = Nr[d][it];
             const int code = side ? codes[2 * d + 1] : codes[2 * d];  // static register indices
             int fpn = 0;
@@ -1448,7 +1527,7 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? (DIM == 3 && P == 4 || MP == 0 ?
                 const Real* un = sn + f * NV * NFP;
 #pragma unroll
                 for (int v = 0; v < NV; ++v) {
-                    uR[v] = un[v * NFP + fpn];
+                    uR[v] = VS ? un[v * NFP + fpn] : xR[d & 1][it][v];
                     uc[v] = Real(0.5) * (uL[v] + uR[v]);
                 }
             } else {
@@ -1462,10 +1541,11 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? (DIM == 3 && P == 4 || MP == 0 ?
                 if (!BND || code >= 0) {
                     const Real* nb = sm + f * NV * NFP + fpn;
 #pragma unroll
-                    for (int v = 0; v < NV; ++v) Fc[v] -= Real(0.5) * (own[v * NFP] - nb[v * NFP]);
+                    for (int v = 0; v < NV; ++v)
+                        Fc[v] -= Real(0.5) * (VS ? own[v * NFP] - nb[v * NFP] : xo[d & 1][it][v] - xn[d & 1][it][v]);
                 } else {
 #pragma unroll
-                    for (int v = 0; v < NV; ++v) Fc[v] -= own[v * NFP];
+                    for (int v = 0; v < NV; ++v) Fc[v] -= VS ? own[v * NFP] : xo[d & 1][it][v];
                 }
             }
 #pragma unroll
@@ -1475,6 +1555,7 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? (DIM == 3 && P == 4 || MP == 0 ?
             }
         }
     }
+    if constexpr (!VS) cp_async_wait<curved ? 1 : 0>();
     grp_sync<T>(warp);
     // tensor-core mode: this thread's B fragment of the line operators, and
     // its place in the MMA tiles (warp wg of the element group, g, t)
@@ -1900,11 +1981,11 @@ __global__ void k_sponge(const __grid_constant__ Sponge<Real> sp, Real* __restri
     for (int i = 0; i < NP; ++i)
 #pragma unroll
         for (int k = 0; k < NP; ++k) pq[i][k] = sp.pm[q][i * MAXNP + k];
-    Real* sa = reinterpret_cast<Real*>(smem) + warp * 2 * NV * NSP;
-    Real* sb = sa + NV * NSP;
+    Real* sa = reinterpret_cast<Real*>(smem) + warp * 2 * Smem<DIM, P>::UA;
+    Real* sb = sa + Smem<DIM, P>::UA;
     const int narr = b ? 2 : 1;
-    warp_stage_vol<DIM, P>(sa, a + e * NV * NSP, lane);
-    if (b) warp_stage_vol<DIM, P>(sb, b + e * NV * NSP, lane);
+    sa = warp_stage_vol<DIM, P>(sa, a + e * NV * NSP, lane);
+    if (b) sb = warp_stage_vol<DIM, P>(sb, b + e * NV * NSP, lane);
     cp_async_commit();
     cp_async_wait<0>();
     __syncwarp();

@@ -63,6 +63,9 @@ template <typename K, typename S>
 int best_tile(K kernel, int T, S smem, int64_t E, int tie = 2) {
     int best = 1, most = blocks_per_sm(kernel, T, smem(1));
     if (E < 20 * int64_t(sm_count())) return 1;
+    // FP64 is bound by its pipe, not by latency: whole warps a block count (4,096
+    // affine elements at p = 3: 427 us a stage with 4, 432 with 2)
+    if (sizeof(FR_REAL) == 8 && smem(4) <= 113 * 1024 && blocks_per_sm(kernel, 4 * T, smem(4)) > 0) return 4;
     for (int epb : {8, 6, 1, 4, 3, 2, tie}) {   // of equal ones the last
         const int n = smem(epb) <= 227 * 1024 ? epb * blocks_per_sm(kernel, T * epb, smem(epb)) : 0;
         if (n >= most) {
@@ -285,7 +288,7 @@ int sponge<FR_REAL, FR_DIM>(int P, const frk::Sponge<FR_REAL>& sp, FR_REAL* a, F
     if (sp.n <= 0) return 0;
     const unsigned blocks = unsigned((sp.n + 3) / 4);
 #define C(PP) (frk::k_sponge<FR_DIM, PP, FR_REAL><<<blocks, 128,                                             \
-                   8 * frk::Sz<FR_DIM, PP>::NV * frk::Sz<FR_DIM, PP>::NSP * sizeof(FR_REAL), s>>>(sp, a, b, \
+                   8 * frk::Smem<FR_DIM, PP>::UA * sizeof(FR_REAL), s>>>(sp, a, b, \
                                                                                               uf_out, op), \
                int(cudaGetLastError()))
     FR_DISPATCH(C)
