@@ -35,6 +35,14 @@ cudaError_t prep(K kernel, size_t smem, unsigned long long& done) {
     return e;
 }
 
+// kernels that run beside the element kernels ask for the same carveout (an SM
+// holds one split of its memory at a time)
+template <typename K>
+int side_prep(K kernel) {
+    return int(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                    int(cudaSharedmemCarveoutMaxShared)));
+}
+
 inline unsigned grid_of(int64_t E, int epb) { return unsigned((E + epb - 1) / epb); }
 
 inline int sm_count() {
@@ -238,6 +246,9 @@ int forces<FR_REAL, FR_DIM>(int P, const FR_REAL* uf, const FR_REAL* fvn, const 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (ncand <= 0) return 0;
     const dim3 grid(frk::FORCE_BLOCKS, unsigned(ncand));
+#define C(PP) side_prep(frk::k_forces<FR_DIM, PP, FR_REAL>)
+    [&]() -> int { FR_DISPATCH(C) }();
+#undef C
 #define C(PP) (frk::k_forces<FR_DIM, PP, FR_REAL><<<grid, 256, 0, s>>>(uf, fvn, wall_ef, wall_off, op, g, gm1, \
                                                                         viscous, part),                      \
                frk::k_forces_fin<<<ncand, 32, 0, s>>>(part, frk::FORCE_BLOCKS, fnow, fsum, fcnt),          \
@@ -251,6 +262,9 @@ int sample<FR_REAL, FR_DIM>(int P, const FR_REAL* u, const frk::Surf<FR_REAL>* s
                             const frk::Phys<FR_REAL>& ph, void* stream) {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const dim3 grid(unsigned((int64_t(most) * 32 + 255) / 256), unsigned(nsurf));
+#define C(PP) side_prep(frk::k_sample<FR_DIM, PP, FR_REAL>)
+    [&]() -> int { FR_DISPATCH(C) }();
+#undef C
 #define C(PP) (frk::k_sample<FR_DIM, PP, FR_REAL><<<grid, 256, 0, s>>>(u, surf, ph),                            \
                frk::k_bump<FR_REAL><<<unsigned((nsurf + 31) / 32), 32, 0, s>>>(surf, nsurf), int(cudaGetLastError()))
     FR_DISPATCH(C)

@@ -17,6 +17,11 @@ cudaError_t red_prep(K kernel, size_t smem, unsigned long long& done) {
     const unsigned long long bit = 1ull << (dev & 63);
     if (done & bit) return cudaSuccess;
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    // the same carveout as the kernels they run beside: an SM holds one split of
+    // its memory at a time, and kernels that ask for another one wait for it to drain
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 int(cudaSharedmemCarveoutMaxShared));
     if (e == cudaSuccess) done |= bit;
     return e;
 }
