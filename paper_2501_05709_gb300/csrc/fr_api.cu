@@ -227,6 +227,11 @@ frk::Ops<Real> ops_of(const frg::Ref1D& r) {
     }
     op.lhm = Real(lhm);
     op.lhp = Real(lhp);
+    for (int i = 0; i < r.np; ++i)
+        for (int j = 0; j < r.np; ++j)
+            op.Dc[i * frk::MAXNP + j] = Real(static_cast<long double>(r.D[i][j]) +
+                                             static_cast<long double>(r.hm[i]) * r.lm[j] -
+                                             static_cast<long double>(r.hp[i]) * r.lp[j]);
     return op;
 }
 

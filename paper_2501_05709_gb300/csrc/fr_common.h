@@ -27,6 +27,9 @@ struct Ops {
     Real w[MAXNP];
     Real dlm[MAXNP];  // l_j'(-1), derivative of the basis at the left end
     Real lhm, lhp;
+    // divergence with the flux jumps of both ends joined in (FP64 kernels):
+    // Dc[i][j] = D[i][j] + hm_i lm_j - hp_i lp_j
+    Real Dc[MAXNP * MAXNP];
 };
 
 // Gas and flow constants (Section 2.1, Eqs. 5-7) and the free stream.

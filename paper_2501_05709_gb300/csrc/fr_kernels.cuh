@@ -305,10 +305,16 @@ template <int DIM, typename Real>
 __device__ __forceinline__ void rusanov_axis(const Real* uL, const Real* uR, int d, Real Nd, Real gamma, Real gm1,
                                              Real* F) {
     constexpr int NV = DIM + 2;
-    const Real a2 = Nd * Nd;
-    const Real ia = rsqrt(a2);
-    const Real area = a2 * ia;
-    const Real nd = Nd * ia;
+    Real area, nd;
+    if constexpr (sizeof(Real) == 8) {
+        area = fabs(Nd);
+        nd = Nd < Real(0) ? Real(-1) : Real(1);
+    } else {
+        const Real a2 = Nd * Nd;
+        const Real ia = rsqrt(a2);
+        area = a2 * ia;
+        nd = Nd * ia;
+    }
     const Real irL = Real(1) / uL[0], irR = Real(1) / uR[0];
     Real m2L = Real(0), m2R = Real(0);
 #pragma unroll
@@ -1754,14 +1760,25 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? (MP != 0 ? 72 : DIM == 3 && P ==
             if (NL % T != 0 && tk.t >= NL) break;
             Real s[NP];
             vload_line<DIM, P>(sF + tk.shift, d * NV + tk.vref, d, tk.ln, s);
-            Real m, pp;
-            ends_of<NP>(op, s, m, pp);
-            const Real cL = sc[2 * d * NV * NFP + tk.t] + m;
-            const Real cR = sc[(2 * d + 1) * NV * NFP + tk.t] - pp;
             Real val[NP];
+            const Real fL = sc[2 * d * NV * NFP + tk.t], fR = sc[(2 * d + 1) * NV * NFP + tk.t];
+            if constexpr (sizeof(Real) == 8) {
+                // one matrix (Ops::Dc): 24 FP64 operations a line at p = 3 instead of 34
 #pragma unroll
-            for (int i = 0; i < NP; ++i) val[i] = op.hm[i] * cL + op.hm[NP - 1 - i] * cR;
-            apply_D<NP>(op, s, val);
+                for (int i = 0; i < NP; ++i) {
+                    val[i] = op.hm[i] * fL + op.hm[NP - 1 - i] * fR;
+#pragma unroll
+                    for (int j = 0; j < NP; ++j) val[i] += op.Dc[i * MAXNP + j] * s[j];
+                }
+            } else {
+                Real m, pp;
+                ends_of<NP>(op, s, m, pp);
+                const Real cL = fL + m;
+                const Real cR = fR - pp;
+#pragma unroll
+                for (int i = 0; i < NP; ++i) val[i] = op.hm[i] * cL + op.hm[NP - 1 - i] * cR;
+                apply_D<NP>(op, s, val);
+            }
             if (d > 0) {
                 Real prev[NP];
                 vload_line<DIM, P>(sd + tk.shift, tk.vref, d, tk.ln, prev);
