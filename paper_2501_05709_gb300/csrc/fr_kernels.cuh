@@ -78,6 +78,12 @@ __device__ __forceinline__ bool face_pt(int lane, int it, int& side, int& fp) {
     }
 }
 
+// face points of one direction per lane
+template <int DIM, int P>
+struct FacePts {
+    static constexpr int N = (2 * Sz<DIM, P>::NFP + Grp<DIM, P>::T - 1) / Grp<DIM, P>::T;
+};
+
 // solution point j (along direction d) of the line through face point fp of a
 // face normal to d; face points enumerate the remaining directions in
 // increasing order, the lower one fastest
@@ -483,7 +489,7 @@ struct Smem {
     // pipelined face kernel on affine meshes: two buffers per element group,
     // each [state U | own traces F | neighbour traces F | S, 1/|J|, normals]
     static constexpr int GEO = (DIM * DIM + 1 + 2 * DIM * DIM + 3) / 4 * 4;
-    static constexpr int pl = UA, pn = pl + al(F + 3), pg = pn + al(F);
+    static constexpr int pl = UA, pn = pl + al(F + 3), pg = pn + (rows16 ? al(F) : 0);
     static constexpr int visc_buf = (pg + GEO + 3) / 4 * 4;
     static constexpr int visc_p = 2 * visc_buf;
 };
@@ -969,8 +975,10 @@ __global__ void k_traces(const Real* __restrict__ u, Real* __restrict__ uf, int6
 // derivatives of the face trace (interpolation to the face and
 // differentiation along it commute), across it the derivative of the normal
 // line at its end, sum_j l_j'(+-1) u_j.
+// VS: neighbour traces staged in sn; else in registers rn of the face points' lanes.
 template <int DIM, int P, typename Real, bool diag, bool BND, bool VS>
-__device__ __forceinline__ void visc_faces_affine(const Real* su, const Real* sl, const Real* sn, const Real* sgeo,
+__device__ __forceinline__ void visc_faces_affine(const Real* su, const Real* sl, const Real* sn,
+                                                  const Real (&rn)[DIM][FacePts<DIM, P>::N][DIM + 2], const Real* sgeo,
                                                   const int (&codes)[2 * DIM], int64_t e, Real* __restrict__ fvn,
                                                   const Ops<Real>& op, const Phys<Real>& ph, int lane) {
     using Z = Sz<DIM, P>;
@@ -1003,7 +1011,7 @@ __device__ __forceinline__ void visc_faces_affine(const Real* su, const Real* sl
                     const Real* un = sn + f * NV * NFP;
                     const int fpn = omap<DIM, NP>(code & 7, fp);
 #pragma unroll
-                    for (int v = 0; v < NV; ++v) jv[v] = Real(0.5) * (un[v * NFP + fpn] - uL[v]);
+                    for (int v = 0; v < NV; ++v) jv[v] = Real(0.5) * ((VS ? un[v * NFP + fpn] : rn[d][it][v]) - uL[v]);
                 } else {
                     Real ug[NV], uc[NV];
                     bc_state<DIM>(-code, uL, N, ph, ug, uc);
@@ -1147,10 +1155,11 @@ __global__ void k_visc_face_aff(
         warp_stage_vol<DIM, P>(b, u + el * NV * NSP, lane, T);
         if constexpr (VS) warp_stage<NF * NV * NFP, VS>(b + SM::pl, uf + el * NF * NV * NFP, lane, T);
         else warp_stage_shift<NF * NV * NFP>(b + SM::pl, uf + el * NF * NV * NFP, lane, T);
+        if constexpr (VS)
 #pragma unroll
-        for (int f = 0; f < NF; ++f)
-            if (!BND || codes[f] >= 0)
-                warp_stage<NV * NFP, VS>(b + SM::pn + f * NV * NFP, uf + int64_t(codes[f] >> 3) * NV * NFP, lane, T);
+            for (int f = 0; f < NF; ++f)
+                if (!BND || codes[f] >= 0)
+                    warp_stage<NV * NFP, VS>(b + SM::pn + f * NV * NFP, uf + int64_t(codes[f] >> 3) * NV * NFP, lane, T);
         for (int k = lane; k < NGEO; k += T) {
             const Real* src = k < DIM * DIM ? g.S + el * g.sS_e + k * g.sS_k
                             : k == DIM * DIM ? g.iJ + el * g.sJ_e
@@ -1158,15 +1167,40 @@ __global__ void k_visc_face_aff(
             cp_async_small<int(sizeof(Real))>(b + SM::pg + k, src);
         }
     };
+    // neighbour traces of this lane's face points, of the element after the current
+    // one (not VS)
+    constexpr int NFI = FacePts<DIM, P>::N;
+    Real rn[DIM][NFI][NV], rnext[DIM][NFI][NV];
+    auto load_nbr = [&](int mine, Real (&r)[DIM][NFI][NV]) {
+        int codes[NF];
+#pragma unroll
+        for (int f = 0; f < NF; ++f) codes[f] = __shfl_sync(0xffffffffu, mine, f);
+#pragma unroll
+        for (int d = 0; d < DIM; ++d)
+#pragma unroll
+            for (int it = 0; it < NFI; ++it) {
+                int side, fp;
+                if (!face_pt<DIM, P>(lane, it, side, fp)) continue;
+                const int code = side ? codes[2 * d + 1] : codes[2 * d];  // static register indices
+                if (BND && code < 0) continue;
+                const Real* un = uf + int64_t(code >> 3) * NV * NFP + omap<DIM, Z::NP>(code & 7, fp);
+#pragma unroll
+                for (int v = 0; v < NV; ++v) r[d][it][v] = un[v * NFP];
+            }
+    };
     int mineA = lw < NF ? g.nbr[e * NF + lw] : 0;                 // codes of e
     int64_t en = e + G;
     int mineB = (en < E && lw < NF) ? g.nbr[en * NF + lw] : 0;   // codes of the next element
     stage(e, buf, mineA);
     cp_async_commit();
+    if constexpr (!VS) load_nbr(mineA, rn);
     int b = 0;
     for (;;) {
         Real* cur = buf + b * BUF;
-        if (en < E) stage(en, buf + (b ^ 1) * BUF, mineB);
+        if (en < E) {
+            stage(en, buf + (b ^ 1) * BUF, mineB);
+            if constexpr (!VS) load_nbr(mineB, rnext);
+        }
         cp_async_commit();
         const int64_t enn = en + G;
         const int mineC = (enn < E && lw < NF) ? g.nbr[enn * NF + lw] : 0;
@@ -1178,14 +1212,21 @@ __global__ void k_visc_face_aff(
         if (!g.order || g.order[e] >= P)
             visc_faces_affine<DIM, P, Real, MP == 2, BND, VS>(
                 staged_vol<DIM, P>(cur, u + e * NV * NSP),
-                cur + SM::pl + (VS ? 0 : stage_shift(uf + e * NF * NV * NFP)), cur + SM::pn, cur + SM::pg, codes, e,
-                fvn, op, ph, lane);
+                cur + SM::pl + (VS ? 0 : stage_shift(uf + e * NF * NV * NFP)), cur + SM::pn, rn, cur + SM::pg, codes,
+                e, fvn, op, ph, lane);
         if (en >= E) break;
         grp_sync<T>(grp);   // every thread is done with cur before it is refilled
         e = en;
         en = enn;
         mineA = mineB;
         mineB = mineC;
+        if constexpr (!VS)
+#pragma unroll
+            for (int d = 0; d < DIM; ++d)
+#pragma unroll
+                for (int it = 0; it < NFI; ++it)
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) rn[d][it][v] = rnext[d][it][v];
         b ^= 1;
     }
 }
