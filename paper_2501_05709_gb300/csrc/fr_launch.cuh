@@ -65,22 +65,25 @@ int blocks_per_sm(K kernel, int threads, size_t smem) {
 // warps (2 or 4 elements a block) and 108 us with 16 (8 a block), on 100,000 curved
 // elements 319 against 342 us.  With fewer than 20 elements per SM the last wave
 // counts more than the number of warps, and blocks of one element level it (2,400
-// curved elements in FP64: 420 us against 440 to 510 us with 2 to 8).  `tie`: the
-// tile taken among equal ones if it is one of them, else the smallest above 1.
+// curved elements in FP64: 420 us against 440 to 510 us with 2 to 8).  `tie`: taken
+// instead if it keeps three quarters of those warps (2 for the persistent face
+// kernel, whose elements of a block wait for each other at every tile: box of 32^3
+// at p = 4 with 2 elements a block 88 us, with 3: 94; p = 3 39.2 against 39.8).
 template <typename K, typename S>
-int best_tile(K kernel, int T, S smem, int64_t E, int tie = 2) {
+int best_tile(K kernel, int T, S smem, int64_t E, int tie = 0) {
     int best = 1, most = blocks_per_sm(kernel, T, smem(1));
     if (E < 20 * int64_t(sm_count())) return 1;
     // FP64 is bound by its pipe, not by latency: whole warps a block count (4,096
     // affine elements at p = 3: 427 us a stage with 4, 432 with 2)
     if (sizeof(FR_REAL) == 8 && smem(4) <= 113 * 1024 && blocks_per_sm(kernel, 4 * T, smem(4)) > 0) return 4;
-    for (int epb : {8, 6, 1, 4, 3, 2, tie}) {   // of equal ones the last
+    for (int epb : {8, 6, 1, 4, 3, 2}) {   // of equal ones the last
         const int n = smem(epb) <= 227 * 1024 ? epb * blocks_per_sm(kernel, T * epb, smem(epb)) : 0;
         if (n >= most) {
             most = n;
             best = epb;
         }
     }
+    if (tie && 4 * tie * blocks_per_sm(kernel, T * tie, smem(tie)) >= 3 * most) best = tie;
     return best;
 }
 
@@ -127,7 +130,7 @@ int visc_p(const FR_REAL* u, const FR_REAL* uf, FR_REAL* fvn, int64_t E, const f
         const size_t sm = smem(std::max(lc.epb, 1));
         static unsigned long long done = 0;
         cudaError_t e = prep(k, sm, done);
-        if (lc.epb < 0) return e == cudaSuccess ? best_tile(k, frk::Grp<FR_DIM, P>::T, smem, E, 4) : 1;
+        if (lc.epb < 0) return e == cudaSuccess ? best_tile(k, frk::Grp<FR_DIM, P>::T, smem, E, 2) : 1;
         if (e != cudaSuccess) return int(e);
         if (E == 0) return 0;
         const int threads = frk::Grp<FR_DIM, P>::T * lc.epb;
