@@ -1946,8 +1946,9 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? (MP != 0 ? 72 : DIM == 3 && P ==
 // stage arrays afterwards equals adding it to R first: stage 0 adds s to R;
 // RK4 stages 1-4 add (dt/2, dt/2, dt, dt/6) s to the stage output (us, us,
 // us, u0) and (dt/6, dt/3, dt/3, -) s to acc (the coefficient form: (c + d f)
-// dt s and f dt s); the element's next traces are then rewritten from its
-// updated stage output.
+// dt s and f dt s); the next traces of the element's energy are then rewritten from
+// its updated stage output.  A chain of dependent loads and one sine: what does not
+// depend on the sine is loaded before it, and the other variables stay.
 template <int DIM, int P, typename Real>
 __global__ void k_source_stage(const __grid_constant__ Src<Real> src, const __grid_constant__ Stage<Real> st,
                                const __grid_constant__ Ops<Real> op) {
@@ -1959,54 +1960,63 @@ __global__ void k_source_stage(const __grid_constant__ Src<Real> src, const __gr
     const int j = blockIdx.x * (blockDim.x >> 5) + warp;
     if (j >= src.nentry) return;
     Real* sst = reinterpret_cast<Real*>(smem) + warp * NV * NSP;   // updated element state (volume placement)
+    constexpr int NI = (NSP + 31) / 32;
     const int64_t e = src.elem[j];
     const int c = src.cand[j];
+    // classic RK4, or the coefficient form (acc gains f dt s, the output (c + d f) dt s)
+    const bool last = st.ls ? st.last != 0 : st.stage == 4;
+    const int64_t gbase = (e * NV + (NV - 1)) * NSP;                             // energy row
+    Real* out = (st.stage == 0 ? st.R : last ? st.u0 : st.us) + gbase;
+    Real* acc = st.stage == 0 || last ? nullptr : st.acc + gbase;
+    Real o[NI], ac[NI];
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+        const int sp = lane + 32 * i;
+        o[i] = sp < NSP ? out[sp] : Real(0);
+        ac[i] = sp < NSP && acc ? acc[sp] : Real(0);
+    }
     const double dt = double(st.dte ? st.dte[e] : st.dt);
     const double t = src.tnow[c] + src.cfac * dt;
-    double amp[MAXSRC];
-#pragma unroll
+    double sv[NI] = {};
     for (int m = 0; m < MAXSRC; ++m) {
         const double a = src.A[c * MAXSRC + m];
-        amp[m] = a != 0.0 ? a * sinpi(2.0 * src.f[c * MAXSRC + m] * t) : 0.0;
-    }
-    // share of the source in the stage output and in acc: classic RK4, or the
-    // coefficient form (acc gains f dt s, the output (c + d f) dt s)
-    const bool last = st.ls ? st.last != 0 : st.stage == 4;
-    const double cs = st.ls ? (double(st.cc) + double(st.cd) * double(st.cf)) * dt
-                            : st.stage == 3 ? dt : st.stage == 4 ? dt / 6.0 : 0.5 * dt;
-    const double ca = st.ls ? double(st.cf) * dt : st.stage == 1 ? dt / 6.0 : dt / 3.0;
-    const int64_t gbase = (e * NV + (NV - 1)) * NSP;                             // energy row
-    for (int sp = lane; sp < NSP; sp += 32) {
-        double sv = 0.0;
+        if (a == 0.0) continue;
+        Real w[NI];
 #pragma unroll
-        for (int m = 0; m < MAXSRC; ++m) sv += amp[m] * double(src.w[(int64_t(j) * MAXSRC + m) * NSP + sp]);
-        if (st.stage == 0) {
-            st.R[gbase + sp] += Real(sv);
-            continue;
+        for (int i = 0; i < NI; ++i) {
+            const int sp = lane + 32 * i;
+            w[i] = sp < NSP ? src.w[(int64_t(j) * MAXSRC + m) * NSP + sp] : Real(0);
         }
-        const Real du = Real(cs * sv);
-        if (last) {
-            st.u0[gbase + sp] += du;
-        } else {
-            st.us[gbase + sp] += du;
-            st.acc[gbase + sp] += Real(ca * sv);
-        }
+        const double amp = a * sinpi(2.0 * src.f[c * MAXSRC + m] * t);
+#pragma unroll
+        for (int i = 0; i < NI; ++i) sv[i] += amp * double(w[i]);
+    }
+    // share of the source in the stage output and in acc
+    const double cs = st.stage == 0 ? 1.0
+                      : st.ls       ? (double(st.cc) + double(st.cd) * double(st.cf)) * dt
+                                    : st.stage == 3 ? dt : st.stage == 4 ? dt / 6.0 : 0.5 * dt;
+    const double ca = st.ls ? double(st.cf) * dt : st.stage == 1 ? dt / 6.0 : dt / 3.0;
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+        const int sp = lane + 32 * i;
+        if (sp >= NSP) break;
+        o[i] += Real(cs * sv[i]);
+        out[sp] = o[i];
+        if (acc) acc[sp] = ac[i] + Real(ca * sv[i]);
+        sst[VL::pt(NV - 1, sp)] = o[i];
     }
     if (st.stage == 0 || !st.uf_next) return;
+    // the next traces of the energy, rewritten from its updated values with the
+    // same line-end arithmetic as every other element's, so that traces always
+    // equal the traces of the state (a state set from outside gets the same
+    // values bit for bit); no such element is of reduced degree (fr_set_source)
     __syncwarp();
-    // the next traces of this element, rewritten from its updated state with
-    // the same line-end arithmetic as every other element's, so that traces
-    // always equal the traces of the state (a state set from outside gets the
-    // same values bit for bit)
-    const Real* out = (last ? st.u0 : st.us) + e * NV * NSP;
-    for (int k = lane; k < NV * NSP; k += 32) sst[VL::pt(k / NSP, k % NSP)] = out[k];
-    __syncwarp();
-    Real* uf = st.uf_next + e * NF * NV * NFP;
+    Real* uf = st.uf_next + (e * NF * NV + NV - 1) * NFP;
 #pragma unroll
     for (int d = 0; d < DIM; ++d)
-        for (int t = lane; t < NV * NFP; t += 32) {
+        for (int t = lane; t < NFP; t += 32) {
             Real m, p;
-            line_ends<DIM, P>(sst, t / NFP, op, d, t % NFP, m, p);
+            line_ends<DIM, P>(sst, NV - 1, op, d, t, m, p);
             uf[2 * d * NV * NFP + t] = m;
             uf[(2 * d + 1) * NV * NFP + t] = p;
         }
