@@ -225,9 +225,54 @@ __device__ __forceinline__ void visc_flux(const Real* u, const Real (*G)[DIM], R
     }
 }
 
+// FP64: F - F_vis from gradients that still lack a factor c[j] in direction j, with
+// ir = 1/rho and a symmetric F[1 + i][j].  The FP64 pipe bounds the kernel, so 1/rho,
+// mu and c enter as one factor on differences of raw gradients, and each symmetric
+// entry is formed once: 64 operations a point for 101 with visc_flux in 3D
+// (axis-aligned elements; 88 for 115 on others).
+template <int DIM>
+__device__ __forceinline__ void visc_sub(const double* u, double ir, const double (*G)[DIM], const double* c, double mu,
+                                         double kappa, double (*F)[DIM]) {
+    constexpr int NV = DIM + 2;
+    double V[DIM], g[DIM][DIM], w[DIM];
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) V[i] = u[1 + i] * ir;
+    const double Er = u[NV - 1] * ir, mr = mu * ir, kr = kappa * ir;
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) {
+        double s = G[NV - 1][j] - Er * G[0][j];
+#pragma unroll
+        for (int i = 0; i < DIM; ++i) {
+            const double d = G[1 + i][j] - V[i] * G[0][j];
+            s -= V[i] * d;
+            g[i][j] = d * (mr * c[j]);
+        }
+        w[j] = s * (kr * c[j]);
+    }
+    double div = 0.0;
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) div += g[i][i];
+    div *= 2.0 / 3.0;
+#pragma unroll
+    for (int i = 0; i < DIM; ++i)
+#pragma unroll
+        for (int j = i; j < DIM; ++j) {
+            const double t = i == j ? 2.0 * g[i][i] - div : g[i][j] + g[j][i];
+            F[1 + i][j] -= t;
+            w[j] += V[i] * t;
+            if (i != j) {
+                F[1 + j][i] = F[1 + i][j];
+                w[i] += V[j] * t;
+            }
+        }
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) F[NV - 1][j] -= w[j];
+}
+
 // The same viscous flux contracted with a vector N, F_vis(u, G).N, without
 // forming the tensor: (tau N)_i = mu sum_j (dV_i/dx_j + dV_j/dx_i) N_j
-// - (2/3) mu div V N_i and the energy entry V.(tau N) - q.N.
+// - (2/3) mu div V N_i and the energy entry V.(tau N) - q.N.  In FP64 1/rho and
+// mu are one factor at the end.
 template <int DIM, typename Real>
 __device__ __forceinline__ void visc_flux_n(const Real* u, const Real (*G)[DIM], Real mu, Real kappa, const Real* N,
                                             Real* Fn) {
@@ -239,12 +284,17 @@ __device__ __forceinline__ void visc_flux_n(const Real* u, const Real (*G)[DIM],
     Real gV[DIM][DIM];
     Real gn = Real(0);
     const Real Er = u[NV - 1] * ir;
+    const Real sr = sizeof(Real) == 8 ? Real(1) : ir;   // 1/rho: here, or at the end
+    if (sizeof(Real) == 8) {
+        mu *= ir;
+        kappa *= ir;
+    }
 #pragma unroll
     for (int j = 0; j < DIM; ++j) {
-        Real s = (G[NV - 1][j] - Er * G[0][j]) * ir;
+        Real s = (G[NV - 1][j] - Er * G[0][j]) * sr;
 #pragma unroll
         for (int i = 0; i < DIM; ++i) {
-            gV[i][j] = (G[1 + i][j] - V[i] * G[0][j]) * ir;
+            gV[i][j] = (G[1 + i][j] - V[i] * G[0][j]) * sr;
             s -= V[i] * gV[i][j];
         }
         gn += s * N[j];
@@ -279,6 +329,25 @@ __device__ __forceinline__ void visc_flux_axis(const Real* u, const Real (*G)[DI
     Real V[DIM];
 #pragma unroll
     for (int i = 0; i < DIM; ++i) V[i] = u[1 + i] * ir;
+    if constexpr (sizeof(Real) == 8) {   // 1/rho, mu and Nd as one factor at the end
+        const Real cm = mu * ir * Nd, ck = kappa * ir * Nd, Er = u[NV - 1] * ir;
+        Real g[DIM], div = Real(0), en = Real(0), s = G[NV - 1][d] - Er * G[0][d];
+#pragma unroll
+        for (int i = 0; i < DIM; ++i) {
+            g[i] = G[1 + i][d] - V[i] * G[0][d];
+            s -= V[i] * g[i];
+            div += i == d ? g[i] : G[1 + i][i] - V[i] * G[0][i];
+        }
+        Fn[0] = Real(0);
+#pragma unroll
+        for (int i = 0; i < DIM; ++i) {
+            const Real t = i == d ? Real(2) * g[i] - Real(2.0 / 3.0) * div : g[i] + (G[1 + d][i] - V[d] * G[0][i]);
+            Fn[1 + i] = cm * t;
+            en += V[i] * Fn[1 + i];
+        }
+        Fn[NV - 1] = en + ck * s;
+        return;
+    }
     Real gV[DIM][DIM];
 #pragma unroll
     for (int j = 0; j < DIM; ++j)
@@ -1680,17 +1749,20 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? (MP != 0 ? 72 : DIM == 3 && P ==
             const Real vj = uu[1 + j] * ir;
             F[0][j] = uu[1 + j];
 #pragma unroll
-            for (int i = 0; i < DIM; ++i) F[1 + i][j] = uu[1 + i] * vj + (i == j ? p : Real(0));
+            for (int i = 0; i < DIM; ++i)
+                F[1 + i][j] = sizeof(Real) == 8 && i < j ? F[1 + j][i] : uu[1 + i] * vj + (i == j ? p : Real(0));
             F[NV - 1][j] = (uu[NV - 1] + p) * vj;
         }
         if constexpr (VISC) {
             const Real iJ = curved ? sg[DIM * DIM * NSP + sp] : g.iJ[e * g.sJ_e];
             Real G[NV][DIM];
+            constexpr bool late = sizeof(Real) == 8;   // 1/|J| (and a diagonal S) as factors of visc_sub
             if constexpr (diag) {
 #pragma unroll
                 for (int v = 0; v < NV; ++v)
 #pragma unroll
-                    for (int i = 0; i < DIM; ++i) G[v][i] = S[i * DIM + i] * sF[VL::pt(i * NV + v, sp)] * iJ;
+                    for (int i = 0; i < DIM; ++i)
+                        G[v][i] = late ? sF[VL::pt(i * NV + v, sp)] : S[i * DIM + i] * sF[VL::pt(i * NV + v, sp)] * iJ;
             } else {
                 if constexpr (sizeof(Real) == 4) {
 #pragma unroll
@@ -1714,15 +1786,22 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? (MP != 0 ? 72 : DIM == 3 && P ==
                         Real acc = Real(0);
 #pragma unroll
                         for (int d = 0; d < DIM; ++d) acc += S[d * DIM + i] * sF[VL::pt(d * NV + v, sp)];
-                        G[v][i] = acc * iJ;
+                        G[v][i] = late ? acc : acc * iJ;
                     }
             }
-            Real Fv[NV][DIM];
-            visc_flux<DIM>(uu, G, ph.mu, ph.kappa, Fv);
+            if constexpr (late) {
+                Real c[DIM];
 #pragma unroll
-            for (int v = 0; v < NV; ++v)
+                for (int i = 0; i < DIM; ++i) c[i] = diag ? S[i * DIM + i] * iJ : iJ;
+                visc_sub<DIM>(uu, ir, G, c, ph.mu, ph.kappa, F);
+            } else {
+                Real Fv[NV][DIM];
+                visc_flux<DIM>(uu, G, ph.mu, ph.kappa, Fv);
 #pragma unroll
-                for (int i = 0; i < DIM; ++i) F[v][i] -= Fv[v][i];
+                for (int v = 0; v < NV; ++v)
+#pragma unroll
+                    for (int i = 0; i < DIM; ++i) F[v][i] -= Fv[v][i];
+            }
         }
         if constexpr (diag) {
 #pragma unroll
