@@ -319,8 +319,10 @@ int fwh_clear(fr_ctx* ctx, int handle);
  * Minf[3] (mean-flow Mach vector), c0, rho0, p0.  ncopies must be odd.
  * Output: p_out (device double [nobs][cap]) receives p'(t*_i) for
  * i < nt_out[o]; t0_out[o] (host) is the first unified time of observer o;
- * the unified step is dtau.  The library allocates and frees its own
- * scratch (one partial-sum row per block of panels).  Errors: FR_EINVAL
+ * the unified step is dtau.  The library takes its own scratch (the series of
+ * a batch of panels and partial-sum rows) from a pool of the device that keeps
+ * at most 256 MB between calls and gives them back in fr_mesh_load and
+ * fr_destroy; without memory pools it allocates and frees.  Errors: FR_EINVAL
  * (nt < 5, even ncopies, |Minf| >= 1), FR_EWINDOW (empty window for some
  * observer, or longer than cap), FR_ENOMEM, FR_ECUDA.  Synchronises stream. */
 int fwh_integrate(const double* hist, int nt, int npts, const double* y, const double* n,
@@ -344,8 +346,8 @@ int fwh_integrate(const double* hist, int nt, int npts, const double* y, const d
  *   - Every call looks up the array's device address in the current
  *     device's context (cudaGetSymbolAddress, which allocates nothing), so
  *     the address is never stale, e.g. after cudaDeviceReset.  Like
- *     fwh_integrate, the call reads the panel positions back to the host
- *     and synchronises the stream before it returns.
+ *     fwh_integrate, the call reads the observers' smallest and largest
+ *     delays back to the host and synchronises the stream before it returns.
  *   - Every call on a device shares the one array: calls that overlap on
  *     the GPU (other streams or threads) race and give wrong results.  Each
  *     call writes all the scratch it reads, so nothing needs clearing.
@@ -370,7 +372,7 @@ int fwh_integrate_noalloc(const double* hist, int nt, int npts, const double* y,
  *   nfreq_out  host int: L/2 + 1
  * Errors: FR_EINVAL for null pointers, nobs < 1, nseg < 1, ld < nt, dt <= 0,
  * L < 2 (record too short) or cap < L/2 + 1; FR_ENOMEM if its scratch
- * (twiddle table, windowed segments: 16 L + 8 nobs nseg L bytes) cannot be
+ * (twiddle table, folded segments: 16 L + 8 nobs nseg (L + 2) bytes) cannot be
  * allocated.  Synchronises the stream before returning. */
 int fwh_psd(const double* p, int nobs, int nt, int ld, double dt, int nseg, double* psd, int cap,
             int* nfreq_out, void* stream);
