@@ -167,7 +167,6 @@ class Clocks:
 # ----------------------------------------------------------------------------- ncu counters
 KERNEL_SOURCES = ("csrc/fr_kernels.cuh", "csrc/fr_common.h", "csrc/fr_launch.cuh", "csrc/fr_f32_3d.cu",
                   "csrc/fr_f64_3d.cu", "build.py")
-FWH_SOURCES = ("csrc/fwh.cu", "build.py")
 
 
 def kernel_source_hash(files=KERNEL_SOURCES):
@@ -194,7 +193,7 @@ def ncu_counter(workload, precision, kernel, key):
         lines = open(path).read().splitlines()
     except OSError:
         return None
-    src = kernel_source_hash(FWH_SOURCES if kernel.startswith("fwh") else KERNEL_SOURCES)
+    src = kernel_source_hash()
     for ln in lines:
         if ln.startswith("#") or "=" not in ln:
             continue
@@ -602,20 +601,20 @@ def fwh_leg():
     torch.cuda.synchronize()
     t_psd = time.perf_counter() - t0
     work = len(y) * len(obs) * 3 * nt
-    # FP64-bound: executed FP64 flops of one call (ncu, all FW-H kernels)
-    # against the FP64 FMA rate measured on this GPU; the time is the whole call
-    fl = ncu_counter("fwh_directivity", "fp64", "fwh_integrate", "fp64_flops_per_call")
-    pk = F.fr_probe_fp64_peak()
-    ach = fl / t_int / 1e9 if fl else None
+    # bound by the wide integer multiply-adds of k_fwh_accum: 7 integrands of 24 products
+    # for 4 samples and 12 more products a sample, against 32 a clock and SM (measured
+    # with a loop of them) at the highest clock; the time is the whole call
+    ops = 3.0 * len(y) * int(np.sum(nt_out)) * (7 * 24 / 4 + 12)
+    pk = 32 * torch.cuda.get_device_properties(0).multi_processor_count * 2.07
+    ach = ops / t_int / 1e9
     return {"panels": int(len(y)), "observers": int(len(obs)), "copies": 3, "samples": nt,
             "window_samples_min": nmin, "fwh_integrate_ms": 1e3 * t_int,
             "panel_observer_copy_samples_per_s": work / t_int, "fwh_psd_ms": 1e3 * t_psd,
-            "roofline": {"bound": "alu", "kernel": "fwh_integrate (k_fwh_series + k_fwh_accum + k_fwh_reduce), FP64",
-                         "achieved": ach, "peak": pk, "unit": "GFLOP/s", "frac": ach / pk if ach else None,
-                         "flops_per_call": fl,
-                         "peak_source": "measured: FP64 FMA throughput probe (fr_probe_fp64_peak) on this GPU"},
+            "roofline": {"bound": "alu", "kernel": "fwh_integrate (k_fwh_accum, 60-bit fixed point on the integer pipe)",
+                         "achieved": ach, "peak": pk, "unit": "G wide integer multiply-adds/s", "frac": ach / pk,
+                         "peak_source": "32 a clock and SM at 2.07 GHz"},
             "note": "host wall time around each call (each call synchronises and includes its scratch set-up "
-                    "and the host-side observer windows)"}
+                    "and the observer windows)"}
 
 
 def main():
