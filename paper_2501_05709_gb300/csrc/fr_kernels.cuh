@@ -228,8 +228,9 @@ __device__ __forceinline__ void visc_flux(const Real* u, const Real (*G)[DIM], R
 // FP64: F - F_vis from gradients that still lack a factor c[j] in direction j, with
 // ir = 1/rho and a symmetric F[1 + i][j].  The FP64 pipe bounds the kernel, so 1/rho,
 // mu and c enter as one factor on differences of raw gradients, and each symmetric
-// entry is formed once: 64 operations a point for 101 with visc_flux in 3D
-// (axis-aligned elements; 88 for 115 on others).
+// entry is formed once: with the gradients 76 operations a point for 110 with
+// visc_flux in 3D (axis-aligned elements; 118 for 140 on others).  k_residual on
+// 4,096 axis-aligned elements at p = 3: 302 to 283 us.
 template <int DIM>
 __device__ __forceinline__ void visc_sub(const double* u, double ir, const double (*G)[DIM], const double* c, double mu,
                                          double kappa, double (*F)[DIM]) {
