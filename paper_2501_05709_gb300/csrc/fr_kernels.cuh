@@ -2180,8 +2180,11 @@ __global__ void k_sponge(const __grid_constant__ Sponge<Real> sp, Real* __restri
 // Bounds of one point: v = |V| + sqrt(gamma p / rho) in FP32 is off by at most 16
 // roundings (divisions and roots by approximations of 2 units in the last place)
 // of each term, the pressure's own cancellation included, which is relative to
-// gamma - 1 times the sum of its two terms: 1e-6 covers 16 roundings of 6e-8.  A
-// point without a positive finite pressure has no bound (up_e = infinity).
+// gamma - 1 times the sum of its two terms: 1e-6 covers 16 roundings of 6e-8 (and
+// 2e-19 / rho what squares below the smallest normal number leave out).  A point
+// whose pressure is not positive beyond that rounding (S below) has no bounds
+// (up_e = infinity, and it does not raise the candidate's lower bound): in double
+// its pressure may be negative, and the point is then left out of the maximum.
 template <int DIM, int P, typename Real>
 __global__ void k_cfl_bound(const Real* __restrict__ u, const Real* __restrict__ hlen, int64_t E,
                             const int64_t* __restrict__ cand_off, int ncand, const __grid_constant__ Phys<Real> ph,
@@ -2205,9 +2208,10 @@ __global__ void k_cfl_bound(const Real* __restrict__ u, const Real* __restrict__
         const float En = float(ue[(NV - 1) * NSP + sp]);
         const float ir = 1.0f / rho, ke = 0.5f * m2 * ir, p = gm1 * (En - ke);
         const float V = sqrtf(m2) * ir, c = sqrtf(float(ph.gamma) * p * ir);
-        const float off = 1e-6f * (V + c * (1.0f + gm1 * (fabsf(En) + fabsf(ke)) / p));
+        const float S = gm1 * (fabsf(En) + fabsf(ke) + 2e-32f * ir);
+        const float off = 1e-6f * (V + c * (1.0f + S / p)) + 2e-19f * ir;
         // (bit tests: fast-math code may drop comparisons with infinity)
-        if (!(p > 0.0f && rho > 0.0f) || not_finite(V) || not_finite(c) || not_finite(off)) {
+        if (!(p > 1e-6f * S && c > 1e-18f && rho > 0.0f) || not_finite(V) || not_finite(c) || not_finite(off)) {
             hi = __int_as_float(0x7f800000);
         } else {
             hi = fmaxf(hi, V + c + off);
