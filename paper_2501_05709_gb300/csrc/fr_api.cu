@@ -105,8 +105,8 @@ struct fr_ctx {
     double adaptive_cfl = 0.0;
     void* hlen = nullptr;                // device Real [E]: element length
     int64_t* cand_off_d = nullptr;       // device [ncand + 1]
-    unsigned long long* lam = nullptr;   // device [ncand]: max spectral rate (double bits)
-    float* cfl_up = nullptr;             // device [E + ncand]: FP32 bounds of the rates (not in FP64)
+    unsigned long long* lam = nullptr;   // device [ncand]: max spectral rate (double bits), then unsigned [ncand]: its lower bounds
+    float* cfl_up = nullptr;             // device [E]: FP32 bounds of the rates (null: none are taken)
     // variable polynomial order (sponge zones), see frk::Sponge
     std::vector<std::vector<int32_t>> order;  // per candidate: [count] degree caps (empty: all p)
     int sp_n = 0;                             // capped elements (0: none)
@@ -462,18 +462,17 @@ int ensure_traces(fr_ctx* c, cudaStream_t s, Prof* pr = nullptr) {
 // ends with the traces of the new u0 in ufb[0].
 template <typename Real>
 int enqueue_adaptive_dt(fr_ctx* c, cudaStream_t s) {
-    CK(cudaMemsetAsync(c->lam, 0, sizeof(unsigned long long) * c->ncand, s));
+    unsigned* low = reinterpret_cast<unsigned*>(c->lam + c->ncand);
+    CK(cudaMemsetAsync(c->lam, 0, (sizeof(unsigned long long) + sizeof(unsigned)) * c->ncand, s));
     const auto ph = phys_of<Real>(c);
     const Real* u = static_cast<const Real*>(c->u0);
     const Real* h = static_cast<const Real*>(c->hlen);
-    unsigned* low = reinterpret_cast<unsigned*>(c->cfl_up ? c->cfl_up + c->E : nullptr);
-    if (low) CK(cudaMemsetAsync(low, 0, sizeof(unsigned) * c->ncand, s));
     int rc = c->dim == 2 ? frl::cfl<Real, 2>(c->p, u, h, c->E, c->cand_off_d, c->ncand, ph, c->lam, c->cfl_up, low, s)
                          : frl::cfl<Real, 3>(c->p, u, h, c->E, c->cand_off_d, c->ncand, ph, c->lam, c->cfl_up, low, s);
     CKL(rc, "time step kernel");
     k_dt_fill<Real><<<256, 256, 0, s>>>(c->lam, c->adaptive_cfl, c->cand_off_d, c->ncand, c->E,
                                         static_cast<Real*>(c->dte), c->dtc);
-    c->launches += low ? 3 : 2;
+    c->launches += c->cfl_up ? 3 : 2;
     CK(cudaGetLastError());
     return FR_OK;
 }
@@ -1754,9 +1753,15 @@ int ensure_dt_buffers(fr_ctx* c) {
         }
         CK(cudaGetLastError());
     }
-    if (!c->lam && cudaMalloc(&c->lam, nc * sizeof(unsigned long long)) != cudaSuccess)
+    if (!c->lam && cudaMalloc(&c->lam, nc * (sizeof(unsigned long long) + sizeof(unsigned))) != cudaSuccess)
         return fail(FR_ENOMEM, "cannot allocate step buffers");
-    if (!c->cfl_up && c->prec != FR_FP64 && cudaMalloc(&c->cfl_up, (size_t(c->E) + nc) * sizeof(float)) != cudaSuccess) {
+    // FP32 bounds of the rates (k_cfl_bound) from 12 elements per SM on: below, all
+    // elements are evaluated at once and the bounds cost a launch more (whole step
+    // size on 1,000 elements at p = 2 10.5 us without, 12.5 with; on 4,096: 31 and 14)
+    int nsm = 1;
+    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) nsm = 1;
+    if (!c->cfl_up && c->prec != FR_FP64 && c->E >= 12 * int64_t(nsm) &&
+        cudaMalloc(&c->cfl_up, size_t(c->E) * sizeof(float)) != cudaSuccess) {
         c->cfl_up = nullptr;
         return fail(FR_ENOMEM, "cannot allocate step buffers");
     }

@@ -2171,11 +2171,12 @@ __global__ void k_sponge(const __grid_constant__ Sponge<Real> sp, Real* __restri
 // 2 |J| / |S[d,:]|, precomputed); the candidate's maximum is kept by an
 // atomic maximum on the bits of the non-negative double (order-independent).
 // Five FP64 divisions and roots a point bind this to the FP64 pipe (708 us on
-// 125,000 elements at p = 2).  For FP32 states k_cfl_bound first takes bounds
-// up_e >= lambda_e in FP32 and the largest lower bound of each candidate; k_cfl then
-// evaluates only the elements whose upper bound reaches it, so the maximum is the
-// same double (708 to about 25 us a
-// step).
+// 125,000 elements at p = 2).  For FP32 states of many elements k_cfl_bound first
+// takes bounds up_e >= lambda_e in FP32 and the largest lower bound of each candidate;
+// k_cfl then evaluates only the elements whose upper bound reaches it, so the maximum
+// is the same double (whole step size on 125,000 elements with 1% of noise 713 to 61
+// us).  Where the rates of most elements agree to 1e-6, as in a uniform flow on a
+// uniform mesh, all of them are evaluated after the bounds (750 us there).
 //
 // Bounds of one point: v = |V| + sqrt(gamma p / rho) in FP32 is off by at most 16
 // roundings (divisions and roots by approximations of 2 units in the last place)
@@ -2244,23 +2245,24 @@ __global__ void k_cfl_bound(const Real* __restrict__ u, const Real* __restrict__
     }
 }
 
-// a warp looks at 32 elements (all of them without bounds) and evaluates, one
-// after the other, those that can hold the candidate's maximum
+// a warp looks at `per` <= 32 elements and evaluates, one after the other, those
+// that can hold the candidate's maximum (without bounds: all)
 template <int DIM, int P, typename Real>
 __global__ void k_cfl(const Real* __restrict__ u, const Real* __restrict__ hlen, int64_t E,
                       const int64_t* __restrict__ cand_off, int ncand, const __grid_constant__ Phys<Real> ph,
-                      const float* __restrict__ up, const unsigned* __restrict__ low,
+                      const float* __restrict__ up, const unsigned* __restrict__ low, int per,
                       unsigned long long* __restrict__ lam) {
     using Z = Sz<DIM, P>;
     constexpr int NSP = Z::NSP, NV = Z::NV;
     const int lane = threadIdx.x & 31;
-    const int64_t e0 = (int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32;
+    const int64_t e0 = (int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per;
     if (e0 >= E) return;
     const int64_t mine = e0 + lane;
     int c = 0;
     while (c + 1 < ncand && mine >= cand_off[c + 1]) ++c;
     // non-negative floats (and infinity) order as their bits do
-    unsigned todo = __ballot_sync(0xffffffffu, mine < E && (!up || __float_as_uint(up[mine < E ? mine : 0]) >= low[c]));
+    const bool in = lane < per && mine < E;
+    unsigned todo = __ballot_sync(0xffffffffu, in && (!up || __float_as_uint(up[in ? mine : 0]) >= low[c]));
     while (todo) {
         const int w = __ffs(todo) - 1;
         todo &= todo - 1;
@@ -2291,7 +2293,8 @@ __global__ void k_cfl(const Real* __restrict__ u, const Real* __restrict__ hlen,
             const double k = double((P + 1) * (P + 1));
             double l = vmax * k / h;
             if (ph.viscous) l += numax * k * k / (h * h);
-            atomicMax(lam + ce, static_cast<unsigned long long>(__double_as_longlong(l)));
+            const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(l));
+            if (b > *static_cast<volatile unsigned long long*>(lam + ce)) atomicMax(lam + ce, b);
         }
     }
 }
