@@ -2245,29 +2245,33 @@ __global__ void k_cfl_bound(const Real* __restrict__ u, const Real* __restrict__
     }
 }
 
-// a warp looks at `per` <= 32 elements and evaluates, one after the other, those
-// that can hold the candidate's maximum (without bounds: all)
-template <int DIM, int P, typename Real>
+// MANY: a warp looks at 4 elements and evaluates, one after the other, those that can
+// hold the candidate's maximum; else at one (without bounds it evaluates every one)
+template <int DIM, int P, typename Real, bool MANY>
 __global__ void k_cfl(const Real* __restrict__ u, const Real* __restrict__ hlen, int64_t E,
                       const int64_t* __restrict__ cand_off, int ncand, const __grid_constant__ Phys<Real> ph,
-                      const float* __restrict__ up, const unsigned* __restrict__ low, int per,
+                      const float* __restrict__ up, const unsigned* __restrict__ low,
                       unsigned long long* __restrict__ lam) {
     using Z = Sz<DIM, P>;
-    constexpr int NSP = Z::NSP, NV = Z::NV;
+    constexpr int NSP = Z::NSP, NV = Z::NV, PER = MANY ? 4 : 1;
     const int lane = threadIdx.x & 31;
-    const int64_t e0 = (int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per;
+    const int64_t e0 = (int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5)) * PER;
     if (e0 >= E) return;
-    const int64_t mine = e0 + lane;
-    int c = 0;
-    while (c + 1 < ncand && mine >= cand_off[c + 1]) ++c;
+    auto cand = [&](int64_t e) {
+        int c = 0;
+        while (c + 1 < ncand && e >= cand_off[c + 1]) ++c;
+        return c;
+    };
     // non-negative floats (and infinity) order as their bits do
-    const bool in = lane < per && mine < E;
-    unsigned todo = __ballot_sync(0xffffffffu, in && (!up || __float_as_uint(up[in ? mine : 0]) >= low[c]));
+    unsigned todo = 1;
+    if (MANY || up) {
+        const int64_t mine = min(e0 + (MANY ? lane & (PER - 1) : 0), E - 1);
+        const bool may = __float_as_uint(up[mine]) >= low[cand(mine)];
+        todo = __ballot_sync(0xffffffffu, may && lane < PER && e0 + lane < E);
+    }
     while (todo) {
-        const int w = __ffs(todo) - 1;
+        const int64_t e = e0 + (__ffs(todo) - 1);
         todo &= todo - 1;
-        const int64_t e = e0 + w;
-        const int ce = __shfl_sync(0xffffffffu, c, w);
         const Real* ue = u + e * NV * NSP;
         double vmax = 0.0, numax = 0.0;
         for (int sp = lane; sp < NSP; sp += 32) {
@@ -2293,8 +2297,7 @@ __global__ void k_cfl(const Real* __restrict__ u, const Real* __restrict__ hlen,
             const double k = double((P + 1) * (P + 1));
             double l = vmax * k / h;
             if (ph.viscous) l += numax * k * k / (h * h);
-            const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(l));
-            if (b > *static_cast<volatile unsigned long long*>(lam + ce)) atomicMax(lam + ce, b);
+            atomicMax(lam + cand(e), static_cast<unsigned long long>(__double_as_longlong(l)));
         }
     }
 }

@@ -320,13 +320,14 @@ int cfl<FR_REAL, FR_DIM>(int P, const FR_REAL* u, const FR_REAL* hlen, int64_t E
     if (E == 0) return 0;
     const unsigned blocks = unsigned((E + 7) / 8);
     // elements a warp looks at in k_cfl: one, or four where bounds leave most of them
-    // out and the warps still fill every SM (125,000 elements at p = 2: 62
-    // us with 4, 72 with 1; with 16 60, but 798 against 750 in a uniform flow, where
-    // all of them are evaluated)
-    const int per = up && E >= 32 * int64_t(sm_count()) ? 4 : 1;
-    const int64_t warps = (E + per - 1) / per;
+    // out and the warps still fill every SM (125,000 elements at p = 2: 62 us with 4, 72
+    // with 1; with 16 60, but 798 against 750 in a uniform flow, where all of them are
+    // evaluated)
+    const bool many = up && E >= 32 * int64_t(sm_count());
+    const unsigned warps = unsigned(many ? (E + 3) / 4 : E);
 #define C(PP) ((up ? (frk::k_cfl_bound<FR_DIM, PP, FR_REAL><<<blocks, 256, 0, s>>>(u, hlen, E, cand_off, ncand, ph, up, low), 0) : 0), \
-               frk::k_cfl<FR_DIM, PP, FR_REAL><<<unsigned((warps + 7) / 8), 256, 0, s>>>(u, hlen, E, cand_off, ncand, ph, up, low, per, lam), \
+               (many ? frk::k_cfl<FR_DIM, PP, FR_REAL, true> : frk::k_cfl<FR_DIM, PP, FR_REAL, false>)                        \
+                   <<<(warps + 7) / 8, 256, 0, s>>>(u, hlen, E, cand_off, ncand, ph, up, low, lam),                           \
                int(cudaGetLastError()))
     FR_DISPATCH(C)
 #undef C
