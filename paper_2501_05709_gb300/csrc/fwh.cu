@@ -16,12 +16,15 @@
 //                  tau = t* - R/c0 (Eq. B.13) with a 4-point cubic Lagrange
 //                  stencil and sums (Eq. B.14), on the integer pipe; one
 //                  partial row per panel group.
+//   k_fwh_accum64: the same sums in double, for the observers whose records the
+//                  fixed point would hold with fewer bits than a double does.
 //   k_fwh_reduce : sums the partial rows in a fixed order, divides by 4 pi.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <climits>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -139,13 +142,11 @@ __global__ void __launch_bounds__(256) k_fwh_series(const double* __restrict__ h
 
 // Fixed-point form of a number: N = x 2^(60 - e) for |x| < 2^e, as two limbs
 // N = h 2^30 + l with -2^29 <= l < 2^29.  e follows from the largest high word H
-// of the series.  A series of zeros has H = 0; a panel with an infinity, a NaN or
-// values below 2^-959 keeps its doubles and is summed in double (fwh_wide).
-__device__ __forceinline__ bool fwh_wide(int H) { return H >= 0x7ff00000 || (H > 0 && H < (64 << 20)); }
-__device__ __forceinline__ bool fwh_wide_panel(const int* hw) {
-    bool w = false;
-    for (int v = 0; v < 8; ++v) w = w || fwh_wide(hw[v]);
-    return w;
+// of the series.  A series of zeros has H = 0; a record with an infinity, a NaN or
+// a series of magnitudes beyond 2^500 either way is summed in double.
+__device__ __forceinline__ bool fwh_wide(int hi) {
+    const int ex = (hi >> 20) & 0x7ff;
+    return (hi & 0x7fffffff) != 0 && (ex < 523 || ex > 1523);
 }
 // mantissa of |x| as an integer < 2^53 (x normal or 0), shifted left by s and
 // right by d with rounding
@@ -162,15 +163,19 @@ __device__ __forceinline__ int2 fwh_limbs(long long N) {
     return make_int2(h, int(N - (static_cast<long long>(h) << 30)));
 }
 
-// the series of a batch to fixed point, in place (16 bytes, two series, a thread)
-__global__ void k_fwh_fix(double* __restrict__ X, const int* __restrict__ hw, int nt, int np) {
+// the series of a batch to fixed point, in place (16 bytes, two series, a thread);
+// *wide is set if one has no fixed-point form
+__global__ void k_fwh_fix(double* __restrict__ X, const int* __restrict__ hw, int nt, int np, int* __restrict__ wide) {
     const int64_t n = int64_t(np) * 4 * nt;
     for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
         const int64_t p = i / (4 * int64_t(nt));
         const unsigned at = unsigned(i - p * 4 * nt);
         const int* H = hw + p * 8;
-        if (fwh_wide_panel(H)) continue;
         const int v = 2 * ((at ^ (at >> 3)) & 3);   // the series of this slot (fwh_slot)
+        if (fwh_wide(H[v]) || fwh_wide(H[v + 1])) {
+            *wide = 1;
+            continue;
+        }
         const double2 x = reinterpret_cast<const double2*>(X)[i];
         auto conv = [](double x, int H) {
             const int ex = (__double2hiint(x) >> 20) & 0x7ff;
@@ -186,13 +191,11 @@ __device__ void panel_coefs(const double* y, double dS, const double* obs, const
                             double* delay) {
     double r[3];
     for (int i = 0; i < 3; ++i) r[i] = obs[i] - y[i];
-    double Mr = 0, rr = 0, MM = 0;
+    double Mr = 0, rr = 0;
     for (int i = 0; i < 3; ++i) {
         Mr += k.M[i] * r[i];
         rr += r[i] * r[i];
-        MM += k.M[i] * k.M[i];
     }
-    (void)MM;
     const double b2 = k.b2;
     const double Rs = sqrt(rr + b2 * Mr * Mr) / sqrt(b2);          // Eq. B.8
     const double R = b2 * (Rs - Mr);                               // Eq. B.9
@@ -214,10 +217,11 @@ __device__ void panel_coefs(const double* y, double dS, const double* obs, const
     *delay = R / k.c0;
 }
 
-// One observer of a launch: position, first time and length of its window.
+// One observer of a launch: position, first time and length of its window, and its
+// row of the output.
 struct FwhObs {
     double x[3], tstart;
-    int T, pad;
+    int T, row;
 };
 
 // the delay R / c0 of a panel copy at y (Eqs. B.8, B.9)
@@ -266,25 +270,10 @@ __device__ __forceinline__ void cubic_weights(double x, double (&wt)[4]) {
     wt[2] = -x * (x - 1.0) * (x - 3.0) / 2.0;
     wt[3] = x * (x - 1.0) * (x - 2.0) / 6.0;
 }
-// FP64 form of one sample at source index s (stencil clamped to the record), for
-// panel copies that are not in fixed point
-__device__ double fwh_sample_fp64(const int4* xp, const int* hw, bool wide, int nt, const double* cf, double s) {
-    const int j = max(0, min(nt - 4, int(floor(s)) - 1));
-    double wt[4];
-    cubic_weights(s - double(j), wt);
-    double sum = 0.0;
-    for (int m = 0; m < 4; ++m) {
-        double Ik = 0.0;
-        for (int v = 0; v < NSER; ++v) {
-            const int2 q = reinterpret_cast<const int2*>(xp + fwh_slot(fwh_place(j + m, nt), v >> 1))[v & 1];
-            double val;
-            if (wide) val = __hiloint2double(q.y, q.x);
-            else val = hw[v] ? scalbn(double((static_cast<long long>(q.x) << 30) + q.y), (hw[v] >> 20) - 1082) : 0.0;
-            Ik += cf[v] * val;
-        }
-        sum += wt[m] * Ik;
-    }
-    return sum;
+// start j of the stencil of source index s = i + off, clamped to the record (its
+// position in the stencil is (i - j) + off: s itself rounds off's last bits away)
+__device__ __forceinline__ int fwh_stencil(double s, int nt) {
+    return int(fmin(fmax(floor(s) - 1.0, 0.0), double(nt - 4)));
 }
 
 // Coefficients and source index of sample 0 of panel copy (p, cc)
@@ -295,50 +284,67 @@ __device__ void fwh_panel(const double* y, const double* dS, int p, int cc, doub
     panel_coefs(yy, dS[p], ob.x, k, cf, &delay);
     *off = (ob.tstart - k.tau0 - delay) / k.dtau;
 }
-__device__ __noinline__ double fwh_wide_sample(const int4* xp, const int* hw, bool wide, int nt, const double* y,
-                                        const double* dS, int p, int cc, double Lspan, const FwhObs* ob,
-                                        const FwhConst& k, int i) {
-    double cf[NSER], off;
-    fwh_panel(y, dS, p, cc, Lspan, *ob, k, cf, &off);
-    return fwh_sample_fp64(xp, hw, wide, nt, cf, double(i) + off);
-}
-
 // Sum over panel copies of the interpolated integrand (Eqs. B.2, B.13, B.14), in
 // fixed point on the integer pipe: this GPU multiplies 32-bit integers 32 times
 // as fast as it does FP64, and 18 FP64 operations a panel copy and sample bound
 // the sum in double (18,840 panels, 36 observers, 3 copies, 690 samples: 72 ms in
-// double at 0.6 of the FP64 rate, 13 ms here).
-//   I = sum_v cf_v X_v(j) with X_v = x_v 2^e_v and cf_v 2^e_v = c_v 2^E, E the
-//   panel copy's own exponent, |I| < 2^E: x, c and I have 60 bits below their
-//   exponents, products of limbs h h' + ((h l' + l h') >> 30) drop only l l',
-//   2^-58 of the bound; then p += sum_m w_m I(j + m) with the cubic weights
-//   scaled by 2^(E - Emax - b) (Emax over the block's copies, 2^b twice their
+// double at 0.6 of the FP64 rate, 14 ms here).
+//   I = sum_v cf_v x_v(j) with |x_v| <= m_v < 2^e_v over the record and
+//   sum_v |cf_v| m_v < 2^E: x_v, cf_v 2^e_v / 2^E and I have 60 bits below 2^e_v, 1
+//   and 2^E, products of limbs h h' + ((h l' + l h') >> 30) drop only l l', 2^-62 of
+//   the bound; then p += sum_m w_m I(j + m) with the cubic weights scaled by
+//   2^(E - top - r) (top the largest E of the block's copies, 2^(r + 3) twice their
 //   number), kept as the two sums hh and mid of 64 bits, with which a sum over a
 //   block is exact; it becomes a double once, at the block's end.
-// Each quantity thus carries at least as many bits as a double of the size of its
-// bound (weights of copies that count for less than the block's largest lose bits
-// in proportion).  Error against a reference in another order of summation, 2-norm:
-// 1.3e-13 to 1.5e-12 here, 1.5e-13 to 1.8e-12 in double (it comes from the sources).
+// One exponent holds for the whole record and for all copies of a block, so what is
+// lost is relative to the largest of them: at 96 copies about 2^-54 of 2^top (2-norm
+// of dropped l l' and rounded weights), where double loses about 2^-51 of the largest
+// |I| at that sample.  A sample at which no copy's integrand reaches 2^-10 of 2^top (a
+// transient's rise or decay, the quiet part of a record with one large outlier) may be
+// held worse than by a double.  The kernel takes the largest |I| of each sample's
+// stencils, over those points that count (weight at least 1/32), over some of the block's
+// copies, and marks the observer where that is too small (fwh_loud); a marked observer
+// is summed again in double (k_fwh_accum64).
+// Error against a reference in another order of summation, 2-norm: 1.3e-13 to 1.5e-12
+// here, 1.5e-13 to 1.8e-12 in double (it comes from the sources).
 // A block: one group of panels and one observer; a warp takes 124 samples of it, a
 // lane 4 consecutive ones (31 lanes; lane 31 only supplies the integrands that
 // lane 30's stencils need).  Each integrand is formed once and passed to the lane
 // before it by shuffles: 24 + 12 products of limb pairs, 4 loads of 16 bytes and
-// 1.5 shuffles a sample.  Bound by the multiplier (IMAD.WIDE, about 70% busy).  With
-// 8 samples a lane and 128 registers 1.80 ms against 1.51 ms at 2,198 panels.
+// 1.5 shuffles a sample.  Issue and latency bound it: at 18,840 panels, 36 observers and
+// 3 copies the products need 5.1 of 13.8 ms (at 32 wide multiply-adds a clock and SM),
+// the rest goes to limbs, loads and shuffles at 24 warps an SM.  With 8 samples a lane
+// and 128 registers 1.80 ms against 1.51 ms at 2,198 panels.
 constexpr int ACC_PC = 96;        // panel copies set up at a time
 constexpr int ACC_LANES = 31;     // lanes with samples of their own
 constexpr int ACC_WARPS = 8;      // warps (sample chunks) of a block at most
 constexpr int ACC_S = KO * ACC_LANES;
 
-struct FwhPc {
+constexpr int SILENT = -100000;    // exponent of a copy without a contribution (no branch: that cost 1.5%)
+constexpr int ACC_QUIET = 21;      // bits of a top limb of 2^-10 of the bound (2^20)
+
+struct __align__(16) FwhPc {   // read in 16-byte pieces
     int c[2 * NSER];   // coefficient limbs (h, l)
     int w[8];          // weight limbs
+    int count[4];      // -1: this point of the stencil counts for how loud a sample is, 0: not
     int at[KO];        // place of t = jb + m, m < KO
     double off;        // source index of sample 0
-    int E, sc;         // exponent E; weights are scaled by 2^sc
-    int jb, p, cc, kind;   // kind 1: fixed point, 0: double, 2: no contribution
+    int E, sc;         // exponent E (SILENT: all coefficients and weights are 0); weights are scaled by 2^sc
+    int jb;
 };
+static_assert(sizeof(FwhPc) % 16 == 0 && offsetof(FwhPc, w) % 16 == 0 && offsetof(FwhPc, count) % 16 == 0, "");
 
+// top limb of one integrand (by the top limbs of its factors alone)
+__device__ __forceinline__ int fwh_top(const int* c, const int4* xp, unsigned at) {
+    long long a = 0;
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+        const int4 q = xp[fwh_slot(at, v)];
+        a += static_cast<long long>(c[4 * v]) * q.x;
+        a += static_cast<long long>(c[4 * v + 2]) * q.z;
+    }
+    return abs(int(a >> 30));
+}
 // one integrand, N = I 2^60 / 2^E, of a panel's series at place `at`
 __device__ __forceinline__ long long fwh_integrand(const int (&c)[2 * NSER], const int4* xp, unsigned at) {
     long long a = 0, b = 0;
@@ -360,10 +366,9 @@ __device__ __noinline__ void fwh_end(const FwhPc* rc, const int4* xp, int nt, in
     int c[2 * NSER];
 #pragma unroll
     for (int v = 0; v < 2 * NSER; v += 4) *reinterpret_cast<int4*>(c + v) = *reinterpret_cast<const int4*>(rc->c + v);
-    const double s = double(i) + rc->off;
-    const int j = max(0, min(nt - 4, int(floor(s)) - 1));
+    const int j = fwh_stencil(double(i) + rc->off, nt);
     double wt[4];
-    cubic_weights(s - double(j), wt);
+    cubic_weights(double(i - j) + rc->off, wt);
     long long a = 0, b = 0;
     for (int m = 0; m < 4; ++m) {
         const int2 q = fwh_limbs(fwh_integrand(c, xp, fwh_place(j + m, nt)));
@@ -376,13 +381,66 @@ __device__ __noinline__ void fwh_end(const FwhPc* rc, const int4* xp, int nt, in
     *mid = b & ((1ll << 30) - 1);
 }
 
+// How loud a lane's samples are: for each the bits of the largest top limb, in units
+// of 2^top, over the points of its stencils that count (4 x 8 bits; or-ed, so that one
+// bit too many is possible), over every step-th of the n copies at rec.  A loop of its
+// own: inside k_fwh_accum's it took registers, and 1.1 ms of 14.2 (18,840 panels, 36
+// observers, 3 copies) instead of 0.3.
+__device__ __noinline__ unsigned fwh_loud(const FwhPc* rec, int n, int step, int top, const int4* X, int first, int c0,
+                                          int ncopies, int nt, int unit, int samples) {
+    int loud[KO] = {};
+    for (int w = 0; w < n; w += step) {
+        const FwhPc& rc = rec[w];
+        const int4* xp = X + int64_t(first + (c0 + w) / ncopies) * 4 * nt;
+        const int down = min(31, top - rc.E), t0 = KO * unit + rc.jb;
+        int ih[KO + 3];
+#pragma unroll
+        for (int m = 0; m < KO; ++m) ih[m] = fwh_top(rc.c, xp, min(unsigned(rc.at[m] + unit), unsigned(nt - 1)));
+#pragma unroll
+        for (int m = 0; m < 3; ++m) ih[KO + m] = __shfl_down_sync(0xffffffffu, ih[m], 1);
+#pragma unroll
+        for (int q = 0; q < KO; ++q) {
+            if (t0 + q >= 0 && t0 + q + 3 < nt) {
+                loud[q] |= ((ih[q] & rc.count[0]) | (ih[q + 1] & rc.count[1]) | (ih[q + 2] & rc.count[2]) |
+                            (ih[q + 3] & rc.count[3])) >> down;
+            } else if (q < samples) {   // over an end of the record: the sample's own stencil
+                const int i = KO * unit + q, j = fwh_stencil(double(i) + rc.off, nt);
+                double wt[4];
+                cubic_weights(double(i - j) + rc.off, wt);
+                for (int m = 0; m < 4; ++m)
+                    if (fabs(wt[m]) >= 0.03125) loud[q] |= fwh_top(rc.c, xp, fwh_place(j + m, nt)) >> down;
+            }
+        }
+    }
+    unsigned bits = 0;
+#pragma unroll
+    for (int q = 0; q < KO; ++q) bits |= unsigned(32 - __clz(loud[q])) << (8 * q);
+    return bits;
+}
+
+// a block's panels, samples and copies (k_fwh_accum and k_fwh_accum64)
+struct FwhBlock {
+    int o, row, lane, T, unit, i0, gp0, npc, K;
+    bool mine, idle;
+    __device__ FwhBlock(const FwhObs* obs, int group, int np, int ncopies)
+        : o(blockIdx.x), row(blockIdx.y), lane(threadIdx.x & 31), T(obs[blockIdx.x].T) {
+        unit = lane + ACC_LANES * (int(blockIdx.z) * int(blockDim.x >> 5) + int(threadIdx.x >> 5));
+        i0 = KO * unit;
+        mine = lane < ACC_LANES && i0 < T;                    // this lane stores samples i0.. of its own
+        idle = __shfl_sync(0xffffffffu, i0, 0) >= T;          // no lane of this warp does
+        gp0 = row * group;                                    // panels of this block, within the batch
+        npc = min(group, np - gp0) * ncopies;
+        K = (ncopies - 1) / 2;
+    }
+};
+
 __global__ void __launch_bounds__(32 * ACC_WARPS, 3)
     k_fwh_accum(const int4* __restrict__ X, const int* __restrict__ hwb, int nt, int p0, int np, int nrows,
                 const double* __restrict__ y, const double* __restrict__ dS, const __grid_constant__ FwhConst k,
                 const FwhObs* __restrict__ obs, int Tmax, int ncopies, double Lspan, int group,
-                double* __restrict__ partial) {
+                double* __restrict__ partial, volatile int* flag, volatile int* wide) {
     __shared__ __align__(16) FwhPc rec[ACC_PC];
-    __shared__ int s_top, s_wide;
+    __shared__ int s_top, s_double;
     const int o = blockIdx.x, row = blockIdx.y;
     const int lane = threadIdx.x & 31;
     const int T = obs[o].T;
@@ -393,64 +451,57 @@ __global__ void __launch_bounds__(32 * ACC_WARPS, 3)
     const int gp0 = row * group, gnp = min(group, np - gp0);   // panels of this block, within the batch
     const int npc = gnp * ncopies, K = (ncopies - 1) / 2;
     double* out = partial + (int64_t(o) * nrows + row) * Tmax;   // adds up over the batches of panels
-    const int headroom = 33 - __clz(min(npc, ACC_PC));         // b: 2^b >= 2 npc
+    const int room = max(0, 30 - __clz(min(npc, ACC_PC)));     // r
+    if (threadIdx.x == 0) s_double = *wide | flag[o];
+    __syncthreads();
+    if (s_double) return;   // this observer is summed in double anyway
     for (int c0 = 0; c0 < npc; c0 += ACC_PC) {
         const int n = min(ACC_PC, npc - c0);
         __syncthreads();
-        if (threadIdx.x == 0) {
-            s_top = INT_MIN;
-            s_wide = 0;
-        }
+        if (threadIdx.x == 0) s_top = INT_MIN;
         __syncthreads();
         // coefficients and weights of this chunk's panel copies
-        for (int base = 0; base < n; base += blockDim.x) {
-            const int w = base + threadIdx.x;
-            int E = INT_MIN;
-            if (w < n) {
-                FwhPc& rc = rec[w];
-                const int pl = gp0 + (c0 + w) / ncopies, cc = (c0 + w) % ncopies - K;
-                const int* hw = hwb + pl * 8;
-                double cf[NSER], off;
-                fwh_panel(y, dS, p0 + pl, cc, Lspan, obs[o], k, cf, &off);
-                bool fixed = fabs(off) < 1e9 && !fwh_wide_panel(hw);
+        for (int w = threadIdx.x; w < n; w += blockDim.x) {
+            FwhPc& rc = rec[w];
+            const int pl = gp0 + (c0 + w) / ncopies, cc = (c0 + w) % ncopies - K;
+            const int* hw = hwb + pl * 8;
+            double cf[NSER], off, S = 0.0;
+            fwh_panel(y, dS, p0 + pl, cc, Lspan, obs[o], k, cf, &off);
+            bool fixed = fabs(off) < 1e9;
+#pragma unroll
+            for (int v = 0; v < NSER; ++v) {
+                fixed = fixed && !fwh_wide(__double2hiint(cf[v]));
+                if (hw[v]) S += fabs(cf[v]) * __hiloint2double(hw[v], -1);
+            }
+            if (!fixed) flag[o] = 1;
+            fixed = fixed && S != 0.0;
+            int E = SILENT;
+            const int jb = fixed ? int(floor(off)) - 1 : 0;
+#pragma unroll
+            for (int m = 0; m < KO; ++m) rc.at[m] = fwh_place(jb + m, nt);
+            rc.jb = jb;
+#pragma unroll
+            for (int v = 0; v < 2 * NSER; ++v) rc.c[v] = 0;
+            if (fixed) {
+                E = ((__double2hiint(S * (1.0 + 1e-15)) >> 20) & 0x7ff) - 1022;   // S < 2^E
 #pragma unroll
                 for (int v = 0; v < NSER; ++v) {
+                    // cf 2^e / 2^E, below 2 since 2^e is at most twice the series' largest value
                     const int ex = (__double2hiint(cf[v]) >> 20) & 0x7ff;
-                    fixed = fixed && ex != 0x7ff && (ex != 0 || cf[v] == 0.0);
-                    if (ex != 0 && hw[v] != 0) E = max(E, ex + (hw[v] >> 20) - 2044);
+                    const int2 q = hw[v] == 0 ? make_int2(0, 0) : fwh_limbs(fwh_fix(cf[v], 8, 2045 + E - ex - (hw[v] >> 20)));
+                    rc.c[2 * v] = q.x;
+                    rc.c[2 * v + 1] = q.y;
                 }
-                rc.kind = !fixed ? 0 : E == INT_MIN ? 2 : 1;
-                if (rc.kind == 1) {
-                    E += 3;   // eight terms
-#pragma unroll
-                    for (int v = 0; v < NSER; ++v) {
-                        const int ex = (__double2hiint(cf[v]) >> 20) & 0x7ff;
-                        const int2 q = hw[v] == 0 ? make_int2(0, 0)
-                                                  : fwh_limbs(fwh_fix(cf[v], 4, E - 3 - (ex + (hw[v] >> 20) - 2044)));
-                        rc.c[2 * v] = q.x;
-                        rc.c[2 * v + 1] = q.y;
-                    }
-                    const int jb = int(floor(off)) - 1;
-#pragma unroll
-                    for (int m = 0; m < KO; ++m) rc.at[m] = fwh_place(jb + m, nt);
-                    rc.jb = jb;
-                    atomicMax(&s_top, E);
-                } else {
-                    E = INT_MIN;
-                    if (rc.kind == 0) s_wide = 1;
-                }
-                rc.p = pl;
-                rc.cc = cc;
-                rc.E = E;
-                rc.off = off;
+                atomicMax(&s_top, E);
             }
+            rc.E = E;
+            rc.off = off;
         }
         __syncthreads();
         const int top = s_top;
         for (int w = threadIdx.x; w < n; w += blockDim.x) {
             FwhPc& rc = rec[w];
-            if (rc.kind != 1) continue;
-            const int sc = max(-200, 60 - headroom + rc.E - top);
+            const int sc = rc.E == SILENT ? -200 : max(-200, 60 - room + rc.E - top);
             rc.sc = sc;
             double wt[4];
             cubic_weights(rc.off - floor(rc.off) + 1.0, wt);   // position in the stencil, [1, 2)
@@ -459,6 +510,7 @@ __global__ void __launch_bounds__(32 * ACC_WARPS, 3)
                 const int2 q = fwh_limbs(__double2ll_rn(scalbn(wt[m], sc)));
                 rc.w[2 * m] = q.x;
                 rc.w[2 * m + 1] = q.y;
+                rc.count[m] = fabs(wt[m]) >= 0.03125 ? -1 : 0;
             }
         }
         __syncthreads();
@@ -466,7 +518,7 @@ __global__ void __launch_bounds__(32 * ACC_WARPS, 3)
         long long hh[KO], mid[KO];
 #pragma unroll
         for (int q = 0; q < KO; ++q) hh[q] = mid[q] = 0;
-        bool carry = false;
+        bool carry = n & 1;   // the last copy's sums are carried over
         int pl = gp0 + c0 / ncopies, copy = c0 % ncopies;   // panel copy w (kept uniform: one base address for all lanes)
         for (int w = 0; w < n; ++w) {
             const FwhPc& rc = rec[w];
@@ -475,7 +527,6 @@ __global__ void __launch_bounds__(32 * ACC_WARPS, 3)
                 copy = 0;
                 ++pl;
             }
-            if (rc.kind != 1) continue;
             int ih[KO + 3], il[KO + 3];
             {
                 int c[2 * NSER];
@@ -533,34 +584,123 @@ __global__ void __launch_bounds__(32 * ACC_WARPS, 3)
                     mid[q] &= (1ll << 30) - 1;
                 }
         }
+        // every 32nd copy looked at (fewer copies: every eighth, or all)
+        const unsigned bits = top == INT_MIN ? 0xffffffffu
+                                             : fwh_loud(rec, n, n >= 64 ? 32 : n >= 16 ? 8 : 1, top, X, gp0, c0, ncopies,
+                                                        nt, unit, mine ? T - i0 : 0);
         if (mine)
 #pragma unroll
             for (int q = 0; q < KO; ++q)
                 if (i0 + q < T) {
-                    double v = top == INT_MIN ? 0.0
-                                              : scalbn(double(hh[q]) + double(mid[q]) * (1.0 / 1073741824.0),
-                                                       top + headroom - 60);
-                    if (s_wide)   // panels that are not in fixed point
-                        for (int w = 0; w < n; ++w)
-                            if (rec[w].kind == 0) {
-                                const int* hw = hwb + rec[w].p * 8;
-                                v += fwh_wide_sample(X + int64_t(rec[w].p) * 4 * nt, hw, fwh_wide_panel(hw), nt, y, dS,
-                                              p0 + rec[w].p, rec[w].cc, Lspan, obs + o, k, i0 + q);
-                            }
+                    if (int((bits >> (8 * q)) & 255) < ACC_QUIET) flag[o] = 1;
+                    const double v = top == INT_MIN ? 0.0
+                                                    : scalbn(double(hh[q]) + double(mid[q]) * (1.0 / 1073741824.0),
+                                                             top + room - 60);
                     out[i0 + q] = p0 + c0 == 0 ? v : out[i0 + q] + v;
                 }
     }
 }
 
+// The sums in double, with the blocks, lanes and shared integrands of k_fwh_accum:
+// 12 FP64 operations a panel copy and sample (18 where a thread formed 7 integrands
+// for 4 samples of its own), bound by the FP64 pipe.
+struct __align__(16) FwhPc64 {
+    double c[NSER], w[4], off;
+    int at[KO];
+    int jb, pad;
+};
+// sample i of a panel copy whose stencil runs over an end of the record
+__device__ __noinline__ double fwh_end64(const FwhPc64* rc, const double2* xp, int nt, int i) {
+    const int j = fwh_stencil(double(i) + rc->off, nt);
+    double wt[4], sum = 0.0;
+    cubic_weights(double(i - j) + rc->off, wt);
+    for (int m = 0; m < 4; ++m) {
+        double I = 0.0;
+        for (int v = 0; v < 4; ++v) {
+            const double2 q = xp[fwh_slot(fwh_place(j + m, nt), v)];
+            I += rc->c[2 * v] * q.x;
+            I += rc->c[2 * v + 1] * q.y;
+        }
+        sum += wt[m] * I;
+    }
+    return sum;
+}
+__global__ void __launch_bounds__(32 * ACC_WARPS, 3)
+    k_fwh_accum64(const double2* __restrict__ X, int nt, int p0, int np, int nrows, const double* __restrict__ y,
+                  const double* __restrict__ dS, const __grid_constant__ FwhConst k, const FwhObs* __restrict__ obs,
+                  int Tmax, int ncopies, double Lspan, int group, double* __restrict__ partial) {
+    __shared__ __align__(16) FwhPc64 rec[ACC_PC];
+    const FwhBlock B(obs, group, np, ncopies);
+    const int T = B.T, i0 = B.i0;
+    double* out = partial + (int64_t(B.o) * nrows + B.row) * Tmax;
+    for (int c0 = 0; c0 < B.npc; c0 += ACC_PC) {
+        const int n = min(ACC_PC, B.npc - c0);
+        __syncthreads();
+        for (int w = threadIdx.x; w < n; w += blockDim.x) {
+            FwhPc64& rc = rec[w];
+            const int pl = B.gp0 + (c0 + w) / ncopies, cc = (c0 + w) % ncopies - B.K;
+            fwh_panel(y, dS, p0 + pl, cc, Lspan, obs[B.o], k, rc.c, &rc.off);
+            cubic_weights(rc.off - floor(rc.off) + 1.0, rc.w);   // position in the stencil, [1, 2)
+            // (no such offset: every sample takes its own stencil)
+            const int jb = fabs(rc.off) < 1e9 ? int(floor(rc.off)) - 1 : INT_MIN / 2;
+#pragma unroll
+            for (int m = 0; m < KO; ++m) rc.at[m] = fwh_place(jb + m, nt);
+            rc.jb = jb;
+        }
+        __syncthreads();
+        if (B.idle) continue;
+        double acc[KO] = {};
+        for (int w = 0; w < n; ++w) {
+            const FwhPc64& rc = rec[w];
+            const double2* xp = X + int64_t(B.gp0 + (c0 + w) / ncopies) * 4 * nt;
+            double I[KO + 3];
+#pragma unroll
+            for (int m = 0; m < KO; ++m) {
+                // a place outside the record (a lane without samples there) reads the last one
+                const unsigned at = min(unsigned(rc.at[m] + B.unit), unsigned(nt - 1));
+                I[m] = 0.0;
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    const double2 q = xp[fwh_slot(at, v)];
+                    I[m] += rc.c[2 * v] * q.x;
+                    I[m] += rc.c[2 * v + 1] * q.y;
+                }
+            }
+#pragma unroll
+            for (int m = 0; m < 3; ++m) I[KO + m] = __shfl_down_sync(0xffffffffu, I[m], 1);
+            const int t0 = i0 + rc.jb;
+#pragma unroll
+            for (int q = 0; q < KO; ++q) {
+                if (!B.mine || i0 + q >= T) continue;
+                double sum = 0.0;
+                if (t0 + q >= 0 && t0 + q + 3 < nt) {
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) sum += rc.w[m] * I[q + m];
+                } else {
+                    sum = fwh_end64(&rc, xp, nt, i0 + q);
+                }
+                acc[q] += sum;
+            }
+        }
+        if (B.mine)
+#pragma unroll
+            for (int q = 0; q < KO; ++q)
+                if (i0 + q < T) out[i0 + q] = p0 + c0 == 0 ? acc[q] : out[i0 + q] + acc[q];
+    }
+}
+
 // p'(t_i) = (1/4 pi) sum over panel groups of the partial sums: 32 samples x
 // 32 group slices per block, each slice summing groups g = slice (mod 32) in
-// order, then a fixed-order tree over the slices (the same order every call)
+// order, then a fixed-order tree over the slices (the same order every call).
+// Observers marked in `flag` (null: none) are left out.
 __global__ void k_fwh_reduce(const double* __restrict__ partial, int ngroups, int Tmax,
-                             const FwhObs* __restrict__ obs, double* __restrict__ p_out, int cap) {
+                             const FwhObs* __restrict__ obs, double* __restrict__ p_out, int cap,
+                             const int* __restrict__ flag, const int* __restrict__ wide) {
     __shared__ double red[32][33];
     const int i = blockIdx.x * 32 + threadIdx.x, o = blockIdx.y, T = obs[o].T;
     const double* row = partial + int64_t(o) * ngroups * Tmax;
-    double* out = p_out + int64_t(o) * cap;
+    if (flag && (flag[o] | *wide)) return;
+    double* out = p_out + int64_t(obs[o].row) * cap;
     double s = 0.0;
     if (i < T)
         for (int g = threadIdx.y; g < ngroups; g += 32) s += row[int64_t(g) * Tmax + i];
@@ -593,7 +733,9 @@ struct FwhPlan {
 // Device scratch of one integration: the source series of a batch of panels X
 // [nbatch][4][nt][2] doubles, their largest high words hw [nbatch][8], partial
 // sums [observers of a launch][groups][Tmax] (npartial doubles), and the
-// observer table of a launch (up to OBS_MAX observers) with its delay bounds.
+// observer table of a launch (up to OBS_MAX observers) with its delay bounds, whose
+// place the marks of the observers to be summed in double take afterwards (the last
+// one of them: all).
 constexpr int OBS_MAX = 2048;
 struct FwhScratch {
     double* X = nullptr;
@@ -603,12 +745,12 @@ struct FwhScratch {
     size_t npartial = 0;
     FwhObs* obs = nullptr;
     unsigned long long* ext = nullptr;
+    int* flag() const { return reinterpret_cast<int*>(ext); }   // [OBS_MAX + 1], after the plan is made
 };
 constexpr size_t OBS_BYTES = OBS_MAX * (sizeof(FwhObs) + 2 * sizeof(unsigned long long));
 
-int fwh_plan(int nt, int npts, const double* y, const double* n, const double* dS, const double* hist, double dtau,
-             double tau0, const double* obs, int nobs, const double Minf[3], double c0, double rho0, double p0,
-             double Lspan, int ncopies, const double* p_out, int cap, const int* nt_out, const double* t0_out,
+int fwh_plan(int nt, int npts, const double* y, double dtau, double tau0, const double* obs, int nobs,
+             const double Minf[3], double c0, double rho0, double p0, double Lspan, int ncopies, int cap,
              cudaStream_t s, const FwhScratch& sc, FwhPlan& pl) {
     const double MM = Minf[0] * Minf[0] + Minf[1] * Minf[1] + Minf[2] * Minf[2];
     FwhConst& k = pl.k;
@@ -620,8 +762,10 @@ int fwh_plan(int nt, int npts, const double* y, const double* n, const double* d
     k.tau0 = tau0;
     k.b2 = 1.0 / (1.0 - MM);
     pl.obs.assign(nobs, FwhObs{});
-    for (int o = 0; o < nobs; ++o)
+    for (int o = 0; o < nobs; ++o) {
         for (int i = 0; i < 3; ++i) pl.obs[o].x[i] = obs[o * 3 + i];
+        pl.obs[o].row = o;
+    }
     // unified observer windows from the delay bounds
     std::vector<unsigned long long> ext(2 * size_t(std::min(nobs, OBS_MAX)));
     for (int o0 = 0; o0 < nobs; o0 += OBS_MAX) {
@@ -685,6 +829,7 @@ size_t fwh_partial_doubles(const FwhPlan& pl) { return size_t(pl.ngroups) * pl.T
 // The kernels of one integration (all scratch is fully written before it is
 // read), then a synchronisation of the stream.  Panels go in batches of
 // sc.nbatch, whose series are formed once for all observers of a launch.
+// Observers that the fixed point marks are summed again in double.
 // Panels per block: enough for one resident wave of blocks over the GPU, at
 // most what one set-up pass of k_fwh_accum takes, and no fewer than the room for
 // partial sums asks for.
@@ -700,29 +845,52 @@ int fwh_run(const FwhPlan& pl, const double* hist, int nt, int npts, const doubl
     const int ngroups = (batch + group - 1) / group;
     const int obs_fit = int(std::min<size_t>(OBS_MAX, sc.npartial / (size_t(ngroups) * pl.Tmax)));
     cudaError_t err = cudaFuncSetAttribute(k_fwh_series, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SER_SMEM));
-    for (int o0 = 0; o0 < nobs && err == cudaSuccess; o0 += obs_fit) {
-        const int no = std::min(obs_fit, nobs - o0);
-        err = cudaMemcpyAsync(sc.obs, pl.obs.data() + o0, sizeof(FwhObs) * no, cudaMemcpyHostToDevice, s);
+    int *flag = sc.flag(), *wide = flag + OBS_MAX;
+    // the panels of a launch of `no` observers, in fixed point or in double
+    auto sums = [&](const FwhObs* table, int no, bool fixed, bool series) {
+        err = cudaMemcpyAsync(sc.obs, table, sizeof(FwhObs) * no, cudaMemcpyHostToDevice, s);
+        if (err == cudaSuccess && fixed) err = cudaMemsetAsync(flag, 0, sizeof(int) * (OBS_MAX + 1), s);
         for (int p0 = 0; p0 < npts && err == cudaSuccess; p0 += batch) {
             const int np = std::min(batch, npts - p0);
-            if (o0 == 0 || batch < npts) {
+            if (series || batch < npts) {
                 err = cudaMemsetAsync(sc.hw, 0, sizeof(int) * 8 * size_t(np), s);
-                if (err != cudaSuccess) break;
+                if (err != cudaSuccess) return;
                 k_fwh_series<<<dim3((np + SER_P - 1) / SER_P, (nt + SER_T - 1) / SER_T), 256, SER_SMEM, s>>>(
                     hist, nt, npts, p0, np, n, pl.k, sc.X, sc.hw);
                 const int64_t places = int64_t(np) * 4 * nt;
-                k_fwh_fix<<<unsigned(std::min<int64_t>((places + 255) / 256, 152 * 32)), 256, 0, s>>>(sc.X, sc.hw, nt, np);
+                if (fixed)
+                    k_fwh_fix<<<unsigned(std::min<int64_t>((places + 255) / 256, 152 * 32)), 256, 0, s>>>(
+                        sc.X, sc.hw, nt, np, wide);
             }
-            k_fwh_accum<<<dim3(no, (np + group - 1) / group, chunks), 32 * bw, 0, s>>>(
-                reinterpret_cast<const int4*>(sc.X), sc.hw, nt, p0, np, ngroups, y, dS, pl.k, sc.obs,
-                pl.Tmax, ncopies, Lspan, group, sc.partial);
+            const dim3 grid(no, (np + group - 1) / group, chunks);
+            if (fixed)
+                k_fwh_accum<<<grid, 32 * bw, 0, s>>>(reinterpret_cast<const int4*>(sc.X), sc.hw, nt, p0, np, ngroups, y,
+                                                     dS, pl.k, sc.obs, pl.Tmax, ncopies, Lspan, group, sc.partial, flag,
+                                                     wide);
+            else
+                k_fwh_accum64<<<grid, 32 * bw, 0, s>>>(reinterpret_cast<const double2*>(sc.X), nt, p0, np, ngroups, y, dS,
+                                                       pl.k, sc.obs, pl.Tmax, ncopies, Lspan, group, sc.partial);
             err = cudaGetLastError();
         }
-        if (err != cudaSuccess) break;
-        k_fwh_reduce<<<dim3((pl.Tmax + 31) / 32, no), dim3(32, 32), 0, s>>>(sc.partial, ngroups, pl.Tmax, sc.obs,
-                                                                           p_out + size_t(o0) * cap, cap);
+        if (err != cudaSuccess) return;
+        k_fwh_reduce<<<dim3((pl.Tmax + 31) / 32, no), dim3(32, 32), 0, s>>>(
+            sc.partial, ngroups, pl.Tmax, sc.obs, p_out, cap, fixed ? flag : nullptr, wide);
         err = cudaGetLastError();
+    };
+    std::vector<FwhObs> again;   // observers to be summed in double
+    std::vector<int> mark(OBS_MAX + 1, 0);
+    for (int o0 = 0; o0 < nobs && err == cudaSuccess; o0 += obs_fit) {
+        const int no = std::min(obs_fit, nobs - o0);
+        if (!mark[OBS_MAX]) {   // (a record without a fixed-point form: all that are left)
+            sums(pl.obs.data() + o0, no, true, o0 == 0);
+            if (err == cudaSuccess) err = cudaMemcpyAsync(mark.data(), flag, sizeof(int) * (OBS_MAX + 1), cudaMemcpyDeviceToHost, s);
+            if (err == cudaSuccess) err = cudaStreamSynchronize(s);
+        }
+        for (int o = 0; o < no; ++o)
+            if (mark[OBS_MAX] || mark[o]) again.push_back(pl.obs[o0 + o]);
     }
+    for (size_t o0 = 0; o0 < again.size() && err == cudaSuccess; o0 += obs_fit)
+        sums(again.data() + o0, int(std::min<size_t>(obs_fit, again.size() - o0)), false, o0 == 0);
     for (int o = 0; o < nobs; ++o) {
         nt_out[o] = pl.obs[o].T;
         t0_out[o] = pl.obs[o].tstart;
@@ -758,8 +926,7 @@ extern "C" int fwh_integrate(const double* hist, int nt, int npts, const double*
     sc.obs = static_cast<FwhObs*>(tab);
     sc.ext = reinterpret_cast<unsigned long long*>(sc.obs + OBS_MAX);
     FwhPlan pl;
-    rc = fwh_plan(nt, npts, y, n, dS, hist, dtau, tau0, obs, nobs, Minf, c0, rho0, p0, Lspan, ncopies, p_out,
-                  cap, nt_out, t0_out, s, sc, pl);
+    rc = fwh_plan(nt, npts, y, dtau, tau0, obs, nobs, Minf, c0, rho0, p0, Lspan, ncopies, cap, s, sc, pl);
     if (rc == FR_OK) {
         // up to 160 MiB of series at a time and 64 MiB of partial sums (never
         // less than the panels of one block and the rows of one observer)
@@ -830,8 +997,7 @@ extern "C" int fwh_integrate_noalloc(const double* hist, int nt, int npts, const
     rc = noalloc_scratch(&sc);
     if (rc != FR_OK) return rc;
     FwhPlan pl;
-    rc = fwh_plan(nt, npts, y, n, dS, hist, dtau, tau0, obs, nobs, Minf, c0, rho0, p0, Lspan, ncopies, p_out,
-                  cap, nt_out, t0_out, s, sc, pl);
+    rc = fwh_plan(nt, npts, y, dtau, tau0, obs, nobs, Minf, c0, rho0, p0, Lspan, ncopies, cap, s, sc, pl);
     if (rc != FR_OK) return rc;
     // the series and the partial rows must fit the fixed scratch
     const size_t need = fwh_series_doubles(npts, nt) + fwh_partial_doubles(pl);
