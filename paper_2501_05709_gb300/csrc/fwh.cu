@@ -44,13 +44,17 @@ struct FwhConst {
 };
 
 // The sources of one panel sample h = (rho, V1, V2, V3, p): n its normal, U = c0 M
-// the mean flow and Un = U.n; the disturbance u = V - U has u.n + U.n = V.n
+// the mean flow and Un = U.n.  rho (V.n) is formed from the disturbance u = V - U as
+// rho (u.n + Un), so that the rounding of Un, the same in both terms, leaves their
+// difference Q (with V.n Q is off by a rounding of |U| even on panels along the flow,
+// where Un is small).
 __device__ __forceinline__ void sources(const double* h, const double* n, const double* U, double Un,
                                         const FwhConst& k, double* out) {
-    const double rv = h[0] * (h[1] * n[0] + h[2] * n[1] + h[3] * n[2]);
+    const double u[3] = {h[1] - U[0], h[2] - U[1], h[3] - U[2]};
+    const double rv = h[0] * ((u[0] * n[0] + u[1] * n[1] + u[2] * n[2]) + Un);
     out[0] = rv - k.rho0 * Un;
     const double dp = h[4] - k.p0;
-    for (int i = 0; i < 3; ++i) out[1 + i] = dp * n[i] + rv * (h[1 + i] - U[i]);
+    for (int i = 0; i < 3; ++i) out[1 + i] = dp * n[i] + rv * u[i];
 }
 
 // The source series of a batch of panels: layout of one panel [nt places][4 pairs]
@@ -72,7 +76,7 @@ __host__ __device__ __forceinline__ unsigned fwh_slot(unsigned a, unsigned v) { 
 // into shared memory, then warp w writes panel w's eight series, 32 neighbouring
 // places per store, and keeps each series' largest magnitude (high word of the
 // double, a total order on magnitudes) for the fixed-point form.  Bound by the FP64
-// pipe (31 operations a panel and time).  At 18,840 panels x 1000 times 1.45 ms;
+// pipe (32 operations a panel and time).  At 18,840 panels x 1000 times 1.45 ms;
 // one thread per (panel, time) with six source evaluations each and stores 64 kB
 // apart took 4.93 ms.
 constexpr int SER_P = 8, SER_T = 256, SER_H = 4, SER_W = SER_T + 2 * SER_H;
@@ -87,7 +91,8 @@ __global__ void __launch_bounds__(256) k_fwh_series(const double* __restrict__ h
         const int lp = threadIdx.x % SER_P;
         const int p = p0 + min(pb + lp, np - 1);
         const double n[3] = {nrm[p * 3 + 0], nrm[p * 3 + 1], nrm[p * 3 + 2]};
-        const double U[3] = {k.c0 * k.M[0], k.c0 * k.M[1], k.c0 * k.M[2]};
+        // rounded products: fused into V - U they would leave U's rounding in u
+        const double U[3] = {__dmul_rn(k.c0, k.M[0]), __dmul_rn(k.c0, k.M[1]), __dmul_rn(k.c0, k.M[2])};
         const double Un = U[0] * n[0] + U[1] * n[1] + U[2] * n[2];
         for (int i = threadIdx.x / SER_P; i < SER_W; i += 256 / SER_P) {
             const int t = min(max(tb - SER_H + i, 0), nt - 1);
