@@ -319,12 +319,12 @@ int fwh_clear(fr_ctx* ctx, int handle);
  * Minf[3] (mean-flow Mach vector), c0, rho0, p0.  ncopies must be odd.
  * Output: p_out (device double [nobs][cap]) receives p'(t*_i) for
  * i < nt_out[o]; t0_out[o] (host) is the first unified time of observer o;
- * the unified step is dtau.  The sums are formed in 60-bit fixed point, relative
- * to the largest value that a panel group's records can give at any time, and
- * again in double for every observer with a sample of 2^-10 of that or less (a
- * transient's rise or decay, one outlier, infinities, NaN; about 2 to 3 times the
- * time), so that no sample is held with fewer bits than a double's sum leaves it.
- * The library takes its own scratch (the series of
+ * the unified step is dtau.  The sums are formed in 60-bit fixed point, with an
+ * error of about 3e-17 of the largest value that a group of panels can give at any
+ * time, and again in double (2 to 3 times the time) for every observer with a
+ * sample at which none gives 2^-10 of that: a transient's rise or decay, one large
+ * outlier, infinities, NaN.  An observer's result has the same bits whichever
+ * other observers the call has.  The library takes its own scratch (the series of
  * a batch of panels and partial-sum rows) from a pool of the device that keeps
  * at most 256 MB between calls and gives them back in fr_mesh_load and
  * fr_destroy; without memory pools it allocates and frees.  Errors: FR_EINVAL

@@ -35,7 +35,7 @@
 namespace {
 
 constexpr int NSER = 8;  // Q, L1, L2, L3, dQ, dL1, dL2, dL3
-constexpr int kFwhGroup = 32;   // panel copies per row of partial sums that the fixed scratch is counted by
+constexpr int kFwhGroup = 32;   // panel copies per row of partial sums
 
 struct FwhConst {
     double M[3];
@@ -302,7 +302,7 @@ __device__ void fwh_panel(const double* y, const double* dS, int p, int cc, doub
 //   number), kept as the two sums hh and mid of 64 bits, with which a sum over a
 //   block is exact; it becomes a double once, at the block's end.
 // One exponent holds for the whole record and for all copies of a block, so what is
-// lost is relative to the largest of them: at 96 copies about 2^-54 of 2^top (2-norm
+// lost is relative to the largest of them: at 32 copies about 2^-55 of 2^top (2-norm
 // of dropped l l' and rounded weights), where double loses about 2^-51 of the largest
 // |I| at that sample.  A sample at which no copy's integrand reaches 2^-10 of 2^top (a
 // transient's rise or decay, the quiet part of a record with one large outlier) may be
@@ -312,9 +312,11 @@ __device__ void fwh_panel(const double* y, const double* dS, int p, int cc, doub
 // is summed again in double (k_fwh_accum64).
 // Error against a reference in another order of summation, 2-norm: 1.3e-13 to 1.5e-12
 // here, 1.5e-13 to 1.8e-12 in double (it comes from the sources).
-// A block: one group of panels and one observer; a warp takes 124 samples of it, a
-// lane 4 consecutive ones (31 lanes; lane 31 only supplies the integrands that
-// lane 30's stencils need).  Each integrand is formed once and passed to the lane
+// A block: one group of panels and one observer; a warp takes 124 samples of one of
+// ns slices of its copies (a few observers leave too few warps otherwise; the integer
+// sums of the slices add up exactly, whatever ns), a lane 4 consecutive ones (31
+// lanes; lane 31 only supplies the integrands that lane 30's stencils need).  Each
+// integrand is formed once and passed to the lane
 // before it by shuffles: 24 + 12 products of limb pairs, 4 loads of 16 bytes and
 // 1.5 shuffles a sample.  Issue and latency bound it: at 18,840 panels, 36 observers and
 // 3 copies the products need 5.1 of 13.8 ms (at 32 wide multiply-adds a clock and SM),
@@ -388,13 +390,13 @@ __device__ __noinline__ void fwh_end(const FwhPc* rc, const int4* xp, int nt, in
 
 // How loud a lane's samples are: for each the bits of the largest top limb, in units
 // of 2^top, over the points of its stencils that count (4 x 8 bits; or-ed, so that one
-// bit too many is possible), over every step-th of the n copies at rec.  A loop of its
-// own: inside k_fwh_accum's it took registers, and 1.1 ms of 14.2 (18,840 panels, 36
-// observers, 3 copies) instead of 0.3.
-__device__ __noinline__ unsigned fwh_loud(const FwhPc* rec, int n, int step, int top, const int4* X, int first, int c0,
-                                          int ncopies, int nt, int unit, int samples) {
+// bit too many is possible), over those of the copies w0..w1 - 1 of rec that are
+// multiples of step.  A loop of its own: inside k_fwh_accum's it took registers, and 1.1
+// ms of 14.2 (18,840 panels, 36 observers, 3 copies) instead of 0.3.
+__device__ __noinline__ unsigned fwh_loud(const FwhPc* rec, int w0, int w1, int step, int top, const int4* X, int first,
+                                          int c0, int ncopies, int nt, int unit, int samples) {
     int loud[KO] = {};
-    for (int w = 0; w < n; w += step) {
+    for (int w = (w0 + step - 1) / step * step; w < w1; w += step) {
         const FwhPc& rc = rec[w];
         const int4* xp = X + int64_t(first + (c0 + w) / ncopies) * 4 * nt;
         const int down = min(31, top - rc.E), t0 = KO * unit + rc.jb;
@@ -423,35 +425,23 @@ __device__ __noinline__ unsigned fwh_loud(const FwhPc* rec, int n, int step, int
     return bits;
 }
 
-// a block's panels, samples and copies (k_fwh_accum and k_fwh_accum64)
-struct FwhBlock {
-    int o, row, lane, T, unit, i0, gp0, npc, K;
-    bool mine, idle;
-    __device__ FwhBlock(const FwhObs* obs, int group, int np, int ncopies)
-        : o(blockIdx.x), row(blockIdx.y), lane(threadIdx.x & 31), T(obs[blockIdx.x].T) {
-        unit = lane + ACC_LANES * (int(blockIdx.z) * int(blockDim.x >> 5) + int(threadIdx.x >> 5));
-        i0 = KO * unit;
-        mine = lane < ACC_LANES && i0 < T;                    // this lane stores samples i0.. of its own
-        idle = __shfl_sync(0xffffffffu, i0, 0) >= T;          // no lane of this warp does
-        gp0 = row * group;                                    // panels of this block, within the batch
-        npc = min(group, np - gp0) * ncopies;
-        K = (ncopies - 1) / 2;
-    }
-};
-
+template <bool SLICED>   // false: ns = 1
 __global__ void __launch_bounds__(32 * ACC_WARPS, 3)
     k_fwh_accum(const int4* __restrict__ X, const int* __restrict__ hwb, int nt, int p0, int np, int nrows,
                 const double* __restrict__ y, const double* __restrict__ dS, const __grid_constant__ FwhConst k,
                 const FwhObs* __restrict__ obs, int Tmax, int ncopies, double Lspan, int group,
-                double* __restrict__ partial, volatile int* flag, volatile int* wide) {
+                double* __restrict__ partial, int ns, volatile int* flag, volatile int* wide) {
     __shared__ __align__(16) FwhPc rec[ACC_PC];
+    __shared__ long long s_sum[SLICED ? 2 * KO : 1][32 * ACC_WARPS];
+    __shared__ unsigned s_bits[32 * ACC_WARPS];
     __shared__ int s_top, s_double;
     const int o = blockIdx.x, row = blockIdx.y;
     const int lane = threadIdx.x & 31;
     const int T = obs[o].T;
-    const int unit = lane + ACC_LANES * (int(blockIdx.z) * int(blockDim.x >> 5) + int(threadIdx.x >> 5));
+    const int bw = int(blockDim.x >> 5) / (SLICED ? ns : 1), slice = SLICED ? int(threadIdx.x >> 5) / bw : 0;
+    const int unit = lane + ACC_LANES * (int(blockIdx.z) * bw + int(threadIdx.x >> 5) - slice * bw);
     const int i0 = KO * unit;
-    const bool mine = lane < ACC_LANES && i0 < T;              // this lane stores samples i0.. of its own
+    const bool mine = lane < ACC_LANES && i0 < T;              // samples i0.. are this lane's
     const bool idle = __shfl_sync(0xffffffffu, i0, 0) >= T;    // no lane of this warp does
     const int gp0 = row * group, gnp = min(group, np - gp0);   // panels of this block, within the batch
     const int npc = gnp * ncopies, K = (ncopies - 1) / 2;
@@ -519,13 +509,14 @@ __global__ void __launch_bounds__(32 * ACC_WARPS, 3)
             }
         }
         __syncthreads();
-        if (idle) continue;
+        if (!SLICED && idle) continue;
         long long hh[KO], mid[KO];
 #pragma unroll
         for (int q = 0; q < KO; ++q) hh[q] = mid[q] = 0;
-        bool carry = n & 1;   // the last copy's sums are carried over
-        int pl = gp0 + c0 / ncopies, copy = c0 % ncopies;   // panel copy w (kept uniform: one base address for all lanes)
-        for (int w = 0; w < n; ++w) {
+        const int w0 = SLICED ? n * slice / ns : 0, w1 = !SLICED ? n : idle ? w0 : n * (slice + 1) / ns;
+        bool carry = (w1 - w0) & 1;   // the last copy's sums are carried over
+        int pl = gp0 + (c0 + w0) / ncopies, copy = (c0 + w0) % ncopies;   // of w (uniform: one base address for all lanes)
+        for (int w = w0; w < w1; ++w) {
             const FwhPc& rc = rec[w];
             const int4* xp = X + int64_t(pl) * 4 * nt;
             if (++copy == ncopies) {
@@ -590,10 +581,33 @@ __global__ void __launch_bounds__(32 * ACC_WARPS, 3)
                 }
         }
         // every 32nd copy looked at (fewer copies: every eighth, or all)
-        const unsigned bits = top == INT_MIN ? 0xffffffffu
-                                             : fwh_loud(rec, n, n >= 64 ? 32 : n >= 16 ? 8 : 1, top, X, gp0, c0, ncopies,
-                                                        nt, unit, mine ? T - i0 : 0);
-        if (mine)
+        unsigned bits = top == INT_MIN ? 0xffffffffu
+                                       : fwh_loud(rec, w0, w1, n >= 64 ? 32 : n >= 16 ? 8 : 1, top, X, gp0, c0, ncopies, nt,
+                                                  unit, mine ? T - i0 : 0);
+        if constexpr (SLICED) {
+#pragma unroll
+            for (int q = 0; q < KO; ++q) {
+                s_sum[q][threadIdx.x] = hh[q];
+                s_sum[KO + q][threadIdx.x] = mid[q];
+            }
+            s_bits[threadIdx.x] = bits;
+            __syncthreads();
+            if (slice > 0) continue;
+            for (int t = threadIdx.x + 32 * bw; t < blockDim.x; t += 32 * bw) {
+#pragma unroll
+                for (int q = 0; q < KO; ++q) {
+                    hh[q] += s_sum[q][t];
+                    mid[q] += s_sum[KO + q][t];
+                }
+                bits = __vmaxu4(bits, s_bits[t]);
+            }
+#pragma unroll
+            for (int q = 0; q < KO; ++q) {
+                hh[q] += mid[q] >> 30;
+                mid[q] &= (1ll << 30) - 1;
+            }
+        }
+        if (mine && slice == 0)
 #pragma unroll
             for (int q = 0; q < KO; ++q)
                 if (i0 + q < T) {
@@ -606,9 +620,11 @@ __global__ void __launch_bounds__(32 * ACC_WARPS, 3)
     }
 }
 
-// The sums in double, with the blocks, lanes and shared integrands of k_fwh_accum:
-// 12 FP64 operations a panel copy and sample (18 where a thread formed 7 integrands
-// for 4 samples of its own), bound by the FP64 pipe.
+// The sums in double, with the lanes and shared integrands of k_fwh_accum: 12 FP64
+// operations a panel copy and sample (18 where a thread formed 7 integrands for 4
+// samples of its own), bound by the FP64 pipe.  Always in D_NS slices of a block's
+// copies, added in order.
+constexpr int D_NS = 4;
 struct __align__(16) FwhPc64 {
     double c[NSER], w[4], off;
     int at[KO];
@@ -633,18 +649,26 @@ __device__ __noinline__ double fwh_end64(const FwhPc64* rc, const double2* xp, i
 __global__ void __launch_bounds__(32 * ACC_WARPS, 3)
     k_fwh_accum64(const double2* __restrict__ X, int nt, int p0, int np, int nrows, const double* __restrict__ y,
                   const double* __restrict__ dS, const __grid_constant__ FwhConst k, const FwhObs* __restrict__ obs,
-                  int Tmax, int ncopies, double Lspan, int group, double* __restrict__ partial) {
+                  int Tmax, int ncopies, double Lspan, int group, double* __restrict__ partial, int z0) {
     __shared__ __align__(16) FwhPc64 rec[ACC_PC];
-    const FwhBlock B(obs, group, np, ncopies);
-    const int T = B.T, i0 = B.i0;
-    double* out = partial + (int64_t(B.o) * nrows + B.row) * Tmax;
-    for (int c0 = 0; c0 < B.npc; c0 += ACC_PC) {
-        const int n = min(ACC_PC, B.npc - c0);
+    __shared__ double s_sum[KO][32 * ACC_WARPS];
+    const int o = blockIdx.x, row = blockIdx.y;
+    const int lane = threadIdx.x & 31;
+    const int T = obs[o].T;
+    const int bw = int(blockDim.x >> 5) / D_NS, slice = int(threadIdx.x >> 5) / bw;
+    const int unit = lane + ACC_LANES * ((z0 + int(blockIdx.z)) * bw + int(threadIdx.x >> 5) - slice * bw);
+    const int i0 = KO * unit;
+    const bool mine = lane < ACC_LANES && i0 < T;
+    const bool idle = __shfl_sync(0xffffffffu, i0, 0) >= T;
+    const int gp0 = row * group, npc = min(group, np - gp0) * ncopies, K = (ncopies - 1) / 2;
+    double* out = partial + (int64_t(o) * nrows + row) * Tmax;
+    for (int c0 = 0; c0 < npc; c0 += ACC_PC) {
+        const int n = min(ACC_PC, npc - c0);
         __syncthreads();
         for (int w = threadIdx.x; w < n; w += blockDim.x) {
             FwhPc64& rc = rec[w];
-            const int pl = B.gp0 + (c0 + w) / ncopies, cc = (c0 + w) % ncopies - B.K;
-            fwh_panel(y, dS, p0 + pl, cc, Lspan, obs[B.o], k, rc.c, &rc.off);
+            const int pl = gp0 + (c0 + w) / ncopies, cc = (c0 + w) % ncopies - K;
+            fwh_panel(y, dS, p0 + pl, cc, Lspan, obs[o], k, rc.c, &rc.off);
             cubic_weights(rc.off - floor(rc.off) + 1.0, rc.w);   // position in the stencil, [1, 2)
             // (no such offset: every sample takes its own stencil)
             const int jb = fabs(rc.off) < 1e9 ? int(floor(rc.off)) - 1 : INT_MIN / 2;
@@ -653,16 +677,16 @@ __global__ void __launch_bounds__(32 * ACC_WARPS, 3)
             rc.jb = jb;
         }
         __syncthreads();
-        if (B.idle) continue;
         double acc[KO] = {};
-        for (int w = 0; w < n; ++w) {
+        const int w1 = idle ? 0 : n * (slice + 1) / D_NS;
+        for (int w = n * slice / D_NS; w < w1; ++w) {
             const FwhPc64& rc = rec[w];
-            const double2* xp = X + int64_t(B.gp0 + (c0 + w) / ncopies) * 4 * nt;
+            const double2* xp = X + int64_t(gp0 + (c0 + w) / ncopies) * 4 * nt;
             double I[KO + 3];
 #pragma unroll
             for (int m = 0; m < KO; ++m) {
                 // a place outside the record (a lane without samples there) reads the last one
-                const unsigned at = min(unsigned(rc.at[m] + B.unit), unsigned(nt - 1));
+                const unsigned at = min(unsigned(rc.at[m] + unit), unsigned(nt - 1));
                 I[m] = 0.0;
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
@@ -676,7 +700,7 @@ __global__ void __launch_bounds__(32 * ACC_WARPS, 3)
             const int t0 = i0 + rc.jb;
 #pragma unroll
             for (int q = 0; q < KO; ++q) {
-                if (!B.mine || i0 + q >= T) continue;
+                if (!mine || i0 + q >= T) continue;
                 double sum = 0.0;
                 if (t0 + q >= 0 && t0 + q + 3 < nt) {
 #pragma unroll
@@ -687,10 +711,16 @@ __global__ void __launch_bounds__(32 * ACC_WARPS, 3)
                 acc[q] += sum;
             }
         }
-        if (B.mine)
+#pragma unroll
+        for (int q = 0; q < KO; ++q) s_sum[q][threadIdx.x] = acc[q];
+        __syncthreads();
+        if (mine && slice == 0)
 #pragma unroll
             for (int q = 0; q < KO; ++q)
-                if (i0 + q < T) out[i0 + q] = p0 + c0 == 0 ? acc[q] : out[i0 + q] + acc[q];
+                if (i0 + q < T) {
+                    for (int t = threadIdx.x + 32 * bw; t < blockDim.x; t += 32 * bw) acc[q] += s_sum[q][t];
+                    out[i0 + q] = p0 + c0 == 0 ? acc[q] : out[i0 + q] + acc[q];
+                }
     }
 }
 
@@ -831,24 +861,48 @@ int fwh_check(const double* hist, int nt, int npts, const double* y, const doubl
 size_t fwh_series_doubles(int npts, int nt) { return size_t(npts) * NSER * nt; }
 size_t fwh_partial_doubles(const FwhPlan& pl) { return size_t(pl.ngroups) * pl.Tmax; }
 
+// Panels of a block (a row of partial sums) and of a batch, and a batch's rows.  The
+// order of summation, and the exponent that a block's copies share, follow from the
+// panels, copies and record alone: an observer's p' has the same bits whichever other
+// observers are in the call.  kFwhGroup copies a block (18,840 panels, 36 observers, 3
+// copies: k_fwh_accum 13.6 ms, with 96 a block 13.8).  At one observer, 752 panels and
+// 2,400 samples it takes 54 us in 8 slices, without slices 113; blocks of few panels,
+// chosen by the number of observers, took 49.
+struct FwhSplit {
+    int group, batch, rows;
+    FwhSplit(int npts, int ncopies, int nbatch) {
+        group = std::max(1, kFwhGroup / ncopies);
+        const int nb = std::min(npts, nbatch);
+        if (nb == npts) {   // rows of even length
+            const int n = (npts + group - 1) / group;
+            group = (npts + n - 1) / n;
+        }
+        batch = nb == npts && npts <= 65535 * int64_t(group) ? npts : std::min(nb / group, 65535) * group;
+        rows = (batch + group - 1) / group;
+    }
+};
+
 // The kernels of one integration (all scratch is fully written before it is
 // read), then a synchronisation of the stream.  Panels go in batches of
 // sc.nbatch, whose series are formed once for all observers of a launch.
 // Observers that the fixed point marks are summed again in double.
-// Panels per block: enough for one resident wave of blocks over the GPU, at
-// most what one set-up pass of k_fwh_accum takes, and no fewer than the room for
-// partial sums asks for.
+// Warps of a block: time chunks and slices of copies, as many slices as it takes to
+// have 24 warps for every SM.
 int fwh_run(const FwhPlan& pl, const double* hist, int nt, int npts, const double* y, const double* n,
             const double* dS, const double* obs, int nobs, double Lspan, int ncopies, double* p_out, int cap,
             int* nt_out, double* t0_out, const FwhScratch& sc, cudaStream_t s) {
-    const int warps = (pl.Tmax + ACC_S - 1) / ACC_S, bw = std::min(warps, ACC_WARPS), chunks = (warps + bw - 1) / bw;
-    const int64_t wave = std::max(1, 152 * 24 / bw);
-    const int64_t nb = std::min(npts, sc.nbatch);
-    int group = int(std::min<int64_t>(std::max(1, ACC_PC / ncopies), (nb * nobs * chunks + wave - 1) / wave));
-    while (size_t((nb + group - 1) / group) * pl.Tmax > sc.npartial) ++group;
-    const int batch = nb == npts && npts <= 65535 * group ? npts : int(std::min<int64_t>(nb / group, 65535)) * group;
-    const int ngroups = (batch + group - 1) / group;
+    const FwhSplit sp(npts, ncopies, sc.nbatch);
+    const int group = sp.group, batch = sp.batch, ngroups = sp.rows;
     const int obs_fit = int(std::min<size_t>(OBS_MAX, sc.npartial / (size_t(ngroups) * pl.Tmax)));
+    int dev = 0, nsm = 1;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return fr_set_error_from_fwh(FR_ECUDA, "no device");
+    const int warps = (pl.Tmax + ACC_S - 1) / ACC_S;
+    int ns = 1;
+    while (ns < ACC_WARPS && int64_t(ngroups) * std::min(nobs, obs_fit) * warps * ns < 24 * int64_t(nsm)) ns *= 2;
+    // time chunks of a block (even) and blocks in time, in ns slices
+    auto chunks = [warps](int ns) { return (warps + ACC_WARPS / ns - 1) / (ACC_WARPS / ns); };
+    auto threads = [warps, chunks](int ns) { return 32 * ns * ((warps + chunks(ns) - 1) / chunks(ns)); };
     cudaError_t err = cudaFuncSetAttribute(k_fwh_series, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SER_SMEM));
     int *flag = sc.flag(), *wide = flag + OBS_MAX;
     // the panels of a launch of `no` observers, in fixed point or in double
@@ -864,17 +918,19 @@ int fwh_run(const FwhPlan& pl, const double* hist, int nt, int npts, const doubl
                     hist, nt, npts, p0, np, n, pl.k, sc.X, sc.hw);
                 const int64_t places = int64_t(np) * 4 * nt;
                 if (fixed)
-                    k_fwh_fix<<<unsigned(std::min<int64_t>((places + 255) / 256, 152 * 32)), 256, 0, s>>>(
+                    k_fwh_fix<<<unsigned(std::min<int64_t>((places + 255) / 256, nsm * 32)), 256, 0, s>>>(
                         sc.X, sc.hw, nt, np, wide);
             }
-            const dim3 grid(no, (np + group - 1) / group, chunks);
+            const unsigned rows = unsigned((np + group - 1) / group);
             if (fixed)
-                k_fwh_accum<<<grid, 32 * bw, 0, s>>>(reinterpret_cast<const int4*>(sc.X), sc.hw, nt, p0, np, ngroups, y,
-                                                     dS, pl.k, sc.obs, pl.Tmax, ncopies, Lspan, group, sc.partial, flag,
-                                                     wide);
-            else
-                k_fwh_accum64<<<grid, 32 * bw, 0, s>>>(reinterpret_cast<const double2*>(sc.X), nt, p0, np, ngroups, y, dS,
-                                                       pl.k, sc.obs, pl.Tmax, ncopies, Lspan, group, sc.partial);
+                (ns > 1 ? k_fwh_accum<true> : k_fwh_accum<false>)<<<dim3(no, rows, chunks(ns)), threads(ns), 0, s>>>(
+                    reinterpret_cast<const int4*>(sc.X), sc.hw, nt, p0, np, ngroups, y, dS, pl.k, sc.obs, pl.Tmax, ncopies,
+                    Lspan, group, sc.partial, ns, flag, wide);
+            else   // (windows above 16 million samples have more chunks than a grid's z)
+                for (int z0 = 0; z0 < chunks(D_NS); z0 += 65535)
+                    k_fwh_accum64<<<dim3(no, rows, std::min(65535, chunks(D_NS) - z0)), threads(D_NS), 0, s>>>(
+                        reinterpret_cast<const double2*>(sc.X), nt, p0, np, ngroups, y, dS, pl.k, sc.obs, pl.Tmax, ncopies,
+                        Lspan, group, sc.partial, z0);
             err = cudaGetLastError();
         }
         if (err != cudaSuccess) return;
@@ -937,8 +993,8 @@ extern "C" int fwh_integrate(const double* hist, int nt, int npts, const double*
         // less than the panels of one block and the rows of one observer)
         const size_t per = sizeof(double) * NSER * size_t(nt);
         sc.nbatch = int(std::min<size_t>(size_t(npts), std::max<size_t>(ACC_PC, (size_t(160) << 20) / per)));
-        const size_t rows = size_t(sc.nbatch) * pl.Tmax * nobs;
-        sc.npartial = std::min(rows, std::max(fwh_partial_doubles(pl), size_t(8) << 20));
+        const size_t one = size_t(FwhSplit(npts, ncopies, sc.nbatch).rows) * pl.Tmax;
+        sc.npartial = std::min(one * nobs, std::max(one, size_t(8) << 20));
         const size_t nx = fwh_series_doubles(sc.nbatch, nt);
         if (!get(&buf, sizeof(double) * (nx + sc.npartial) + 32 * size_t(sc.nbatch), &buf_pooled)) {
             put(tab, tab_pooled);
