@@ -1,11 +1,12 @@
 // Scratch of calls that allocate per call (FW-H integration, spectra): stream-
-// ordered allocations from one memory pool per device.  cudaMalloc and cudaFree
-// cost 65 us a pair below 64 MB and 250 us at 256 MB, and cudaFree waits for the
-// whole device; a pooled pair costs a few microseconds once the pool holds memory.
+// ordered allocations from one memory pool per device context.  cudaMalloc and
+// cudaFree cost 65 us a pair below 64 MB and 250 us at 256 MB, and cudaFree waits for
+// the whole device; a pooled pair costs a few microseconds once the pool holds memory.
 // The pool keeps at most POOL_KEEP bytes between calls (the driver releases what is
 // above at the next synchronisation) and gives everything back when a context is
-// loaded or destroyed (fr_pool_trim).  Safe with several threads and streams: the
-// driver orders the reuse of a block after its last use.
+// loaded or destroyed (fr_pool_trim).  cudaDeviceReset ends a context and its pool;
+// the next call makes another.  Safe with several threads and streams: the driver
+// orders the reuse of a block after its last use.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -16,5 +17,5 @@ constexpr unsigned long long POOL_KEEP = 256ull << 20;
 // grow (the caller then allocates for itself)
 bool fr_pool_alloc(void** p, size_t n, cudaStream_t s);
 void fr_pool_free(void* p, cudaStream_t s);
-// returns the unused memory of the current device's pool to the device
+// returns the unused memory of the current context's pool to the device
 void fr_pool_trim();
