@@ -64,15 +64,17 @@ int blocks_per_sm(K kernel, int threads, size_t smem) {
 // 16 to 24 of their warps: at p = 3 k_residual runs 92 us on the 32^3 box with 20
 // warps (2 or 4 elements a block) and 108 us with 16 (8 a block), on 100,000 curved
 // elements 319 against 342 us.  With fewer than 20 elements per SM the last wave
-// counts more than the number of warps, and blocks of one element level it (2,400
-// curved elements in FP64: 420 us against 440 to 510 us with 2 to 8).  `tie`: taken
+// counts more than the number of warps, and blocks of one element level it in FP64
+// (2,400 curved elements: 420 us against 440 to 510 us with 2 to 8); in FP32 blocks
+// of two do (2,310 elements at p = 4: 20 us, with 1: 26, with 8: 20 to 21; at p <= 3
+// all within 2%).  `tie`: taken
 // instead if it keeps three quarters of those warps (2 for the persistent face
 // kernel, whose elements of a block wait for each other at every tile: box of 32^3
 // at p = 4 with 2 elements a block 88 us, with 3: 94; p = 3 39.2 against 39.8).
 template <typename K, typename S>
 int best_tile(K kernel, int T, S smem, int64_t E, int tie = 0) {
     int best = 1, most = blocks_per_sm(kernel, T, smem(1));
-    if (E < 20 * int64_t(sm_count())) return 1;
+    if (E < 20 * int64_t(sm_count())) return sizeof(FR_REAL) == 8 ? 1 : 2;
     // FP64 is bound by its pipe, not by latency: whole warps a block count (4,096
     // affine elements at p = 3: 427 us a stage with 4, 432 with 2)
     if (sizeof(FR_REAL) == 8 && smem(4) <= 113 * 1024 && blocks_per_sm(kernel, 4 * T, smem(4)) > 0) return 4;
@@ -97,6 +99,13 @@ int traces_p(const FR_REAL* u, FR_REAL* uf, int64_t E, const frk::Ops<FR_REAL>& 
     const size_t sm = smem(std::max(lc.epb, 1));
     static unsigned long long done = 0;
     cudaError_t e = prep(k, sm, done);
+    if (lc.epb < 0 && sizeof(FR_REAL) == 4) {
+        // a copy with a few operations a value: in FP32 it wants large blocks (residual
+        // of 64,000 elements in 2D at p = 2 45 us with 8 elements a block, 54 with 2)
+        int epb = 8;
+        while (epb > 1 && smem(epb) > 96 * 1024) epb /= 2;
+        return epb;
+    }
     if (lc.epb < 0) return e == cudaSuccess ? best_tile(k, frk::Grp<FR_DIM, P>::T, smem, E) : 1;
     if (e != cudaSuccess) return int(e);
     if (E == 0) return 0;
