@@ -724,7 +724,8 @@ int max_epb(const fr_ctx* c) { return tpe_of(c) == 64 ? 15 : 32; }
 
 // the default tiles: asked of the launchers (frl::best_tile); the tensor-core
 // residual kernels take 8 elements per block, fewer when a block would need more
-// than 96 KB of shared memory
+// than 96 KB of shared memory, and two on less than 20 elements per SM (120 elements
+// at p = 4 in TF32 23 us, with 4: 26)
 template <typename Real>
 void default_launch_of(fr_ctx* c) {
     for (auto& l : c->lc) l.epb = -1;
@@ -734,6 +735,10 @@ void default_launch_of(fr_ctx* c) {
     if (c->prec < FR_TF32_TC) epb[2] = L_resid<Real>(c, nullptr, nullptr, st, nullptr);
     else
         while (epb[2] > 1 && smem_of(c, 2, epb[2]) > 96 * 1024) epb[2] /= 2;
+    int nsm = 0;
+    if (c->prec >= FR_TF32_TC && cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device) == cudaSuccess &&
+        c->E < 20 * int64_t(nsm))
+        epb[2] = std::min(epb[2], 2);
     c->launches = launches;
     for (int k = 0; k < 3; ++k) c->lc[k] = frk::Launch{epb[k], tpe_of(c) * epb[k]};
 }

@@ -1499,12 +1499,23 @@ __global__ void __maxnreg__(sizeof(Real) == 4 ? 80 : 168) k_visc_face(const Real
 // OPM: the gradient and divergence line operators as FP32 FMAs (0) or on the
 // tensor cores with TF32 (1) or BF16x3 (2) operands (float only).  Register
 // caps in FP32: 72 on affine meshes (box at p = 4 195 us, with 88: 212; Euler box
-// of 50^3 at p = 2 175, with 80: 187; of 40^3 at p = 3 131, with 96: 137); on
-// curved ones 88 (100,000 elements at p = 3: 314 us, with 72: 323, with 96: 319), at
-// p = 4 96 (20,000 elements: 156, with 88: 167, with 72: 199), at p = 2 80 (49, with
-// 88 or 96: 52, with 72: 58); 168 in FP64.
+// of 50^3 at p = 2 175, with 80: 187; of 40^3 at p = 3 131, with 96: 137), but where
+// the boundary states' code needs more than it leaves (22,000 elements between walls,
+// viscous, at p = 2: 46 us with 80, 53 with 72; at p = 4 147 with 96, 193 with 72,
+// inviscid 104 with 80, 111 with 72); on curved ones 88 (100,000 elements at p = 3:
+// 314 us, with 72: 323, with 96: 319), at p = 4 96 (20,000 elements: 156, with 88: 167,
+// with 72: 199), at p = 2 80 (49, with 88 or 96: 52, with 72: 58); with tensor-core line
+// operators 80 (22,000 elements in TF32 at p = 4: 374 us, with 72: 393, with 88: 452;
+// between walls 390, 401, 481); 168 in FP64.
+template <int DIM, int P, typename Real>
+constexpr int resid_regs(int MP, bool VISC, bool BND, int OPM) {
+    if (sizeof(Real) == 8) return 168;
+    if (OPM != 0) return 80;
+    if (MP != 0) return DIM == 2 || !BND ? 72 : P == 4 ? (VISC ? 96 : 80) : VISC && P >= 2 ? 80 : 72;
+    return DIM == 3 && P == 4 ? 96 : DIM == 3 && P == 2 ? 80 : 88;
+}
 template <int DIM, int P, typename Real, int MP, bool VISC, bool BND, int OPM = 0>
-__global__ void __maxnreg__(sizeof(Real) == 4 ? (MP != 0 ? 72 : DIM == 3 && P == 4 ? 96 : DIM == 3 && P == 2 ? 80 : 88) : 168) k_residual(const Real* __restrict__ u, const Real* __restrict__ uf,
+__global__ void __maxnreg__((resid_regs<DIM, P, Real>(MP, VISC, BND, OPM))) k_residual(const Real* __restrict__ u, const Real* __restrict__ uf,
                            const Real* __restrict__ fvn, int64_t E, const __grid_constant__ Ops<Real> op,
                            const __grid_constant__ Phys<Real> ph, const __grid_constant__ Geo<Real> g,
                            const __grid_constant__ Stage<Real> st) {
