@@ -384,7 +384,8 @@ int fwh_psd(const double* p, int nobs, int nt, int ld, double dt, int nseg, doub
 
 /* Elements per thread block used by the residual kernels (0 = built-in
  * default; 1..32, or 1..15 in 3D at p = 4, where two warps share each
- * element); fr_autotune times the candidates on the current state and keeps
+ * element; a kernel whose registers admit fewer takes as many as fit);
+ * fr_autotune times the candidates on the current state and keeps
  * the fastest per kernel, returning it in *best. */
 int fr_set_tile(fr_ctx* ctx, int elems_per_block);
 int fr_autotune(fr_ctx* ctx, int* best);

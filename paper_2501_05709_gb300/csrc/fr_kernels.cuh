@@ -22,6 +22,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
+
 #include "fr_common.h"
 
 namespace frk {
@@ -76,6 +78,21 @@ __device__ __forceinline__ bool face_pt(int lane, int it, int& side, int& fp) {
         fp = t - side * NFP;
         return t < 2 * NFP;
     }
+}
+
+// epb, or the most elements (T threads each) that a block of this kernel holds: its
+// registers may admit fewer than the tile asked for, and results do not depend on the
+// tile.  `most` belongs to the caller's kernel instantiation (0: not asked yet).
+template <typename K>
+int fit_tile(K kernel, int T, int epb, std::atomic<int>& most) {
+    int n = most.load();
+    if (n == 0) {
+        cudaFuncAttributes a;
+        if (cudaFuncGetAttributes(&a, kernel) != cudaSuccess) return epb;
+        n = a.maxThreadsPerBlock / T;
+        most.store(n = n > 0 ? n : 1);
+    }
+    return epb < n ? epb : n;
 }
 
 // face points of one direction per lane

@@ -3,7 +3,6 @@
 #include "fr_kernels.cuh"
 
 #include <algorithm>
-#include <atomic>
 
 namespace frl {
 
@@ -108,8 +107,10 @@ int traces_p(const FR_REAL* u, FR_REAL* uf, int64_t E, const frk::Ops<FR_REAL>& 
     }
     if (lc.epb < 0) return e == cudaSuccess ? best_tile(k, frk::Grp<FR_DIM, P>::T, smem, E) : 1;
     if (e != cudaSuccess) return int(e);
+    static std::atomic<int> most{0};
+    const int epb = frk::fit_tile(k, frk::Grp<FR_DIM, P>::T, lc.epb, most);
     if (E == 0) return 0;
-    k<<<grid_of(E, lc.epb), frk::Grp<FR_DIM, P>::T * lc.epb, sm, s>>>(u, uf, E, op);
+    k<<<grid_of(E, epb), frk::Grp<FR_DIM, P>::T * epb, smem(epb), s>>>(u, uf, E, op);
     return int(cudaGetLastError());
 }
 
@@ -127,8 +128,10 @@ int visc_p(const FR_REAL* u, const FR_REAL* uf, FR_REAL* fvn, int64_t E, const f
         cudaError_t e = prep(k, sm, done);
         if (lc.epb < 0) return e == cudaSuccess ? best_tile(k, frk::Grp<FR_DIM, P>::T, smem, E) : 1;
         if (e != cudaSuccess) return int(e);
+        static std::atomic<int> most{0};
+        const int epb = frk::fit_tile(k, frk::Grp<FR_DIM, P>::T, lc.epb, most);
         if (E == 0) return 0;
-        k<<<grid_of(E, lc.epb), frk::Grp<FR_DIM, P>::T * lc.epb, sm, s>>>(u, uf, fvn, E, op, ph, g);
+        k<<<grid_of(E, epb), frk::Grp<FR_DIM, P>::T * epb, smem(epb), s>>>(u, uf, fvn, E, op, ph, g);
         return int(cudaGetLastError());
     } else {
         // affine meshes: the pipelined kernel on a persistent grid of as many
@@ -141,15 +144,17 @@ int visc_p(const FR_REAL* u, const FR_REAL* uf, FR_REAL* fvn, int64_t E, const f
         cudaError_t e = prep(k, sm, done);
         if (lc.epb < 0) return e == cudaSuccess ? best_tile(k, frk::Grp<FR_DIM, P>::T, smem, E, 2) : 1;
         if (e != cudaSuccess) return int(e);
+        static std::atomic<int> most{0};
+        const int epb = frk::fit_tile(k, frk::Grp<FR_DIM, P>::T, lc.epb, most);
         if (E == 0) return 0;
-        const int threads = frk::Grp<FR_DIM, P>::T * lc.epb;
+        const int threads = frk::Grp<FR_DIM, P>::T * epb;
         static std::atomic<int> resident[33];
-        int cap = resident[lc.epb & 31].load();
+        int cap = resident[epb & 31].load();
         if (cap == 0) {
-            cap = std::max(1, blocks_per_sm(k, threads, sm)) * sm_count();
-            resident[lc.epb & 31].store(cap);
+            cap = std::max(1, blocks_per_sm(k, threads, smem(epb))) * sm_count();
+            resident[epb & 31].store(cap);
         }
-        k<<<std::min(grid_of(E, lc.epb), unsigned(cap)), threads, sm, s>>>(u, uf, fvn, E, op, ph, g);
+        k<<<std::min(grid_of(E, epb), unsigned(cap)), threads, smem(epb), s>>>(u, uf, fvn, E, op, ph, g);
         return int(cudaGetLastError());
     }
 }
@@ -166,8 +171,10 @@ int resid_p(const FR_REAL* u, const FR_REAL* uf, const FR_REAL* fvn, int64_t E,
     cudaError_t e = prep(k, sm, done);
     if (lc.epb < 0) return e == cudaSuccess ? best_tile(k, frk::Grp<FR_DIM, P>::T, smem, E) : 1;
     if (e != cudaSuccess) return int(e);
+    static std::atomic<int> most{0};
+    const int epb = frk::fit_tile(k, frk::Grp<FR_DIM, P>::T, lc.epb, most);
     if (E == 0) return 0;
-    k<<<grid_of(E, lc.epb), frk::Grp<FR_DIM, P>::T * lc.epb, sm, s>>>(u, uf, fvn, E, op, ph, g, st);
+    k<<<grid_of(E, epb), frk::Grp<FR_DIM, P>::T * epb, smem(epb), s>>>(u, uf, fvn, E, op, ph, g, st);
     return int(cudaGetLastError());
 }
 

@@ -39,9 +39,11 @@ int resid_tc_p(const float* u, const float* uf, const float* fvn, int64_t E, con
     static unsigned long long done = 0;
     cudaError_t e = prep_tc(k, sm, done);
     if (e != cudaSuccess) return int(e);
+    static std::atomic<int> most{0};
+    const int epb = frk::fit_tile(k, frk::Grp<3, P>::T, lc.epb, most);
     if (E == 0) return 0;
-    const unsigned grid = unsigned((E + lc.epb - 1) / lc.epb);
-    k<<<grid, frk::Grp<3, P>::T * lc.epb, sm, s>>>(u, uf, fvn, E, op, ph, g, st);
+    const unsigned grid = unsigned((E + epb - 1) / epb);
+    k<<<grid, frk::Grp<3, P>::T * epb, frk::smem_resid<3, P, float>(epb, g.sS_sp != 0), s>>>(u, uf, fvn, E, op, ph, g, st);
     return int(cudaGetLastError());
 }
 

@@ -1,5 +1,5 @@
-"""Elements per block: the default tile is about as fast as the best fixed one, and meshes with walls run about as fast
-as periodic ones."""
+"""Elements per block: every tile that fr_set_tile takes runs and gives the bits of the default one, the default tile is
+about as fast as the best fixed one, and meshes with walls run about as fast as periodic ones."""
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -43,6 +43,30 @@ def _residual_us(ctx, u):
         b.synchronize()
         best = min(best, a.elapsed_time(b) * 100.0)
     return best
+
+
+# orders, precisions and meshes whose kernels hold the most registers
+@pytest.mark.parametrize("prec, dim, p, walls, curve", [
+    ("fp64", 3, 2, True, 0.0), ("fp64", 3, 2, False, 0.0), ("fp64", 3, 4, True, 0.0), ("fp64", 2, 4, True, 0.0),
+    ("fp64", 3, 2, False, 0.05), ("fp32", 3, 2, False, 0.0), ("fp32", 3, 4, False, 0.0), ("fp32", 3, 4, False, 0.05),
+    ("fp32", 2, 4, True, 0.0), ("tf32", 3, 4, False, 0.0), ("tf32", 3, 3, True, 0.0)])
+def test_every_tile_that_is_taken_runs(prec, dim, p, walls, curve):
+    from paper_2501_05709_gb300 import fr as F
+    ctx, u = _load(dim, [3, 4, 3][:dim], p, {"fp64": F.FR_FP64, "fp32": F.FR_FP32, "tf32": F.FR_TF32_TC}[prec], True, walls,
+                   curve)
+    with ctx:
+        ref, R = torch.empty_like(u), torch.empty_like(u)
+        F.fr_residual(ctx, u, ref)
+        taken = 0
+        for tile in range(1, 33):
+            try:
+                F.fr_set_tile(ctx, tile)
+            except F.FrError:
+                continue
+            taken += 1
+            F.fr_residual(ctx, u, R.zero_())
+            assert torch.equal(R, ref), tile
+        assert taken >= 4
 
 
 @pytest.mark.parametrize("dim, n, p, visc", [(2, [250, 256], 2, False), (3, [14, 15, 11], 4, True), (3, [28, 28, 28], 1, False)])
