@@ -2120,9 +2120,13 @@ extern "C" int fr_set_tile(fr_ctx* c, int epb) {
 
 extern "C" int fr_autotune(fr_ctx* c, int* best) {
     if (!c) return fail(FR_EINVAL, "null argument");
-    // time each sweep for 1..16 elements (warps) per block on the current
-    // state; keep the fastest per kernel.  Results do not depend on the tile.
-    const int cand[] = {1, 2, 4, 8, 16};
+    // time each sweep for 1..16 elements (warps) per block, and for the tile it has
+    // now, on the current state; keep the fastest per kernel.  Results do not depend
+    // on the tile.
+    const frk::Launch now[3] = {c->lc[0], c->lc[1], c->lc[2]};
+    std::vector<int> cand = {1, 2, 4, 8, 16};
+    for (const auto& l : now)
+        if (std::find(cand.begin(), cand.end(), l.epb) == cand.end()) cand.push_back(l.epb);
     cudaEvent_t a, b;
     CK(cudaEventCreate(&a));
     CK(cudaEventCreate(&b));
@@ -2145,10 +2149,10 @@ extern "C" int fr_autotune(fr_ctx* c, int* best) {
         bool fits = true;
         for (int k = 0; k < 3; ++k) fits = fits && smem_of(c, k, epb) <= 200 * 1024;
         fits = fits && epb <= max_epb(c);
-        if (!fits) continue;
         for (int k = 0; k < 3; ++k) c->lc[k] = frk::Launch{epb, tpe_of(c) * epb};
         for (int kern = 0; kern < 3; ++kern) {
             if (kern == 1 && !c->visc) continue;
+            if (!fits && epb != now[kern].epb) continue;
             float tot = 1e30f;   // best of the timed repetitions
             int rc = 0;
             for (int rep = 0; rep < 12 && rc == 0; ++rep) {

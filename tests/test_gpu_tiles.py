@@ -1,5 +1,6 @@
 """Elements per block: every tile that fr_set_tile takes runs and gives the bits of the default one, the default tile is
-about as fast as the best fixed one, and meshes with walls run about as fast as periodic ones."""
+about as fast as the best fixed one, meshes with walls run about as fast as periodic ones, and fr_autotune times the
+tile in use beside its candidates."""
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -91,3 +92,17 @@ def test_walls_cost_little():
         with ctx:
             us.append(_residual_us(ctx, u))
     assert us[1] <= 1.25 * us[0]
+
+
+def test_autotune_times_the_tile_in_use():
+    from paper_2501_05709_gb300 import fr as F
+    ctx, u = _load(3, [6, 6, 6], 2, F.FR_FP32)
+    with ctx:
+        F.fr_state_set(ctx, u.double())
+        count = []
+        for tile in (4, 3):                  # one of the candidates, and one that is none
+            F.fr_set_tile(ctx, tile)
+            before = F.fr_launch_count(ctx)
+            F.fr_autotune(ctx)
+            count.append(F.fr_launch_count(ctx) - before)
+    assert count[1] == count[0] // 5 * 6
