@@ -35,11 +35,17 @@ cudaError_t prep(K kernel, size_t smem, unsigned long long& done) {
 }
 
 // kernels that run beside the element kernels ask for the same carveout (an SM
-// holds one split of its memory at a time)
+// holds one split of its memory at a time), on their first use on a device (`done` as
+// for prep)
 template <typename K>
-int side_prep(K kernel) {
-    return int(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                    int(cudaSharedmemCarveoutMaxShared)));
+int side_prep(K kernel, unsigned long long& done) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (e != cudaSuccess || (done & bit)) return int(e);
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, int(cudaSharedmemCarveoutMaxShared));
+    if (e == cudaSuccess) done |= bit;
+    return int(e);
 }
 
 inline unsigned grid_of(int64_t E, int epb) { return unsigned((E + epb - 1) / epb); }
@@ -265,7 +271,7 @@ int forces<FR_REAL, FR_DIM>(int P, const FR_REAL* uf, const FR_REAL* fvn, const 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (ncand <= 0) return 0;
     const dim3 grid(frk::FORCE_BLOCKS, unsigned(ncand));
-#define C(PP) side_prep(frk::k_forces<FR_DIM, PP, FR_REAL>)
+#define C(PP) [] { static unsigned long long done = 0; return side_prep(frk::k_forces<FR_DIM, PP, FR_REAL>, done); }()
     [&]() -> int { FR_DISPATCH(C) }();
 #undef C
 #define C(PP) (frk::k_forces<FR_DIM, PP, FR_REAL><<<grid, 256, 0, s>>>(uf, fvn, wall_ef, wall_off, op, g, gm1, \
@@ -281,7 +287,7 @@ int sample<FR_REAL, FR_DIM>(int P, const FR_REAL* u, const frk::Surf<FR_REAL>* s
                             const frk::Phys<FR_REAL>& ph, void* stream) {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const dim3 grid(unsigned((int64_t(most) * 32 + 255) / 256), unsigned(nsurf));
-#define C(PP) side_prep(frk::k_sample<FR_DIM, PP, FR_REAL>)
+#define C(PP) [] { static unsigned long long done = 0; return side_prep(frk::k_sample<FR_DIM, PP, FR_REAL>, done); }()
     [&]() -> int { FR_DISPATCH(C) }();
 #undef C
 #define C(PP) (frk::k_sample<FR_DIM, PP, FR_REAL><<<grid, 256, 0, s>>>(u, surf, ph),                            \
