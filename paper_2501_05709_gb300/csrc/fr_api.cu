@@ -79,6 +79,7 @@ struct fr_ctx {
     cudaStream_t aux_stream = nullptr;
     cudaEvent_t ev_aux[2] = {nullptr, nullptr};
     frk::Launch lc[3]{};
+    bool lc_default = true;   // lc are the default tiles (not fr_set_tile's or fr_autotune's)
     cudaStream_t cap_stream = nullptr;
     // the reduced-degree kernels of a step run on red_stream[q] (one per
     // degree q), forked from the step's stream and joined back (they write
@@ -725,7 +726,10 @@ int max_epb(const fr_ctx* c) { return tpe_of(c) == 64 ? 15 : 32; }
 // the default tiles: asked of the launchers (frl::best_tile); the tensor-core
 // residual kernels take 8 elements per block, fewer when a block would need more
 // than 96 KB of shared memory, and two on less than 20 elements per SM (120 elements
-// at p = 4 in TF32 23 us, with 4: 26)
+// at p = 4 in TF32 23 us, with 4: 26).  FP64 kernels on few elements take one a block,
+// which levels the last wave, but not where reduced-degree elements fill that wave
+// (2,400 curved elements at p = 3, 480 of them reduced: step 1,458 us with 4 elements a
+// block, 1,571 with 1; 720 elements: 886 and 637)
 template <typename Real>
 void default_launch_of(fr_ctx* c) {
     for (auto& l : c->lc) l.epb = -1;
@@ -739,10 +743,17 @@ void default_launch_of(fr_ctx* c) {
     if (c->prec >= FR_TF32_TC && cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device) == cudaSuccess &&
         c->E < 20 * int64_t(nsm))
         epb[2] = std::min(epb[2], 2);
+    bool reduced = false;
+    for (int q = 0; q < c->p; ++q) reduced = reduced || c->red_n[q] > 0;
+    if (reduced && c->prec == FR_FP64 &&
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device) == cudaSuccess && c->E >= 10 * int64_t(nsm))
+        for (int k = 0; k < 3; ++k)
+            if (epb[k] == 1 && smem_of(c, k, 4) <= 113 * 1024) epb[k] = 4;
     c->launches = launches;
     for (int k = 0; k < 3; ++k) c->lc[k] = frk::Launch{epb[k], tpe_of(c) * epb[k]};
 }
 void default_launch(fr_ctx* c) {
+    c->lc_default = true;
     if (c->prec == FR_FP64) default_launch_of<double>(c);
     else default_launch_of<float>(c);
 }
@@ -1733,6 +1744,7 @@ extern "C" int fr_set_element_order(fr_ctx* c, int cand, const int32_t* order) {
     const int rc = build_reduced(c);
     if (rc) return fail(rc, "cannot build the reduced-degree element tables");
     c->traces_valid = false;
+    if (c->lc_default) default_launch(c);
     invalidate_graph(c);
     CK(cudaDeviceSynchronize());
     return FR_OK;
@@ -2109,6 +2121,7 @@ extern "C" int fr_set_tile(fr_ctx* c, int epb) {
     } else {
         for (int k = 0; k < 3; ++k)
             if (smem_of(c, k, epb) > 227 * 1024) return fail(FR_EINVAL, "tile needs too much shared memory");
+        c->lc_default = false;
         for (int k = 0; k < 3; ++k) {
             c->lc[k].epb = epb;
             c->lc[k].threads = tpe_of(c) * epb;
@@ -2193,6 +2206,7 @@ extern "C" int fr_autotune(fr_ctx* c, int* best) {
         }
     }
     for (int k = 0; k < 3; ++k) c->lc[k] = bestl[k];
+    c->lc_default = false;
     cudaFree(R);
     cudaFree(A);
     cudaFree(TR);
