@@ -601,18 +601,26 @@ def fwh_leg():
     torch.cuda.synchronize()
     t_psd = time.perf_counter() - t0
     work = len(y) * len(obs) * 3 * nt
-    # bound by the wide integer multiply-adds of k_fwh_accum: 7 integrands of 24 products
-    # for 4 samples and 12 more products a sample, against 32 a clock and SM (measured
-    # with a loop of them) at the highest clock; the time is the whole call
-    ops = 3.0 * len(y) * int(np.sum(nt_out)) * (7 * 24 / 4 + 12)
-    pk = 32 * torch.cuda.get_device_properties(0).multi_processor_count * 2.07
+    # the SM clock under this load, for the peak below
+    clocks = Clocks(torch.cuda.current_device())
+    t0 = time.perf_counter()
+    while time.perf_counter() - t0 < 1.5:
+        F.fwh_integrate(*args, Lspan=0.2, ncopies=3)
+    ck = clocks.stop()
+    # the work of the sums in wide integer multiply-adds (k_fwh_accum): one integrand of 24
+    # products a sample and 12 more to weight and add it; the time is the whole call
+    ops = 3.0 * len(y) * int(np.sum(nt_out)) * (24 + 12)
+    mhz = ck["sm_mhz"] or ck["sm_max_mhz"]
+    pk = 32 * torch.cuda.get_device_properties(0).multi_processor_count * mhz * 1e-3 if mhz else None
     ach = ops / t_int / 1e9
     return {"panels": int(len(y)), "observers": int(len(obs)), "copies": 3, "samples": nt,
             "window_samples_min": nmin, "fwh_integrate_ms": 1e3 * t_int,
             "panel_observer_copy_samples_per_s": work / t_int, "fwh_psd_ms": 1e3 * t_psd,
             "roofline": {"bound": "alu", "kernel": "fwh_integrate (k_fwh_accum, 60-bit fixed point on the integer pipe)",
-                         "achieved": ach, "peak": pk, "unit": "G wide integer multiply-adds/s", "frac": ach / pk,
-                         "peak_source": "32 a clock and SM at 2.07 GHz"},
+                         "achieved": ach, "peak": pk, "unit": "G wide integer multiply-adds/s",
+                         "frac": ach / pk if pk else None,
+                         "peak_source": "assumed: 32 a clock and SM, at the SM clock sampled during such calls"},
+            "clocks": ck,
             "note": "host wall time around each call (each call synchronises and includes its scratch set-up "
                     "and the observer windows)"}
 
