@@ -322,7 +322,7 @@ int fwh_clear(fr_ctx* ctx, int handle);
  * the unified step is dtau.  The sums are formed in 60-bit fixed point, with an
  * error of about 3e-17 of the largest value that a group of panels can give at any
  * time, and again in double (2 to 3 times the time) for every observer with a
- * sample at which none gives 2^-10 of that: a transient's rise or decay, one large
+ * sample at which none gives 2^-12 of that: a transient's rise or decay, one large
  * outlier, infinities, NaN.  An observer's result has the same bits whichever
  * other observers the call has.  The library takes its own scratch (the series of
  * a batch of panels and partial-sum rows) from a pool of the device that keeps

@@ -304,12 +304,15 @@ __device__ void fwh_panel(const double* y, const double* dS, int p, int cc, doub
 // One exponent holds for the whole record and for all copies of a block, so what is
 // lost is relative to the largest of them: at 32 copies about 2^-55 of 2^top (2-norm
 // of dropped l l' and rounded weights), where double loses about 2^-51 of the largest
-// |I| at that sample.  A sample at which no copy's integrand reaches 2^-10 of 2^top (a
-// transient's rise or decay, the quiet part of a record with one large outlier) may be
-// held worse than by a double.  The kernel takes the largest |I| of each sample's
-// stencils, over those points that count (weight at least 1/32), over some of the block's
-// copies, and marks the observer where that is too small (fwh_loud); a marked observer
-// is summed again in double (k_fwh_accum64).
+// |I| at that sample.  A sample at which no copy's integrand reaches 2^-12 of 2^top (a
+// transient's rise or decay, the quiet part of a record with one large outlier) is not
+// left to fixed point: what it loses is then above 1e-13 of the largest |I|, the size of
+// the sources' own errors.  The kernel takes the largest |I| of each sample's stencils,
+// over those points that count (weight at least 1/32), over some of the block's copies,
+// and marks the observer where that is too small (fwh_loud); a marked observer is summed
+// again in double (k_fwh_accum64).  At 2^-10 the common zero of a block's 32 copies marked
+// an observer in 2 of 12 records of sinusoids (18,840 panels, 36 observers: 18.8 ms for
+// 16.0), at 2^-12 in none.
 // Error against a reference in another order of summation, 2-norm: 1.3e-13 to 1.5e-12
 // here, 1.5e-13 to 1.8e-12 in double (it comes from the sources).
 // A block: one group of panels and one observer; a warp takes 124 samples of one of
@@ -328,7 +331,7 @@ constexpr int ACC_WARPS = 8;      // warps (sample chunks) of a block at most
 constexpr int ACC_S = KO * ACC_LANES;
 
 constexpr int SILENT = -100000;    // exponent of a copy without a contribution (no branch: that cost 1.5%)
-constexpr int ACC_QUIET = 21;      // bits of a top limb of 2^-10 of the bound (2^20)
+constexpr int ACC_QUIET = 19;      // bits of a top limb of 2^-12 of the bound (2^18)
 
 struct __align__(16) FwhPc {   // read in 16-byte pieces
     int c[2 * NSER];   // coefficient limbs (h, l)
